@@ -80,7 +80,9 @@ typedef struct {
   uint64_t seed;               /* SplitMix64 seed of the forecast-noise draws */
   const float *noise_bank;     /* host [bank_B][bank_G][bank_G] screens, or NULL; copied */
   int32_t bank_B, bank_G;      /* bank shape (ignored when noise_bank is NULL) */
-  int32_t max_sweeps;          /* Jacobi sweep limit per node; <= 0 -> 20 */
+  int32_t max_sweeps;          /* <= 0: FP32 node problems of moderate condition are solved by a
+                                  Chebyshev series, the others by Jacobi sweeps (at most 20);
+                                  > 0: every problem by Jacobi sweeps, at most this many */
   int32_t partition;           /* 0: every node is its own local domain (the per-node analysis);
                                   P in 2..64: multi-actuator local domains of a P x P partition
                                   of the node grid (Section 4.1), single instance, FP32, m 2..128;
@@ -253,8 +255,10 @@ letkf_status letkf_set_params(letkf_t h, int32_t i, double rho, double sigma2, d
  * rotations). Measured at the ELT steady state against the FP64 oracle,
  * teacher-forced: the default gives 2e-6 on the analysis mean, 1e-5 on the
  * spread and 4e-5 on the anomalies with 5.7 sweeps per node; stop_cos =
- * rotate_tol gives 2e-6 / 3e-6 / 9e-6 with 8.3 sweeps. FP64 handles and the
- * FP64 fallback keep their own tolerance. LETKF_ERR_ARG outside (0, 1) and
+ * rotate_tol gives 2e-6 / 3e-6 / 9e-6 with 8.3 sweeps. Nodes solved by the
+ * Chebyshev series (letkf_config.max_sweeps) are accurate to FP32 rounding and
+ * have no such rule; FP64 handles and the FP64 fallback keep their own
+ * tolerance. LETKF_ERR_ARG outside (0, 1) and
  * [0, 1). Synchronises. */
 letkf_status letkf_set_jacobi(letkf_t h, double rotate_tol, double stop_cos);
 
@@ -366,7 +370,8 @@ letkf_status letkf_sync(letkf_t h);
 /* Counters of the last analysis, host pointers (any may be NULL): nodes that
  * took the FP64 fallback, the largest and the total number of Jacobi sweeps
  * over the nodes (a node of the FP64 fallback counts the sweeps of its FP32
- * and of its FP64 eigensolve). Synchronises. */
+ * and of its FP64 eigensolve, a node solved by the Chebyshev series one).
+ * Synchronises. */
 letkf_status letkf_stats(letkf_t h, int32_t *fp64_points, int32_t *max_sweeps,
                          int32_t *total_sweeps);
 

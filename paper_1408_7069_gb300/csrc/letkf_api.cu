@@ -74,7 +74,7 @@ void release(letkf_ctx *h) {
   void *bufs[] = {h->X,          h->Ybp,      h->dp,       h->taper,    h->pid_map,
                   h->pts,        h->saps,     h->bank,     h->basis,    h->basis64,  h->counters,
                   h->worklist,   h->frame,    h->partial,  h->tickets,  h->d_inst,   h->obs_items,
-                  h->node_items, h->tiles[0], h->tiles[1], h->tiles[2], h->noise_pre};
+                  h->node_items, h->tiles[0], h->tiles[1], h->tiles[2], h->noise_pre, h->cheb32};
   for (void *p : bufs)
     if (p) cudaFree(p);
 }
@@ -430,6 +430,8 @@ letkf_status build_handle(const letkf_config *cfgs, int n, void *stream, letkf_t
     for (int cls = 0; cls < 3; ++cls) LK_TRY(build_tiles(h, cls, pids));
   }
   e = lk_setup_analysis(h);
+  // an explicit sweep limit asks for the iterative eigensolve it limits
+  if (e == cudaSuccess && cfgs[0].max_sweeps <= 0) e = lk_setup_cheb(h);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) LK_TRY(cuda_fail(h, e, "device set-up"));
 #undef LK_TRY

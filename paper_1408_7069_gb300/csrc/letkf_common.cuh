@@ -38,6 +38,14 @@ constexpr int LK_WARP_CTA = 64;
 // square, far below what the FP32 outputs resolve.
 constexpr double LK_WARM_STOP64 = 1e-8;
 
+// Chebyshev series of (1 + g)^-1/2 and (1 + g)^-1 on [0, ratio] (letkf_cheb.cu):
+// classes of ratio LK_CHEB_R0 LK_CHEB_STEP^c, one row of LK_CHEB_LD32 pairs per
+// class: (2 / ratio, degree), then the coefficients (a_k, b_k), k = 0 .. degree.
+// The step of 1.25 costs at most one product in nine over the exact ratio.
+constexpr double LK_CHEB_R0 = 0.25, LK_CHEB_STEP = 1.25;
+constexpr int LK_CHEB_CLASSES32 = 33, LK_CHEB_LD32 = 192;
+constexpr float LK_CHEB_MAX32 = 300.f;        // below the last class's 315.5
+
 // One AO instance, as the kernels see it (device pointers, by-value copy in a
 // device array). The real type of X, Yb, d, y, truth, taper and the outputs is
 // float (precision 0) or double (precision 1).
@@ -94,6 +102,7 @@ struct letkf_ctx {
   double tol32 = 4e-6, tol64 = 1e-13, fp64_kappa = 300;
   double stop32 = 1e-3;             // FP32 Jacobi stops after a sweep with all cosines <= this
   int max_sweeps = 20;
+  float2 *cheb32 = nullptr;         // FP32 Chebyshev table; NULL: every node by Jacobi sweeps
   int keep_basis = 0;               // store every node's eigenbasis (reverse mode needs it)
 
   int n_inst = 0;
@@ -202,6 +211,8 @@ cudaError_t lk_setup_analysis(letkf_ctx *h);
 // FP32 analysis of width class cls, two columns per lane (letkf_pair.cu).
 cudaError_t lk_launch_pair(letkf_ctx *h, int cls, void *mean, void *spread);
 cudaError_t lk_setup_pair(letkf_ctx *h);
+// Allocates and fills the handle's Chebyshev tables (letkf_cheb.cu).
+cudaError_t lk_setup_cheb(letkf_ctx *h);
 // FP64 analysis with one CTA of four warps per node (letkf_node64.cu): every
 // node of width class cls (0: MP 16, 1: MP 32) of an FP64 handle, or the nodes
 // the pair kernel queued in class cls of an FP32 handle.
@@ -283,6 +294,14 @@ cudaError_t lk_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// Ratio class of the Chebyshev tables: the first whose ratio is at least `ratio`
+// (rounded up by 2e-5, far above the logarithm's error).
+__device__ __forceinline__ int lk_cheb_class(float ratio) {
+  constexpr float inv_log2_step = 3.10628372f;               // 1 / log2(LK_CHEB_STEP)
+  const float l = __log2f(fmaxf(ratio, 1e-30f) * float(1.0 / LK_CHEB_R0)) * inv_log2_step;
+  return max(0, (int)ceilf(l + 1e-4f));
 }
 
 // SplitMix64 output after the state advanced counter + 1 steps from seed

@@ -70,7 +70,7 @@ struct PairCfg {
   static constexpr int NPW = 32 / GL;                          // nodes per warp
   static constexpr int K2 = MP / 2;                            // float2 per column
   static constexpr int CELLF = 2 * MP + 4;                     // floats per halo cell (+4: bank shift)
-  static constexpr int NODE_SCR = 3 * MP + 4;                  // scratch floats per node
+  static constexpr int NODE_SCR = 4 * MP + 4;                  // scratch floats per node
   static constexpr int MPS = MP == 24 ? 32 : MP;               // columns of the stored basis
 };
 
@@ -290,6 +290,95 @@ __device__ __forceinline__ void stage_pair_tile(const LkInst &I, int i0, int j0,
   for (int e = threadIdx.x; e < w * w; e += blockDim.x) tap[e] = (float)taper[e];
 }
 
+// ---------------------------------------------------------------------------
+// Functions of A on the node's two anomaly rows, without an eigensolve. The
+// analysis needs W only as X'_r W = sqrt(m-1) (A^-1/2 x'_r)^T and wbar only as
+// X'_r wbar = (A^-1 x'_r)^T C d, so with A = alpha (I + G / alpha), spectrum of
+// G / alpha inside [0, ratio] (ratio >= |G|_F / alpha), both are Chebyshev
+// series in x = 2 g / (alpha ratio) - 1:
+//   T_0 = x'_r, T_1 = X T_0, T_k+1 = 2 X T_k - T_k-1 with X = 2 G / (alpha ratio) - I
+//   A^-1/2 x'_r = alpha^-1/2 sum_k a_k T_k,   A^-1 x'_r = alpha^-1 sum_k b_k T_k
+// The coefficients and the degree come from a table of ratio classes
+// (lk_cheb_*, letkf_cheb.cu), truncated below FP32 rounding. A loop state's
+// ratio of 2-5 takes 11-18 products of the two vectors with G, 2 m^2 FMAs each:
+// an eighth of one Jacobi sweep per product, against six sweeps, and no
+// rotation chain. P, Q: rows 2li and 2li+1 of G; t0: members 2li, 2li+1 of
+// the two anomaly rows; buf: [2][2][MP] shared floats of the node. A warp runs
+// the largest degree of its nodes; a node takes no term beyond its own, so its
+// bits do not depend on its neighbours. Nodes above LK_CHEB_MAX32 (more than 160
+// products, and the sweeps keep small eigenpairs accurate at any condition),
+// queued nodes and nodes whose basis is kept take the sweeps.
+// Bound by the FP32 pipe (64 packed FMAs per product and lane). Measured on one
+// GB300, whole frames of a running loop, sweeps -> series: 80 x 80, m = 32 188 ->
+// 58 us; 48 systems 6.7 -> 1.65 ms; error against FP64 1.4e-6 -> 1.4e-7.
+// ---------------------------------------------------------------------------
+template <int MP, bool LIVE_ALL>
+__device__ __forceinline__ void direct_apply(const float2 (&P)[MP / 2], const float2 (&Q)[MP / 2],
+                                             float2 x0, float2 x1, int li, bool live, float scale,
+                                             int deg, int deg_warp,
+                                             const float2 *__restrict__ coef, float *buf,
+                                             float2 &u0, float2 &u1, float2 &s0, float2 &s1) {
+  constexpr int K4 = MP / 4;
+  float2 c = __ldg(coef);
+  float2 tp0 = x0, tp1 = x1;                          // T_k-1
+  float2 t0 = x0, t1 = x1;                            // T_k
+  u0 = mul2(f2(c.x), x0);
+  u1 = mul2(f2(c.x), x1);
+  s0 = mul2(f2(c.y), x0);
+  s1 = mul2(f2(c.y), x1);
+  float f = scale;                                    // T_1 = scale G T_0 - T_0
+  float e = 1.f, o = 0.f;
+  for (int k = 1; k <= deg_warp; ++k) {
+    float *b = buf + (k & 1) * 2 * MP;
+    if (LIVE_ALL || live) {
+      reinterpret_cast<float2 *>(b)[li] = t0;
+      reinterpret_cast<float2 *>(b + MP)[li] = t1;
+    }
+    c = k <= deg ? __ldg(coef + k) : f2(0.f);
+    __syncwarp();
+    float2 p0 = f2(0.f), p1 = f2(0.f), q0 = f2(0.f), q1 = f2(0.f);
+    float2 r0 = f2(0.f), r1 = f2(0.f), w0 = f2(0.f), w1 = f2(0.f);
+#pragma unroll
+    for (int j = 0; j < K4; ++j) {
+      const float4 a = reinterpret_cast<const float4 *>(b)[j];
+      const float4 d = reinterpret_cast<const float4 *>(b + MP)[j];
+      const float2 a0 = make_float2(a.x, a.y), a1 = make_float2(a.z, a.w);
+      const float2 d0 = make_float2(d.x, d.y), d1 = make_float2(d.z, d.w);
+      p0 = fma2(P[2 * j], a0, p0);
+      r0 = fma2(P[2 * j + 1], a1, r0);
+      q0 = fma2(Q[2 * j], a0, q0);
+      w0 = fma2(Q[2 * j + 1], a1, w0);
+      p1 = fma2(P[2 * j], d0, p1);
+      r1 = fma2(P[2 * j + 1], d1, r1);
+      q1 = fma2(Q[2 * j], d0, q1);
+      w1 = fma2(Q[2 * j + 1], d1, w1);
+    }
+    p0 = __fadd2_rn(p0, r0);
+    q0 = __fadd2_rn(q0, w0);
+    p1 = __fadd2_rn(p1, r1);
+    q1 = __fadd2_rn(q1, w1);
+    // T_k+1 = f G T_k - e T_k - o T_k-1 (f, e, o = scale, 1, 0, then 2 scale, 2, 1)
+    const float2 g0 = make_float2(p0.x + p0.y, q0.x + q0.y);
+    const float2 g1 = make_float2(p1.x + p1.y, q1.x + q1.y);
+    const float2 n0 = fma2(f2(f), g0, fma2(f2(-e), t0, mul2(f2(-o), tp0)));
+    const float2 n1 = fma2(f2(f), g1, fma2(f2(-e), t1, mul2(f2(-o), tp1)));
+    tp0 = t0;
+    tp1 = t1;
+    t0 = n0;
+    t1 = n1;
+    if (k == 1) {
+      f = 2.f * scale;
+      e = 2.f;
+      o = 1.f;
+    }
+    u0 = fma2(f2(c.x), t0, u0);
+    u1 = fma2(f2(c.x), t1, u1);
+    s0 = fma2(f2(c.y), t0, s0);
+    s1 = fma2(f2(c.y), t1, s1);
+  }
+  __syncwarp();
+}
+
 // One CTA per tile of TI x TJ nodes of one instance; the nodes of the tile are
 // taken in row-major order, NPW per warp. `queue`: FP64 worklist counter slot
 // (MP <= 32), NULL for no fallback.
@@ -311,7 +400,8 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
     analysis_pair_kernel(const LkInst *__restrict__ insts, const LkTile *__restrict__ tiles,
                          float *__restrict__ mean, float *__restrict__ spread, float tol,
                          float stop, int max_sweeps, float kappa_thr, int *__restrict__ counters,
-                         int *__restrict__ queue, int2 *__restrict__ worklist, int keep_basis) {
+                         int *__restrict__ queue, int2 *__restrict__ worklist, int keep_basis,
+                         const float2 *__restrict__ cheb) {
   lk_pdl_wait();   // no early trigger: the next kernel launches as this one's CTAs exit
   LK_PHASE_STAMP(ph0);
   using C = PairCfg<MP>;
@@ -394,6 +484,66 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
       queued = true;
     }
   }
+  // the node's two rows: means and anomalies
+  LK_PHASE_STAMP(ph2);
+  const bool wr = active && !queued;
+  float *xrow = wr ? static_cast<float *>(I.X) + (size_t)pid * 2 * m : nullptr;
+  const int m0 = 2 * li, m1 = 2 * li + 1;
+  const bool in0 = live && m0 < m, in1 = live && m1 < m;
+  const float inv_m = 1.f / float(m);
+  float xb0 = 0.f, xb1 = 0.f;
+  float2 xa0 = f2(0.f), xa1 = f2(0.f);  // anomalies of members m0, m1, then X'_r W
+  float w0 = 0.f, w1 = 0.f;             // X'_r wbar
+  // ---- Chebyshev series, where the ratio has a class (cheb NULL: none) ----
+  bool direct = false;
+  if constexpr (!BASIS) {
+    const float x00 = (wr && in0) ? xrow[m0] : 0.f;
+    const float x01 = (wr && in1) ? xrow[m1] : 0.f;
+    const float x10 = (wr && in0) ? xrow[m + m0] : 0.f;
+    const float x11 = (wr && in1) ? xrow[m + m1] : 0.f;
+    xb0 = group_sum<GL>(x00 + x01) * inv_m;
+    xb1 = group_sum<GL>(x10 + x11) * inv_m;
+    xa0 = make_float2(in0 ? x00 - xb0 : 0.f, in1 ? x01 - xb0 : 0.f);
+    xa1 = make_float2(in0 ? x10 - xb1 : 0.f, in1 ? x11 - xb1 : 0.f);
+    if (cheb) {
+      const float g2 = live ? dotk<K2>(P, P) + dotk<K2>(Q, Q) : 0.f;
+      const float ratio = sqrtf(group_sum<GL>(g2)) / alpha;
+      direct = wr && ratio <= LK_CHEB_MAX32;          // (not with a NaN)
+      int deg = 0;
+      const float2 *coef = cheb;
+      float scale = 0.f;
+      if (direct) {
+        const int cls = lk_cheb_class(ratio);
+        coef = cheb + (size_t)cls * LK_CHEB_LD32;
+        const float2 head = __ldg(coef++);            // (2 / ratio of the class, degree)
+        scale = head.x / alpha;
+        deg = (int)head.y;
+      }
+      const int deg_warp = __reduce_max_sync(FULL, deg);
+      if (deg_warp > 0) {
+        float2 u0, u1, s0, s1;
+        direct_apply<MP, C::LPN == C::GL>(P, Q, xa0, xa1, li, live, scale, deg, deg_warp, coef,
+                                          scr, u0, u1, s0, s1);
+        const float ia = 1.f / alpha;
+        const float d0 = group_sum<GL>(fmaf(s0.x, cd0, s0.y * cd1)) * ia;
+        const float d1 = group_sum<GL>(fmaf(s1.x, cd0, s1.y * cd1)) * ia;
+        if (direct) {
+          const float rt = sqrtf(float(m - 1) * ia);
+          w0 = d0;
+          w1 = d1;
+          xa0 = mul2(f2(rt), u0);
+          xa1 = mul2(f2(rt), u1);
+          if (li == 0) {
+            atomicMax(&counters[2], 1);
+            atomicAdd(&counters[3], 1);
+          }
+        }
+      }
+    }
+  }
+  // ---- Jacobi: every other node, and all of them when their bases are kept ----
+  const bool sweep_node = active && (!direct || keep_basis);
+  if (__any_sync(FULL, sweep_node)) {
   // (m-1)/rho on the diagonal, 1 on the padding; inactive nodes and idle lanes
   // get identity columns
   const bool own = active && live;
@@ -415,12 +565,11 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
   }
 
   // ---- Jacobi sweeps ----
-  LK_PHASE_STAMP(ph2);
   const float tol2 = tol * tol, stop2 = stop * stop;
   const int base = grp * GL;
   const int up = live ? base + (li + 1) % LPN : lane;
   const int dn = live ? base + (li + LPN - 1) % LPN : lane;
-  bool conv = !active;
+  bool conv = !sweep_node;
   int sweeps = 0;
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     if (__all_sync(FULL, conv)) break;
@@ -451,14 +600,13 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
       if ((big & gmask) == 0u) conv = true;
     }
   }
-  if (active && li == 0) {
+  if (sweep_node && !direct && li == 0) {
     atomicMax(&counters[2], sweeps);
     atomicAdd(&counters[3], sweeps);
-    if (!conv) atomicOr(&counters[0], LK_BIT_NOCONVERGE);
   }
+  if (sweep_node && !conv && li == 0) atomicOr(&counters[0], LK_BIT_NOCONVERGE);
 
   // ---- eigenpairs: lambda = |b|, v = b / lambda ----
-  LK_PHASE_STAMP(ph3);
   const float lP = sqrtf(dotk<K2>(P, P)), lQ = sqrtf(dotk<K2>(Q, Q));
   {
     const float iP = 1.f / lP, iQ = 1.f / lQ;
@@ -469,7 +617,7 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
     }
   }
   // ---- eigenbasis for the reverse mode and for queued nodes: U[k][2li], U[k][2li+1] ----
-  if ((BASIS || keep_basis || queued) && active && live) {
+  if ((BASIS || keep_basis || queued) && sweep_node && live) {
     bool ok = true;
 #pragma unroll
     for (int k = 0; k < K2; ++k)
@@ -484,27 +632,15 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
       reinterpret_cast<float2 *>(U + (2 * k + 1) * MPS)[li] = r1;
     }
   }
-  if constexpr (BASIS) return;
-
-  // ---- transform and apply (Section 4.2): Xa_r = xbar_r + X'_r wbar + X'_r W ----
+  // ---- transform (Section 4.2): X'_r wbar and X'_r W of the nodes not done above ----
+  if (!BASIS && __any_sync(FULL, wr && !direct)) {
   float *vcd = scr;                     // C d
   float *vx0 = vcd + MP;                // X'_0
   float *vx1 = vx0 + MP;                // X'_1
-  const bool wr = active && !queued;
-  float *xrow = wr ? static_cast<float *>(I.X) + (size_t)pid * 2 * m : nullptr;
-  const int m0 = 2 * li, m1 = 2 * li + 1;
-  const bool in0 = live && m0 < m, in1 = live && m1 < m;
-  const float x00 = (wr && in0) ? xrow[m0] : 0.f;
-  const float x01 = (wr && in1) ? xrow[m1] : 0.f;
-  const float x10 = (wr && in0) ? xrow[m + m0] : 0.f;
-  const float x11 = (wr && in1) ? xrow[m + m1] : 0.f;
-  const float inv_m = 1.f / float(m);
-  const float xb0 = group_sum<GL>(x00 + x01) * inv_m;
-  const float xb1 = group_sum<GL>(x10 + x11) * inv_m;
   if (live) {
     reinterpret_cast<float2 *>(vcd)[li] = make_float2(cd0, cd1);
-    reinterpret_cast<float2 *>(vx0)[li] = make_float2(in0 ? x00 - xb0 : 0.f, in1 ? x01 - xb0 : 0.f);
-    reinterpret_cast<float2 *>(vx1)[li] = make_float2(in0 ? x10 - xb1 : 0.f, in1 ? x11 - xb1 : 0.f);
+    reinterpret_cast<float2 *>(vx0)[li] = xa0;
+    reinterpret_cast<float2 *>(vx1)[li] = xa1;
   }
   __syncwarp();
   // projections of C d and of the two anomaly rows on this lane's eigenvectors
@@ -524,8 +660,8 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
   const float gP0 = live ? a0P.x + a0P.y : 0.f, gQ0 = live ? a0Q.x + a0Q.y : 0.f;
   const float gP1 = live ? a1P.x + a1P.y : 0.f, gQ1 = live ? a1Q.x + a1Q.y : 0.f;
   const float zP = (uP.x + uP.y) / lP, zQ = (uQ.x + uQ.y) / lQ;
-  const float w0 = group_sum<GL>(gP0 * zP + gQ0 * zQ);    // X'_0 wbar
-  const float w1 = group_sum<GL>(gP1 * zP + gQ1 * zQ);    // X'_1 wbar
+  const float p0 = group_sum<GL>(gP0 * zP + gQ0 * zQ);    // X'_0 wbar
+  const float p1 = group_sum<GL>(gP1 * zP + gQ1 * zQ);    // X'_1 wbar
   const float rP = sqrtf(float(m - 1) / lP), rQ = sqrtf(float(m - 1) / lQ);
   // X'_r W = sum_j h_r,j v_j^T with h_r,j = (X'_r v_j) sqrt((m-1)/lambda_j): this
   // lane's two terms, summed over the node's lanes and scattered by member
@@ -545,8 +681,20 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
   }
   const float2 q0 = reduce_scatter<GL>(v0, li);
   const float2 q1 = reduce_scatter<GL>(v1, li);
-  const float xa00 = xb0 + w0 + q0.x, xa01 = xb0 + w0 + q0.y;
-  const float xa10 = xb1 + w1 + q1.x, xa11 = xb1 + w1 + q1.y;
+  if (!direct) {
+    w0 = p0;
+    w1 = p1;
+    xa0 = q0;
+    xa1 = q1;
+  }
+  }
+  }
+  if constexpr (BASIS) return;
+
+  // ---- apply: Xa_r = xbar_r + X'_r wbar + X'_r W ----
+  LK_PHASE_STAMP(ph3);
+  const float xa00 = xb0 + w0 + xa0.x, xa01 = xb0 + w0 + xa0.y;
+  const float xa10 = xb1 + w1 + xa1.x, xa11 = xb1 + w1 + xa1.y;
   if (wr) {
     if (in0) {
       xrow[m0] = xa00;
@@ -934,7 +1082,8 @@ cudaError_t launch_shape(letkf_ctx *h, const LkTile *tiles, int n_tiles, float *
     return lk_launch_pdl(analysis_pair_kernel<MP, TI, TJ>, n_tiles,
                          TI * TJ * 32 / PairCfg<MP>::NPW, need, h->stream, h->d_inst, tiles, mean,
                          spread, (float)h->tol32, (float)h->stop32, h->max_sweeps, kthr,
-                         h->counters, queue, worklist, h->keep_basis);
+                         h->counters, queue, worklist, h->keep_basis,
+                         (const float2 *)h->cheb32);
   }
 }
 
@@ -975,7 +1124,7 @@ cudaError_t launch_basis_shape(letkf_ctx *h, int cls) {
                          TI * TJ * 32 / PairCfg<MP>::NPW, need, h->stream, h->d_inst,
                          h->tiles[cls], (float *)nullptr, (float *)nullptr, (float)h->tol32,
                          (float)h->stop32, h->max_sweeps, 0.f, h->counters, (int *)nullptr,
-                         (int2 *)nullptr, 1);
+                         (int2 *)nullptr, 1, (const float2 *)nullptr);
   }
 }
 

@@ -1,0 +1,120 @@
+"""The Chebyshev form of the per-node analysis (letkf_pair.cu: direct_apply) at the
+sizes and spectra where it can go wrong, against the FP64 oracle and against the
+eigensolve (a handle with an explicit sweep limit).
+
+Tolerance of the ensemble, for the root mean square of its error over the nodes: A^-1/2
+changes by at most kappa / 2 times the relative change of A, whose FP32 rounding is a
+few units (the Gram's sums), and the series' own rounding is of the order of its degree,
+about 10 sqrt(kappa) units: 32 kappa units of 2^-24 of the anomalies' size cover both.
+The mean moves by X' A^-1 C d, kappa units of the increment's size. Storing the members
+(background and analysis) in FP32 adds two units of their own size."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+from paper_1408_7069_gb300 import synth  # noqa: E402
+from paper_1408_7069_gb300.letkf import Letkf, tile_shapes  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+SIGMA2, RHO = 0.01, 1.03
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.asarray(a) - np.asarray(b)) / np.linalg.norm(b))
+
+
+def anoms(X):
+    X = np.asarray(X, np.float64)
+    return X - X.mean(-1, keepdims=True)
+
+
+def problem(nsub, m, window, taper, scale, square=False, ramp=None):
+    """An ensemble of white member anomalies of size `scale` (times a factor growing from
+    ramp[0] to ramp[1] along the grid), slopes, geometry and the nodes' kappa_hat."""
+    mask = synth.pupil_subap_mask(nsub, 0.0, square)
+    geom = oracle.build_geometry(mask, window, taper, 0.0)
+    rng = np.random.default_rng(1000 * nsub + 10 * m + window)
+    s = np.full(geom.n_pts, scale)
+    if ramp:
+        s = scale * np.geomspace(ramp[0], ramp[1], geom.n_pts)
+    X = 3 * rng.standard_normal((geom.n_pts, 2, 1)) \
+        + s[:, None, None] * rng.standard_normal((geom.n_pts, 2, m))
+    X = X.astype(np.float32)
+    y = rng.standard_normal(geom.p).astype(np.float32)
+    _, _, Yb, _ = oracle.observe(geom, X.astype(np.float64))
+    khat = np.array([1 + RHO / (m - 1) * np.sum((t / SIGMA2)[:, None] * Yb[i] ** 2)
+                     for i, t in zip(geom.win_idx, geom.win_tau)])
+    return mask, geom, X, y, khat
+
+
+def analyse(mask, X, y, m, window, taper, shape=None, cls=None, **kw):
+    f = Letkf(mask, m=m, window=window, taper=taper, rho=RHO, sigma2=SIGMA2, **kw)
+    if shape is not None:
+        f.set_tile_shape(cls, shape)
+    f.set_state(torch.from_numpy(X).cuda())
+    mean, spread = f.analyze(torch.from_numpy(y).cuda())
+    f.sync()
+    out = f.get_state().cpu().numpy(), mean.cpu().numpy(), spread.cpu().numpy(), f.stats()
+    f.close()
+    return out
+
+
+SIZES = [(1, 2, 1, 0), (4, 3, 3, 1), (5, 15, 3, 1), (5, 16, 4, 0), (6, 17, 5, 1), (6, 23, 5, 1),
+         (6, 24, 5, 0), (7, 25, 7, 1), (7, 31, 6, 1), (9, 32, 7, 1), (5, 33, 3, 1), (6, 47, 5, 1),
+         (6, 48, 5, 1), (6, 49, 5, 0), (6, 63, 7, 1), (7, 64, 7, 1)]
+
+
+@pytest.mark.parametrize("scale", [1e-3, 0.06, 0.4], ids=["tiny", "loop", "wide"])
+@pytest.mark.parametrize("nsub,m,window,taper", SIZES)
+def test_series_matches_oracle_and_eigensolve(nsub, m, window, taper, scale):
+    mask, geom, X, y, khat = problem(nsub, m, window, taper, scale)
+    ref = oracle.analysis(geom, X.astype(np.float64), y.astype(np.float64), SIGMA2, RHO)
+    Xa, mean, spread, st = analyse(mask, X, y, m, window, taper)
+    if khat.max() < 299:
+        assert st == (0, 1, geom.n_pts)             # every node by the series
+    assert rel(mean, ref[1]) <= 1e-4 and rel(spread, ref[2]) <= 1e-3
+    if khat.max() < 299:
+        def rms(v):
+            return float(np.sqrt(np.mean(np.square(v))))
+        Xb = X.astype(np.float64)
+        step = ref[1] - Xb.mean(-1)
+        unit = 2.0 ** -24
+        assert rms(Xa - ref[0]) <= 32 * unit * khat.max() * (rms(anoms(Xb)) + rms(step)) \
+            + 2 * unit * rms(Xb)
+    Xj, mj, sj, st = analyse(mask, X, y, m, window, taper, max_sweeps=20)
+    assert st[2] > geom.n_pts or m == 2 or scale == 1e-3
+    assert rel(mean, mj) <= 1e-4 and rel(spread, sj) <= 1e-3
+
+
+@pytest.mark.parametrize("kappa", [0.0, 300.0, 3.0], ids=["no-fp64", "default", "low"])
+@pytest.mark.parametrize("m,cls", [(12, 0), (24, 1), (32, 1), (40, 2)])
+def test_nodes_of_both_kinds_share_warps(m, cls, kappa):
+    """kappa_hat from about 1 to 1e4 along the grid: nodes of the series, of the Jacobi
+    sweeps (fp64_kappa = 0) and of the FP64 queue in one warp, each with its own degree;
+    the outputs meet the FP32 tolerances and do not depend on the tile shape."""
+    mask, geom, X, y, khat = problem(10, m, 5, 1, 0.3, ramp=(0.02, 10.0))
+    assert khat.min() < 2 and khat.max() > 1500
+    ref = oracle.analysis(geom, X.astype(np.float64), y.astype(np.float64), SIGMA2, RHO)
+    Xa, mean, spread, st = analyse(mask, X, y, m, 5, 1, fp64_kappa=kappa)
+    if kappa > 0:
+        assert abs(st[0] - int((khat > kappa).sum())) <= 2
+    assert rel(spread, ref[2]) <= 1e-3
+    # without FP64 the mean of the ill-conditioned nodes is not held to 1e-4
+    assert rel(mean, ref[1]) <= (1e-4 if kappa > 0 else 1e-2)
+    assert rel(anoms(Xa), anoms(ref[0])) <= 1e-3
+    for shape, (a, b) in enumerate(tile_shapes()):
+        if (a * b) % (4 if cls == 0 else 2 if cls == 1 else 1) or (cls == 2 and a * b > 8):
+            continue
+        Xs, *_ = analyse(mask, X, y, m, 5, 1, shape=shape, cls=cls, fp64_kappa=kappa)
+        assert np.array_equal(Xs, Xa), shape
+
+
+def test_nonfinite_node_problem_takes_the_eigensolve_and_is_reported():
+    from paper_1408_7069_gb300.letkf import LetkfError
+    mask, geom, X, y, _ = problem(6, 24, 5, 1, 0.06)
+    X[10, 1, 3] = np.inf
+    with pytest.raises(LetkfError, match="LETKF_ERR_NONFINITE"):
+        analyse(mask, X, y, 24, 5, 1)
