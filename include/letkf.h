@@ -80,7 +80,7 @@ typedef struct {
   uint64_t seed;               /* SplitMix64 seed of the forecast-noise draws */
   const float *noise_bank;     /* host [bank_B][bank_G][bank_G] screens, or NULL; copied */
   int32_t bank_B, bank_G;      /* bank shape (ignored when noise_bank is NULL) */
-  int32_t max_sweeps;          /* <= 0: FP32 node problems of moderate condition are solved by a
+  int32_t max_sweeps;          /* <= 0: node problems of moderate condition are solved by a
                                   Chebyshev series, the others by Jacobi sweeps (at most 20);
                                   > 0: every problem by Jacobi sweeps, at most this many */
   int32_t partition;           /* 0: every node is its own local domain (the per-node analysis);
@@ -352,12 +352,13 @@ letkf_status letkf_autotune(letkf_t h, const void *y_dev, int32_t reps, int32_t 
 letkf_status letkf_set_row_split(letkf_t h, int32_t width_class, int32_t split);
 
 /* Start of the FP64 eigensolve on FP64 handles (Section 4.2's EVD): warm = 1
- * (the default) runs the FP32 two-columns-per-lane eigensolve on the window
+ * (the default) solves well-conditioned nodes by a Chebyshev series (see
+ * letkf_config.max_sweeps) and for the others runs the FP32 two-columns-per-lane eigensolve on the window
  * rounded to FP32 first and starts each node's FP64 one-sided Jacobi from that
  * basis, made orthonormal to FP64 rounding by two Newton-Schulz steps, stopping after a
  * sweep whose cosines all stay below 1e-8 (the next would rotate by about its
- * square); warm = 0 starts from the identity and stops after a sweep without
- * rotations. Both give FP64 results (they differ by rounding). FP64 per-node
+ * square); warm = 0 takes every node by sweeps from the identity and stops after
+ * a sweep without rotations. Both give FP64 results (they differ by rounding). FP64 per-node
  * handles only (LETKF_ERR_ARG otherwise). The FP32 pass takes the class's
  * tile shape, so FP64 handles take the shapes of the whole-column FP32 form.
  * Synchronises; drops the cached CUDA graphs. */

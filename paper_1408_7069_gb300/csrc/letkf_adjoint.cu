@@ -100,15 +100,6 @@ __host__ __device__ size_t adj_warp_bytes(int w) {
          2 * align16((size_t)MP * (MP + 1) * sizeof(T)) + (size_t)S_N * MP * sizeof(T);
 }
 
-struct AdjArgs {
-  const double *lam_a;   // adjoint of this frame's analysis ensemble
-  double *xp_bar, *xbar_bar, *ybw, *dbw, *theta;
-  const double *dtap;
-  double rho, sigma2;
-  int max_sweeps;
-  int *counters;
-};
-
 // hi + lo += a * b with the product's and the sum's rounding errors kept in lo
 // (FMA two-product and Knuth's two-sum): a compensated FP32 accumulation. The
 // _rn intrinsics keep the compiler from contracting the steps into FMAs.
@@ -133,7 +124,7 @@ __global__ void __launch_bounds__(ADJ_WARPS * 32)
     adjoint_node_kernel(const LkInst *__restrict__ insts, const int2 *__restrict__ list,
                         const int *__restrict__ list_len, const float *__restrict__ U0,
                         const double *__restrict__ U64, float kappa_thr,
-                        int2 *__restrict__ queue, int *__restrict__ queue_len, T tol, AdjArgs a) {
+                        int2 *__restrict__ queue, int *__restrict__ queue_len, T tol, LkAdjArgs a) {
   constexpr bool kWarm = std::is_same<T, float>::value;
   LK_ADJ_STAMP(ph0);
   extern __shared__ __align__(16) unsigned char smem[];
@@ -679,11 +670,23 @@ size_t max_node_smem(const letkf_ctx *h) {
 }
 
 template <int MP>
-cudaError_t launch_nodes(letkf_ctx *h, LkAdjWork *W, const void *bk, const AdjArgs &a) {
+cudaError_t launch_nodes(letkf_ctx *h, LkAdjWork *W, const void *bk, const LkAdjArgs &a) {
   const LkInst &I = h->inst[0];
   const int blocks = (I.n_pts + ADJ_WARPS - 1) / ADJ_WARPS;
+  if (lk_series64(h)) {
+    // the series, then the nodes it queued from the eigenbases the forward
+    // list kernel stored for the same nodes
+    cudaError_t e = lk_launch_adj_series64(h, a);
+    if (e != cudaSuccess) return e;
+    adjoint_node_kernel<MP, double, double>
+        <<<blocks, ADJ_WARPS * 32, node_smem<MP, double, double>(I), h->stream>>>(
+            h->d_inst, W->queue, W->queue_len, nullptr, static_cast<const double *>(bk), 0.f,
+            nullptr, nullptr, h->tol64, a);
+    return cudaGetLastError();
+  }
   if (h->precision == 1) {
-    // FP64 handles: the FP64 eigenbasis the forward node64 kernel stored
+    // FP64 handles without the series: the FP64 eigenbasis the forward node64
+    // kernel stored for every node
     adjoint_node_kernel<MP, double, double>
         <<<blocks, ADJ_WARPS * 32, node_smem<MP, double, double>(I), h->stream>>>(
             h->d_inst, nullptr, nullptr, nullptr, static_cast<const double *>(bk), 0.f, nullptr,
@@ -759,7 +762,11 @@ letkf_status ensure_work(letkf_ctx *h, int frames, int ckpt) {
   if (e == cudaSuccess) e = walloc(&W->dtap, wc * sizeof(double));
   if (e == cudaSuccess) e = walloc(&W->queue, (size_t)I.n_pts * sizeof(int2));
   if (e == cudaSuccess) e = walloc(&W->queue_len, sizeof(int));
-  // slope adjoints of subapertures outside the pupil stay zero
+  // window cells outside the taper's support stay zero (the support changes only
+  // with the parameters, which drop this workspace), and so do the slope
+  // adjoints of subapertures outside the pupil
+  if (e == cudaSuccess) e = cudaMemset(W->ybw, 0, (size_t)I.n_pts * wc * 2 * I.m * sizeof(double));
+  if (e == cudaSuccess) e = cudaMemset(W->dbw, 0, (size_t)I.n_pts * wc * 2 * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(W->ybar, 0, cells * 2 * I.m * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(W->dbar, 0, cells * 2 * sizeof(double));
   if (e != cudaSuccess) {
@@ -832,7 +839,7 @@ cudaError_t backward_frame(letkf_ctx *h, LkAdjWork *W, const void *y_k, const vo
   if (e == cudaSuccess) e = lk_launch_obs(h, y_k, nullptr);
   if (e == cudaSuccess) e = cudaMemsetAsync(W->queue_len, 0, sizeof(int), h->stream);
   if (e != cudaSuccess) return e;
-  AdjArgs a;
+  LkAdjArgs a;
   a.lam_a = lam_in;
   a.xp_bar = W->xp_bar;
   a.xbar_bar = W->xbar_bar;
@@ -844,6 +851,8 @@ cudaError_t backward_frame(letkf_ctx *h, LkAdjWork *W, const void *y_k, const vo
   a.sigma2 = h->cfg.sigma2;
   a.max_sweeps = h->max_sweeps;
   a.counters = h->counters;
+  a.queue = W->queue;
+  a.queue_len = W->queue_len;
   e = I.mp == 16 ? launch_nodes<16>(h, W, bk, a) : launch_nodes<32>(h, W, bk, a);
   if (e != cudaSuccess) return e;
   theta_reduce_kernel<<<1, 256, 0, h->stream>>>(W->theta, I.n_pts, W->acc);

@@ -209,14 +209,21 @@ __device__ __forceinline__ void stage_tile(const LkInst &I, int i0, int j0, S *h
   for (int e = threadIdx.x; e < w * w; e += blockDim.x) tap[e] = T(taper[e]);
 }
 
-// One width class: FP64 handles run the FP32 basis pass of the pair kernel
-// (unless switched off) and one CTA per node (letkf_node64.cu); FP32 handles
-// the two-columns-per-lane kernel (letkf_pair.cu), then the FP64 analysis of
-// the nodes it queued.
+// One width class: FP64 handles run the Chebyshev series (letkf_series64.cu) and,
+// for the nodes it queued, the FP32 basis pass of the pair kernel and one CTA per
+// node (letkf_node64.cu); with the series off (an explicit sweep limit or a
+// cold start) those two take every node. FP32 handles run the
+// two-columns-per-lane kernel (letkf_pair.cu), then the FP64 analysis of the
+// nodes it queued.
 template <int MP>
 cudaError_t launch_class(letkf_ctx *h, int cls, void *mean, void *spread) {
   if (h->n_tiles[cls] == 0) return cudaSuccess;
   if (h->precision == 1) {
+    if (lk_series64(h)) {              // the others: FP32 bases, then the FP64 sweeps from them
+      cudaError_t e = lk_launch_series64(h, cls, mean, spread);
+      if (e == cudaSuccess) e = lk_launch_pair_basis(h, cls);
+      return e == cudaSuccess ? lk_launch_list64(h, cls, mean, spread) : e;
+    }
     if (h->fp64_warm) {
       const cudaError_t e = lk_launch_pair_basis(h, cls);
       if (e != cudaSuccess) return e;

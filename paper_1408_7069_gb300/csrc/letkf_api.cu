@@ -74,7 +74,8 @@ void release(letkf_ctx *h) {
   void *bufs[] = {h->X,          h->Ybp,      h->dp,       h->taper,    h->pid_map,
                   h->pts,        h->saps,     h->bank,     h->basis,    h->basis64,  h->counters,
                   h->worklist,   h->frame,    h->partial,  h->tickets,  h->d_inst,   h->obs_items,
-                  h->node_items, h->tiles[0], h->tiles[1], h->tiles[2], h->noise_pre, h->cheb32};
+                  h->node_items, h->tiles[0], h->tiles[1], h->tiles[2], h->noise_pre, h->cheb32,
+                  h->cheb64};
   for (void *p : bufs)
     if (p) cudaFree(p);
 }

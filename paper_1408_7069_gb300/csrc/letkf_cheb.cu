@@ -64,27 +64,45 @@ int cheb_series(double r, double tol, std::vector<double> &a, std::vector<double
 
 std::once_flag g_once;
 std::vector<float2> g_table32;
+std::vector<double2> g_table64;
+
+template <typename V, typename F>
+void fill_table(std::vector<V> &table, int classes, int ld, double tol, F pair) {
+  table.assign((size_t)classes * ld, pair(0.0, 0.0));
+  std::vector<double> a, b;
+  for (int c = 0; c < classes; ++c) {
+    const double r = LK_CHEB_R0 * pow(LK_CHEB_STEP, c);
+    const int deg = cheb_series(r, tol, a, b);
+    V *row = table.data() + (size_t)c * ld;
+    row[0] = pair(2.0 / r, deg);
+    for (int k = 0; k <= deg && k + 1 < ld; ++k) row[k + 1] = pair(a[k], b[k]);
+  }
+}
 
 void build_tables() {
-  g_table32.assign((size_t)LK_CHEB_CLASSES32 * LK_CHEB_LD32, make_float2(0.f, 0.f));
-  std::vector<double> a, b;
-  for (int c = 0; c < LK_CHEB_CLASSES32; ++c) {
-    const double r = LK_CHEB_R0 * pow(LK_CHEB_STEP, c);
-    const int deg = cheb_series(r, 1e-8, a, b);
-    float2 *row = g_table32.data() + (size_t)c * LK_CHEB_LD32;
-    row[0] = make_float2((float)(2.0 / r), (float)deg);
-    for (int k = 0; k <= deg && k + 1 < LK_CHEB_LD32; ++k)
-      row[k + 1] = make_float2((float)a[k], (float)b[k]);
-  }
+  fill_table(g_table32, LK_CHEB_CLASSES32, LK_CHEB_LD32, 1e-8,
+             [](double x, double y) { return make_float2((float)x, (float)y); });
+  fill_table(g_table64, LK_CHEB_CLASSES64, LK_CHEB_LD64, 1e-17,
+             [](double x, double y) { return make_double2(x, y); });
+}
+
+template <typename V>
+cudaError_t upload_table(V **dst, const std::vector<V> &table) {
+  cudaError_t e = cudaMalloc((void **)dst, table.size() * sizeof(V));
+  if (e == cudaSuccess)
+    e = cudaMemcpy(*dst, table.data(), table.size() * sizeof(V), cudaMemcpyHostToDevice);
+  return e;
 }
 
 }  // namespace
 
 cudaError_t lk_setup_cheb(letkf_ctx *h) {
   std::call_once(g_once, build_tables);
-  cudaError_t e = cudaMalloc((void **)&h->cheb32, g_table32.size() * sizeof(float2));
-  if (e == cudaSuccess)
-    e = cudaMemcpy(h->cheb32, g_table32.data(), g_table32.size() * sizeof(float2),
-                   cudaMemcpyHostToDevice);
-  return e;
+  if (h->precision == 0) return upload_table(&h->cheb32, g_table32);
+  const cudaError_t e = upload_table(&h->cheb64, g_table64);
+  return e == cudaSuccess ? lk_setup_series64(h) : e;
+}
+
+bool lk_series64(const letkf_ctx *h) {
+  return h->precision == 1 && h->fp64_warm && h->cheb64 != nullptr;
 }

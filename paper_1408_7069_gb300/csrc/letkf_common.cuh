@@ -45,6 +45,11 @@ constexpr double LK_WARM_STOP64 = 1e-8;
 constexpr double LK_CHEB_R0 = 0.25, LK_CHEB_STEP = 1.25;
 constexpr int LK_CHEB_CLASSES32 = 33, LK_CHEB_LD32 = 192;
 constexpr float LK_CHEB_MAX32 = 300.f;        // below the last class's 315.5
+// The FP64 table, truncated below FP64 rounding: classes up to 42.4, 128 terms.
+// Beyond, the products outnumber an eigensolve's work on the 0.5 FMA per clock
+// that an SM sub-partition issues.
+constexpr int LK_CHEB_CLASSES64 = 24, LK_CHEB_LD64 = 136;
+constexpr float LK_CHEB_MAX64 = 42.f;
 
 // One AO instance, as the kernels see it (device pointers, by-value copy in a
 // device array). The real type of X, Yb, d, y, truth, taper and the outputs is
@@ -103,6 +108,7 @@ struct letkf_ctx {
   double stop32 = 1e-3;             // FP32 Jacobi stops after a sweep with all cosines <= this
   int max_sweeps = 20;
   float2 *cheb32 = nullptr;         // FP32 Chebyshev table; NULL: every node by Jacobi sweeps
+  double2 *cheb64 = nullptr;        // the FP64 one (FP64 handles)
   int keep_basis = 0;               // store every node's eigenbasis (reverse mode needs it)
 
   int n_inst = 0;
@@ -211,6 +217,24 @@ cudaError_t lk_setup_analysis(letkf_ctx *h);
 // FP32 analysis of width class cls, two columns per lane (letkf_pair.cu).
 cudaError_t lk_launch_pair(letkf_ctx *h, int cls, void *mean, void *spread);
 cudaError_t lk_setup_pair(letkf_ctx *h);
+// Inputs and outputs of the reverse mode's node kernels (letkf_adjoint.cu).
+struct LkAdjArgs {
+  const double *lam_a;   // adjoint of this frame's analysis ensemble
+  double *xp_bar, *xbar_bar, *ybw, *dbw, *theta;
+  const double *dtap;
+  double rho, sigma2;
+  int max_sweeps;
+  int *counters;
+  int2 *queue;           // nodes left to the eigensolve form
+  int *queue_len;
+};
+// FP64 node problems by Chebyshev series (letkf_series64.cu): every node of
+// width class cls of an FP64 handle, those above LK_CHEB_MAX64 queued in the
+// class's worklist; and the adjoint of every node, likewise queued in a.queue.
+bool lk_series64(const letkf_ctx *h);     // whether the handle takes this form
+cudaError_t lk_launch_series64(letkf_ctx *h, int cls, void *mean, void *spread);
+cudaError_t lk_launch_adj_series64(letkf_ctx *h, const LkAdjArgs &a);
+cudaError_t lk_setup_series64(letkf_ctx *h);
 // Allocates and fills the handle's Chebyshev tables (letkf_cheb.cu).
 cudaError_t lk_setup_cheb(letkf_ctx *h);
 // FP64 analysis with one CTA of four warps per node (letkf_node64.cu): every

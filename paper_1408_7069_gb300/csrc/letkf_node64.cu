@@ -412,14 +412,15 @@ __global__ void __launch_bounds__(N64_THREADS)
                       keep_basis != 0, 2);
 }
 
-// FP32 handles: the nodes the pair kernel queued, a fixed grid of CTAs walking
-// the queue, each sweep started from the node's stored FP32 basis.
-template <int MP>
+// The nodes the pair kernel (FP32 handles) or the series (FP64 handles, with the
+// two Newton-Schulz steps their outputs need) queued, a fixed grid of CTAs
+// walking the queue, each sweep started from the node's stored FP32 basis.
+template <int MP, typename S>
 __global__ void __launch_bounds__(N64_THREADS)
     node64_list_kernel(const LkInst *__restrict__ insts, const int2 *__restrict__ worklist,
-                       const int *__restrict__ queue_len, float *__restrict__ mean,
-                       float *__restrict__ spread, double tol, int max_sweeps,
-                       int *__restrict__ counters) {
+                       const int *__restrict__ queue_len, S *__restrict__ mean,
+                       S *__restrict__ spread, double tol, int max_sweeps,
+                       int *__restrict__ counters, int keep_basis) {
   extern __shared__ __align__(16) double n64_smem[];
   lk_pdl_wait();   // no early trigger (long kernel): dependents launch as its CTAs exit
   const int qn = *queue_len;
@@ -427,9 +428,9 @@ __global__ void __launch_bounds__(N64_THREADS)
     const int2 it = worklist[idx];
     const LkInst &I = insts[it.x];
     const long long row = I.node_off + it.y;
-    node64<MP, float, true>(I, it.y, mean ? mean + 2 * row : nullptr,
-                            spread ? spread + 2 * row : nullptr, tol, LK_WARM_STOP64, max_sweeps,
-                            counters, n64_smem);
+    node64<MP, S, true>(I, it.y, mean ? mean + 2 * row : nullptr,
+                        spread ? spread + 2 * row : nullptr, tol, LK_WARM_STOP64, max_sweeps,
+                        counters, n64_smem, keep_basis != 0, sizeof(S) == 8 ? 2 : 1);
     __syncthreads();                       // shared memory is reused by the next node
   }
 }
@@ -789,9 +790,15 @@ cudaError_t launch_list64(letkf_ctx *h, int cls, void *mean, void *spread) {
   const long long cap = 4LL * n64_sm_count(h->device);
   const unsigned blocks = (unsigned)(n < cap ? n : cap);
   const size_t smem = n64_smem_doubles<MP>() * sizeof(double);
-  return lk_launch_pdl(node64_list_kernel<MP>, blocks, N64_THREADS, smem, h->stream, h->d_inst,
-                       h->worklist + (size_t)cls * h->n_pts_total, h->counters + 4 + cls,
-                       (float *)mean, (float *)spread, h->tol64, h->max_sweeps, h->counters);
+  const int2 *list = h->worklist + (size_t)cls * h->n_pts_total;
+  const int *len = h->counters + 4 + cls;
+  if (h->precision == 1)
+    return lk_launch_pdl(node64_list_kernel<MP, double>, blocks, N64_THREADS, smem, h->stream,
+                         h->d_inst, list, len, (double *)mean, (double *)spread, h->tol64,
+                         h->max_sweeps, h->counters, h->keep_basis);
+  return lk_launch_pdl(node64_list_kernel<MP, float>, blocks, N64_THREADS, smem, h->stream,
+                       h->d_inst, list, len, (float *)mean, (float *)spread, h->tol64,
+                       h->max_sweeps, h->counters, 0);
 }
 
 cudaError_t launch_list64w(letkf_ctx *h, void *mean, void *spread) {

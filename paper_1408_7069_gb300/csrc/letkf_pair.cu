@@ -393,8 +393,9 @@ struct PairLaunch {
 };
 
 // BASIS (FP64 handles, S = double): the FP32 eigensolve alone, storing every
-// node's eigenbasis as the start of the FP64 sweep of node64_kernel; nothing
-// is queued and X is not touched.
+// node's eigenbasis as the start of the FP64 sweeps of letkf_node64.cu; nothing
+// is queued and X is not touched. `queue`, if given: the length of the list of
+// nodes whose bases are wanted; nothing is done when it is zero.
 template <int MP, int TI, int TJ, typename S = float, bool BASIS = false>
 __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP, TI, TJ>::min_ctas)
     analysis_pair_kernel(const LkInst *__restrict__ insts, const LkTile *__restrict__ tiles,
@@ -407,6 +408,8 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
   using C = PairCfg<MP>;
   constexpr int K2 = C::K2, LPN = C::LPN, GL = C::GL;
   extern __shared__ __align__(16) unsigned char smem[];
+  if constexpr (BASIS)
+    if (queue && *queue == 0) return;
   const LkTile tl = tiles[blockIdx.x];
   const LkInst &I = insts[tl.inst];
   const int w = I.w, m = I.m;
@@ -474,7 +477,7 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
   // It still takes this FP32 eigensolve, whose basis is stored as the start of
   // the FP64 list kernel's sweep; X is left alone and the node is queued.
   bool queued = false;
-  if (queue) {
+  if (!BASIS && queue) {
     const float trg = group_sum<GL>(diag);
     if (active && 1.f + trg / alpha > kappa_thr) {
       if (li == 0) {
@@ -1123,7 +1126,8 @@ cudaError_t launch_basis_shape(letkf_ctx *h, int cls) {
     return lk_launch_pdl(analysis_pair_kernel<MP, TI, TJ, double, true>, h->n_tiles[cls],
                          TI * TJ * 32 / PairCfg<MP>::NPW, need, h->stream, h->d_inst,
                          h->tiles[cls], (float *)nullptr, (float *)nullptr, (float)h->tol32,
-                         (float)h->stop32, h->max_sweeps, 0.f, h->counters, (int *)nullptr,
+                         (float)h->stop32, h->max_sweeps, 0.f, h->counters,
+                         lk_series64(h) ? h->counters + 4 + cls : (int *)nullptr,
                          (int2 *)nullptr, 1, (const float2 *)nullptr);
   }
 }

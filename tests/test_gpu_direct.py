@@ -118,3 +118,65 @@ def test_nonfinite_node_problem_takes_the_eigensolve_and_is_reported():
     X[10, 1, 3] = np.inf
     with pytest.raises(LetkfError, match="LETKF_ERR_NONFINITE"):
         analyse(mask, X, y, 24, 5, 1)
+
+
+# ---------------------------------------------------------------------------
+# FP64 handles (letkf_series64.cu): the FP64 tolerances of the analysis tests, 1e-9 on
+# the mean and 1e-8 on the spread and the anomalies; gradients as in the reverse mode's
+# tests, 1e-8.
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("scale", [1e-3, 0.06, 0.3], ids=["tiny", "loop", "wide"])
+@pytest.mark.parametrize("nsub,m,window,taper",
+                         [(1, 2, 1, 0), (4, 7, 3, 1), (4, 8, 3, 1), (4, 9, 4, 0), (5, 16, 5, 1),
+                          (5, 17, 3, 1), (6, 24, 9, 1), (6, 25, 5, 0), (5, 32, 7, 1)])
+def test_fp64_series_matches_oracle(nsub, m, window, taper, scale):
+    mask, geom, X, y, khat = problem(nsub, m, window, taper, scale)
+    X, y = X.astype(np.float64), y.astype(np.float64)
+    ref = oracle.analysis(geom, X, y, SIGMA2, RHO)
+    Xa, mean, spread, st = analyse(mask, X, y, m, window, taper, precision=1)
+    if khat.max() < 42:
+        assert st[1:] == (1, geom.n_pts)
+    assert rel(mean, ref[1]) <= 1e-9 and rel(spread, ref[2]) <= 1e-8
+    assert rel(anoms(Xa), anoms(ref[0])) <= 1e-8
+
+
+def test_fp64_series_and_eigensolve_nodes_in_one_frame():
+    mask, geom, X, y, khat = problem(8, 20, 5, 1, 0.3, ramp=(0.02, 10.0))
+    X, y = X.astype(np.float64), y.astype(np.float64)
+    assert khat.min() < 2 and khat.max() > 1000
+    ref = oracle.analysis(geom, X, y, SIGMA2, RHO)
+    Xa, mean, spread, st = analyse(mask, X, y, 20, 5, 1, precision=1)
+    assert 1 < st[1] <= 20
+    assert rel(mean, ref[1]) <= 1e-9 and rel(spread, ref[2]) <= 1e-8
+    assert rel(anoms(Xa), anoms(ref[0])) <= 1e-8
+
+
+@pytest.mark.parametrize("nsub,m,window,taper,scale",
+                         [(3, 6, 3, 1, 0.06), (4, 12, 3, 1, 0.06), (4, 20, 5, 1, 0.1),
+                          (5, 24, 9, 0, 0.08), (4, 32, 7, 1, 0.1), (4, 24, 5, 0, 0.12)])
+def test_fp64_series_adjoint_matches_oracle(nsub, m, window, taper, scale):
+    """Gradients through the series: every column width, more slopes than one staged
+    chunk, degrees below and above what the kernel keeps of the terms."""
+    mask, geom, X, y0, khat = problem(nsub, m, window, taper, scale, square=True)
+    assert khat.max() < 60
+    frames, rng = 3, np.random.default_rng(nsub + m)
+    geom = oracle.build_geometry(mask, window, taper, window / 4.0)
+    X = X.astype(np.float64)
+    y = 0.3 * rng.standard_normal((frames, geom.p))
+    truth = rng.standard_normal((frames, geom.n_pts))
+    bank = rng.standard_normal((2, 16, 16)).astype(np.float32)
+    J, g, _ = oracle.closed_loop_grad(geom, truth, y, bank, m, SIGMA2, RHO, 0.999, scale, 9,
+                                      frames, X)
+    f = Letkf(mask, m=m, window=window, taper=taper, rho=RHO, sigma2=SIGMA2, a_ar1=0.999,
+              noise_std=scale, precision=1, seed=9, bank=bank)
+    f.set_state(torch.from_numpy(X).cuda())
+    Jg, gg = f.grad(frames, torch.from_numpy(y).cuda(), torch.from_numpy(truth).cuda(), 2)
+    Xg = f.get_state()
+    f.set_state(torch.from_numpy(X).cuda())
+    f.set_frame(0)
+    f.run(frames, torch.from_numpy(y).cuda())
+    f.sync()
+    assert torch.equal(Xg, f.get_state())               # the state letkf_run leaves
+    f.close()
+    assert Jg == pytest.approx(J, rel=1e-10)
+    assert np.all(np.abs(gg - g) <= 1e-8 * np.maximum(np.abs(g), 1e-6 * np.abs(g).max())), (gg, g)
