@@ -294,7 +294,8 @@ letkf_status letkf_step(letkf_t h, const void *y_host, const void *truth_host, v
  * form exact for equal eigenvalues, so windows with fewer slopes than m - 1
  * (exactly degenerate eigenvalues) need no special case. The backward pass
  * recomputes each node's eigenbasis from the one its forward analysis stored
- * (FP32), and in FP64 for the nodes that the FP64 fallback takes.
+ * (FP32), and in FP64 for the nodes that the FP64 fallback takes; FP64 handles
+ * differentiate the Chebyshev series of the nodes it solves instead.
  * y_seq_dev: device [frames][p] real; truth_seq_dev: device [frames][n_pts] real.
  * ckpt_every: frames per segment; the forward keeps the ensemble and bases at
  *   the start of every segment and the backward recomputes one segment at a

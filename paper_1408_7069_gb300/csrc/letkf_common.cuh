@@ -45,6 +45,7 @@ constexpr double LK_WARM_STOP64 = 1e-8;
 constexpr double LK_CHEB_R0 = 0.25, LK_CHEB_STEP = 1.25;
 constexpr int LK_CHEB_CLASSES32 = 33, LK_CHEB_LD32 = 192;
 constexpr float LK_CHEB_MAX32 = 300.f;        // below the last class's 315.5
+constexpr float LK_CHEB_MAXD = 100.f;         // multi-actuator domains: 94 products
 // The FP64 table, truncated below FP64 rounding: classes up to 42.4, 128 terms.
 // Beyond, the products outnumber an eigensolve's work on the 0.5 FMA per clock
 // that an SM sub-partition issues.

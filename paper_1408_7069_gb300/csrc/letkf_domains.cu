@@ -47,9 +47,11 @@ struct LkDom {
   int *node_dom = nullptr;                        // [n_pts]
   int2 *edges = nullptr;                          // [E] (i, j) point ids, dom(i) != dom(j)
   int *dedge_off = nullptr, *dedge = nullptr;     // per domain: incident edges, +(e+1) / -(e+1)
-  float *KT = nullptr;                            // [D][D] K transposed
+  float *K = nullptr;                             // [D][D] piston projection
+  float *bsum = nullptr;                          // [D][2] per-domain edge sums
+  int *sweep = nullptr;                           // [D] nonzero: left to the eigensolve
+  int series = 0, splits = 1;                     // the series form fits; CTAs per domain
   float *delta = nullptr;                         // [n_pts][2] mean increments
-  float *cpist = nullptr;                         // [D][2] piston constants
   std::vector<double> tau;                        // host: tau of each observed slope
   // one domain covering the grid (partition 1): the global ETKF pipeline
   int global = 0, kchunks = 0, mpt = 0;
@@ -75,6 +77,7 @@ struct DomArgs {
   const float *obs_w;
   float *mean, *spread, *delta;
   int *counters;
+  const int *sweep;      // domains to take (NULL: all)
   float tol, stop, kappa_thr;
   int max_sweeps, max_obs, max_rows;
 };
@@ -172,6 +175,7 @@ __global__ void __launch_bounds__(32 * RPL)
   const LkInst &I = insts[0];
   const int m = I.m, tid = threadIdx.x;
   const int dom = blockIdx.x;
+  if (a.sweep && !a.sweep[dom]) return;
   const int o0 = a.obs_off[dom], np = a.obs_off[dom + 1] - o0;
   const int n0 = a.node_off[dom], nd = 2 * (a.node_off[dom + 1] - n0);
   const DomLayout Ly = dom_layout(MPD, a.max_obs, a.max_rows);
@@ -341,60 +345,368 @@ __global__ void __launch_bounds__(32 * RPL)
   }
 }
 
-// b_d = sum over the border edges of domain d of (delta_other - delta_own) for
-// both state rows (a fixed order: the domain's incident edge list), then
-// c = K b with one thread per domain. One CTA.
-__global__ void __launch_bounds__(1024)
-    piston_solve_kernel(int n_dom, const int2 *__restrict__ edges, const int *__restrict__ dedge_off,
-                        const int *__restrict__ dedge, const float *__restrict__ delta,
-                        const float *__restrict__ KT, float *__restrict__ cpist) {
-  extern __shared__ __align__(16) float bsm[];   // [2][n_dom]
+// ---------------------------------------------------------------------------
+// The same update by Chebyshev series, without the eigensolve (direct_apply in
+// letkf_pair.cu describes the series): the domain's n_d anomaly rows and C d
+// as one more row form a (n_d + 1) x m block T, and a term is
+//   T_k+1 = 2 T_k X - T_k-1, X = 2 G / (alpha ratio) - I:
+// a small matrix product per term, summed with the coefficients of A^-1/2 (rows) and
+// A^-1 (the row of C d, which gives wbar). A converged loop's ratio of about 4
+// (m = 101, 128 slopes) takes 18 terms of 0.36 M FMAs, where the eigensolve's
+// eight sweeps take 14 M in rounds that each wait on two CTA barriers.
+// Domains above LK_CHEB_MAXD are left to domain_kernel (their `sweep` flag).
+//
+// CTA of 4 MPD threads per domain (or per part of a domain's rows, when the
+// domains are too few to fill the GPU; every part forms the same G). Products
+// in 4 x 4 register tiles: thread (row group, column group), rows fastest, so
+// that a warp's loads of T (stored [column][row]) and G are one or two
+// shared-memory wavefronts each for eight packed FMAs. T_k-1 and T_k stay in shared memory
+// (double-buffered, one barrier per term), which keeps the kernel at two CTAs
+// per SM.
+// ---------------------------------------------------------------------------
+constexpr int DS_ROWS = 63;      // rows per pass (and the row of C d: 16 row groups)
+
+struct DomSeriesLayout {
+  int rs, g, sv, xm, wb, red, total;       // offsets in floats; rs: row stride of T
+};
+__host__ __device__ inline DomSeriesLayout dom_series_layout(int mpd, int max_obs, int max_rows,
+                                                             int splits) {
+  DomSeriesLayout L;
+  int rows = (max_rows + splits - 1) / splits;
+  rows = rows < DS_ROWS ? rows : DS_ROWS;
+  L.rs = 4 * ((rows + 1 + 3) / 4);
+  const int s = max_obs * mpd, t = 2 * mpd * L.rs;
+  L.g = s > t ? s : t;                     // S, then the two buffers of T
+  L.sv = L.g + mpd * mpd;
+  L.xm = L.sv + (max_obs + 3) / 4 * 4;
+  L.wb = L.xm + L.rs;
+  L.red = L.wb + mpd;
+  L.total = L.red + 36;
+  return L;
+}
+
+template <int RPL>
+__global__ void __launch_bounds__(32 * RPL, RPL <= 13 ? 2 : 1)
+    domain_series_kernel(const LkInst *__restrict__ insts, DomArgs a, int *__restrict__ sweep,
+                         const float2 *__restrict__ cheb) {
+  constexpr int MPD = 8 * RPL, NT = 4 * MPD, CG = MPD / 4, TILES = CG * (CG + 1) / 2;
+  extern __shared__ __align__(16) float dsm[];
   lk_pdl_wait();
-  for (int d = threadIdx.x; d < n_dom; d += blockDim.x) {
-    float b0 = 0.f, b1 = 0.f;
-    for (int q = dedge_off[d]; q < dedge_off[d + 1]; ++q) {
-      const int se = dedge[q];
-      const int2 ed = edges[(se > 0 ? se : -se) - 1];
-      const int own = se > 0 ? ed.x : ed.y, oth = se > 0 ? ed.y : ed.x;
-      b0 += delta[2 * oth] - delta[2 * own];
-      b1 += delta[2 * oth + 1] - delta[2 * own + 1];
-    }
-    bsm[d] = b0;
-    bsm[n_dom + d] = b1;
+  const LkInst &I = insts[0];
+  const int m = I.m, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int dom = blockIdx.x, splits = gridDim.y;
+  const int o0 = a.obs_off[dom], np = a.obs_off[dom + 1] - o0;
+  const int n0 = a.node_off[dom], nd = 2 * (a.node_off[dom + 1] - n0);
+  const DomSeriesLayout Ly = dom_series_layout(MPD, a.max_obs, a.max_rows, splits);
+  float *S = dsm, *T = dsm, *G = dsm + Ly.g, *sv = dsm + Ly.sv, *xm = dsm + Ly.xm;
+  float *wb = dsm + Ly.wb, *red = dsm + Ly.red;
+  const float *Ybp = static_cast<const float *>(I.Ybp);
+  const float *dp = static_cast<const float *>(I.dp);
+  float *X = static_cast<float *>(I.X);
+  const float alpha = float(I.alpha);
+
+  // ---- S = diag(sqrt(tau/sigma2)) Yb of the region and s, a warp per slope ----
+  for (int k = warp; k < np; k += NT / 32) {
+    const int slot = a.obs_slot[o0 + k];
+    const float sw = sqrtf(a.obs_w[o0 + k]);
+    for (int i = lane; i < MPD; i += 32)
+      S[k * MPD + i] = i < m ? sw * Ybp[(size_t)slot * m + i] : 0.f;
+    if (lane == 0) sv[k] = sw * dp[slot];
   }
   __syncthreads();
-  for (int d = threadIdx.x; d < n_dom; d += blockDim.x) {
-    float c0 = 0.f, c1 = 0.f;
-    for (int e = 0; e < n_dom; ++e) {
-      const float k = KT[(size_t)e * n_dom + d];
-      c0 = fmaf(k, bsm[e], c0);
-      c1 = fmaf(k, bsm[n_dom + e], c1);
+  // ---- G = S^T S by 4 x 4 tiles of its lower triangle, c = S^T s, |G|_F, tr G ----
+  float fro = 0.f, tr = 0.f;
+  for (int tile = tid; tile < TILES; tile += NT) {
+    int ti = (int)((sqrtf(8.f * tile + 1.f) - 1.f) * 0.5f);
+    while (ti * (ti + 1) / 2 > tile) --ti;
+    while ((ti + 1) * (ti + 2) / 2 <= tile) ++ti;
+    const int tj = tile - ti * (ti + 1) / 2;
+    const float4 *pa = reinterpret_cast<const float4 *>(S) + ti;
+    const float4 *pb = reinterpret_cast<const float4 *>(S) + tj;
+    float2 acc[4][2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int k = 0; k < np; ++k) {
+      const float4 x = pa[k * CG], y = pb[k * CG];
+      const float yj[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 yy = make_float2(yj[j], yj[j]);
+        acc[j][0] = __ffma2_rn(make_float2(x.x, x.y), yy, acc[j][0]);
+        acc[j][1] = __ffma2_rn(make_float2(x.z, x.w), yy, acc[j][1]);
+      }
     }
-    cpist[2 * d] = c0;
-    cpist[2 * d + 1] = c1;
+    const float w2 = ti == tj ? 1.f : 2.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float v[4] = {acc[j][0].x, acc[j][0].y, acc[j][1].x, acc[j][1].y};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        G[(4 * tj + j) * MPD + 4 * ti + i] = v[i];
+        fro = fmaf(w2 * v[i], v[i], fro);
+        if (ti == tj && i == j) tr += v[i];
+      }
+      if (ti != tj)
+        for (int i = 0; i < 4; ++i) G[(4 * ti + i) * MPD + 4 * tj + j] = v[i];
+    }
+  }
+  if (tid < MPD) {
+    float c = 0.f;
+    for (int k = 0; k < np; ++k) c = fmaf(S[k * MPD + tid], sv[k], c);
+    wb[tid] = c;
+  }
+  fro = lk_warp_sum(fro);
+  tr = lk_warp_sum(tr);
+  if (lane == 0) {
+    red[warp] = fro;
+    red[16 + warp] = tr;
+  }
+  __syncthreads();
+  fro = tr = 0.f;
+  for (int k = 0; k < NT / 32; ++k) {
+    fro += red[k];
+    tr += red[16 + k];
+  }
+  const float ratio = sqrtf(fro) / alpha;
+  const bool ok = ratio <= LK_CHEB_MAXD;             // (not with a NaN)
+  if (tid == 0 && blockIdx.y == 0) {
+    sweep[dom] = !ok;
+    if (ok) {
+      atomicMax(&a.counters[2], 1);
+      atomicAdd(&a.counters[3], 1);
+      if (a.kappa_thr > 0.f && 1.f + tr / alpha > a.kappa_thr) atomicAdd(&a.counters[1], 1);
+    }
+  }
+  if (!ok) return;
+  const int cls = lk_cheb_class(ratio);
+  const float2 *co = cheb + (size_t)cls * LK_CHEB_LD32;
+  const float2 head = __ldg(co++);
+  const float scale = head.x / alpha;
+  const int deg = (int)head.y;
+  const float inv_m = 1.f / float(m), rt = sqrtf(float(m - 1) / alpha);
+  const int per = (nd + splits - 1) / splits;
+  const int rbeg = blockIdx.y * per, rend = rbeg + per < nd ? rbeg + per : nd;
+  float creg = tid < MPD ? wb[tid] : 0.f;            // C d, kept across the passes
+
+  for (int r0 = rbeg; r0 < rend; r0 += DS_ROWS) {
+    const int nr = rend - r0 < DS_ROWS ? rend - r0 : DS_ROWS;   // rows of this pass
+    const int RT = (nr + 1 + 3) / 4, rs = 4 * RT;
+    __syncthreads();
+    // ---- T_0: anomaly rows (a warp per row), C d, zero rows up to rs ----
+    for (int r = warp; r < nr; r += NT / 32) {
+      const int pid = a.node_ids[n0 + ((r0 + r) >> 1)];
+      const float *x = X + ((size_t)pid * 2 + ((r0 + r) & 1)) * m;
+      float v[(MPD + 31) / 32], sum = 0.f;
+#pragma unroll
+      for (int q = 0; q < (MPD + 31) / 32; ++q) {
+        const int j = lane + 32 * q;
+        v[q] = j < m ? x[j] : 0.f;
+        sum += v[q];
+      }
+      const float mu = lk_warp_sum(sum) * inv_m;
+#pragma unroll
+      for (int q = 0; q < (MPD + 31) / 32; ++q) {
+        const int j = lane + 32 * q;
+        if (j < MPD) T[j * rs + r] = j < m ? v[q] - mu : 0.f;
+      }
+      if (lane == 0) xm[r] = mu;
+    }
+    if (tid < MPD) {
+      T[tid * rs + nr] = creg;
+      for (int r = nr + 1; r < rs; ++r) T[tid * rs + r] = 0.f;
+    }
+    __syncthreads();
+    // ---- the series on this thread's tile: rows 4 rg + i, columns 4 cg + j ----
+    const int rg = tid % RT, cg = tid / RT;
+    const bool work = cg < CG;
+    float2 u[4][2];
+    float f = scale, e = 1.f, o = 0.f;
+    const int ci = nr - 4 * rg;                      // 0..3: C d is this tile's row ci
+    for (int k = 0; k <= deg; ++k) {
+      float *cur = T + (k & 1) * MPD * rs, *nxt = T + ((k + 1) & 1) * MPD * rs;
+      const float2 c = __ldg(co + k);
+      const float2 c01 = make_float2(ci == 0 ? c.y : c.x, ci == 1 ? c.y : c.x);
+      const float2 c23 = make_float2(ci == 2 ? c.y : c.x, ci == 3 ? c.y : c.x);
+      if (work) {
+        float4 *ct = reinterpret_cast<float4 *>(cur) + cg * 4 * RT + rg;
+        float4 *nt = reinterpret_cast<float4 *>(nxt) + cg * 4 * RT + rg;
+        if (k == 0) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float4 t = ct[j * RT];
+            u[j][0] = __fmul2_rn(c01, make_float2(t.x, t.y));
+            u[j][1] = __fmul2_rn(c23, make_float2(t.z, t.w));
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float4 t = ct[j * RT];
+            u[j][0] = __ffma2_rn(c01, make_float2(t.x, t.y), u[j][0]);
+            u[j][1] = __ffma2_rn(c23, make_float2(t.z, t.w), u[j][1]);
+          }
+        }
+        if (k < deg) {
+          float2 acc[4][2];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
+          const float4 *pt = reinterpret_cast<const float4 *>(cur) + rg;
+          const float4 *pg = reinterpret_cast<const float4 *>(G) + cg;
+#pragma unroll 4
+          for (int q = 0; q < MPD; ++q) {
+            const float4 x = pt[q * RT], y = pg[q * CG];
+            const float yj[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float2 yy = make_float2(yj[j], yj[j]);
+              acc[j][0] = __ffma2_rn(make_float2(x.x, x.y), yy, acc[j][0]);
+              acc[j][1] = __ffma2_rn(make_float2(x.z, x.w), yy, acc[j][1]);
+            }
+          }
+          // T_k+1 = f T_k G - e T_k - o T_k-1 (f, e, o = scale, 1, 0, then 2 scale, 2, 1)
+          const float2 ff = make_float2(f, f), ee = make_float2(-e, -e), oo = make_float2(-o, -o);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float4 t = ct[j * RT];
+            float4 pv = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (k) pv = nt[j * RT];
+            const float2 n0v = __ffma2_rn(ff, acc[j][0], __ffma2_rn(ee, make_float2(t.x, t.y),
+                                          __fmul2_rn(oo, make_float2(pv.x, pv.y))));
+            const float2 n1v = __ffma2_rn(ff, acc[j][1], __ffma2_rn(ee, make_float2(t.z, t.w),
+                                          __fmul2_rn(oo, make_float2(pv.z, pv.w))));
+            nt[j * RT] = make_float4(n0v.x, n0v.y, n1v.x, n1v.y);
+          }
+        }
+      }
+      f = 2.f * scale;
+      e = 2.f;
+      o = 1.f;
+      __syncthreads();
+    }
+    // ---- the sums, row-major in the first buffer; wbar ----
+    if (work) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = 4 * rg + i;
+        const float v[4] = {i & 1 ? u[0][i >> 1].y : u[0][i >> 1].x,
+                            i & 1 ? u[1][i >> 1].y : u[1][i >> 1].x,
+                            i & 1 ? u[2][i >> 1].y : u[2][i >> 1].x,
+                            i & 1 ? u[3][i >> 1].y : u[3][i >> 1].x};
+        if (r == nr)
+          for (int j = 0; j < 4; ++j) wb[4 * cg + j] = v[j] / alpha;
+        else if (r < nr)
+          reinterpret_cast<float4 *>(T + (size_t)r * MPD)[cg] =
+              make_float4(v[0], v[1], v[2], v[3]);
+      }
+    }
+    __syncthreads();
+    // ---- apply, a warp per row: Xa_r = xbar_r + X'_r wbar + sqrt((m-1)/alpha) u_r ----
+    for (int r = warp; r < nr; r += NT / 32) {
+      const int pid = a.node_ids[n0 + ((r0 + r) >> 1)], comp = (r0 + r) & 1;
+      float *x = X + ((size_t)pid * 2 + comp) * m;
+      const float mu0 = xm[r];
+      float v[(MPD + 31) / 32], w = 0.f;
+#pragma unroll
+      for (int q = 0; q < (MPD + 31) / 32; ++q) {
+        const int j = lane + 32 * q;
+        if (j < m) w = fmaf(x[j] - mu0, wb[j], w);
+      }
+      w = lk_warp_sum(w);
+      float sum = 0.f;
+#pragma unroll
+      for (int q = 0; q < (MPD + 31) / 32; ++q) {
+        const int j = lane + 32 * q;
+        v[q] = 0.f;
+        if (j < m) {
+          v[q] = mu0 + w + rt * T[(size_t)r * MPD + j];
+          x[j] = v[q];
+        }
+        sum += v[q];
+      }
+      const float mu = lk_warp_sum(sum) * inv_m;
+      float sq = 0.f;
+#pragma unroll
+      for (int q = 0; q < (MPD + 31) / 32; ++q) {
+        const float d = lane + 32 * q < m ? v[q] - mu : 0.f;
+        sq = fmaf(d, d, sq);
+      }
+      const float sp = sqrtf(lk_warp_sum(sq) / float(m - 1));
+      if (lane == 0) {
+        if (a.mean) a.mean[(size_t)pid * 2 + comp] = mu;
+        if (a.spread) a.spread[(size_t)pid * 2 + comp] = sp;
+        a.delta[(size_t)pid * 2 + comp] = mu - mu0;
+        if (!isfinite(mu) || !isfinite(sp)) atomicOr(&a.counters[0], LK_BIT_NONFINITE);
+      }
+    }
   }
 }
 
-// Every member of every node row moves by its domain's constant (and so does
-// the analysis mean). A warp per node.
+// b_d = sum over the border edges of domain d of (delta_other - delta_own) for
+// both state rows: a warp per domain, its incident edges over the lanes.
 __global__ void __launch_bounds__(LK_WARP_CTA)
-    piston_apply_kernel(const LkInst *__restrict__ insts, const int *__restrict__ node_dom,
-                        const float *__restrict__ cpist, float *__restrict__ mean) {
+    piston_sum_kernel(int n_dom, const int2 *__restrict__ edges, const int *__restrict__ dedge_off,
+                      const int *__restrict__ dedge, const float *__restrict__ delta,
+                      float *__restrict__ bsum) {
+  lk_pdl_wait();
+  lk_pdl_trigger();
+  const int d = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (d >= n_dom) return;
+  float b0 = 0.f, b1 = 0.f;
+  for (int q = dedge_off[d] + lane; q < dedge_off[d + 1]; q += 32) {
+    const int se = dedge[q];
+    const int2 ed = edges[(se > 0 ? se : -se) - 1];
+    const int own = se > 0 ? ed.x : ed.y, oth = se > 0 ? ed.y : ed.x;
+    b0 += delta[2 * oth] - delta[2 * own];
+    b1 += delta[2 * oth + 1] - delta[2 * own + 1];
+  }
+  b0 = lk_warp_sum(b0);
+  b1 = lk_warp_sum(b1);
+  if (lane == 0) {
+    bsum[2 * d] = b0;
+    bsum[2 * d + 1] = b1;
+  }
+}
+
+// c_d = (K b)_d, then every member of the domain's rows moves by it (and so does
+// the analysis mean): a CTA per domain, so that the product's n_dom^2 terms are
+// read by as many CTAs as there are rows (one CTA for all took 17 us at 75
+// domains and 53 us at 373; the two kernels take about 3 us each).
+__global__ void __launch_bounds__(128)
+    piston_apply_kernel(const LkInst *__restrict__ insts, int n_dom,
+                        const int *__restrict__ node_off, const int *__restrict__ node_ids,
+                        const float *__restrict__ K, const float *__restrict__ bsum,
+                        float *__restrict__ mean) {
+  __shared__ float part[2][4];
   lk_pdl_wait();
   const LkInst &I = insts[0];
-  const int node = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (node >= I.n_pts) return;
-  const int d = node_dom[node];
-  const float c0 = cpist[2 * d], c1 = cpist[2 * d + 1];
-  float *x = static_cast<float *>(I.X) + (size_t)node * 2 * I.m;
-  for (int j = lane; j < I.m; j += 32) {
-    x[j] += c0;
-    x[I.m + j] += c1;
+  const int d = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float c0 = 0.f, c1 = 0.f;
+  for (int e = threadIdx.x; e < n_dom; e += 128) {
+    const float k = K[(size_t)d * n_dom + e];
+    const float2 b = reinterpret_cast<const float2 *>(bsum)[e];
+    c0 = fmaf(k, b.x, c0);
+    c1 = fmaf(k, b.y, c1);
   }
-  if (lane == 0 && mean) {
-    mean[2 * node] += c0;
-    mean[2 * node + 1] += c1;
+  c0 = lk_warp_sum(c0);
+  c1 = lk_warp_sum(c1);
+  if (lane == 0) {
+    part[0][warp] = c0;
+    part[1][warp] = c1;
+  }
+  __syncthreads();
+  c0 = (part[0][0] + part[0][1]) + (part[0][2] + part[0][3]);
+  c1 = (part[1][0] + part[1][1]) + (part[1][2] + part[1][3]);
+  for (int q = node_off[d] + warp; q < node_off[d + 1]; q += 4) {
+    const int node = node_ids[q];
+    float *x = static_cast<float *>(I.X) + (size_t)node * 2 * I.m;
+    for (int j = lane; j < I.m; j += 32) {
+      x[j] += c0;
+      x[I.m + j] += c1;
+    }
+    if (lane == 0 && mean) {
+      mean[2 * node] += c0;
+      mean[2 * node + 1] += c1;
+    }
   }
 }
 
@@ -716,8 +1028,17 @@ cudaError_t setup_global_rpl(const LkDom &D, int m) {
 }
 
 template <int RPL>
-cudaError_t launch_rpl(letkf_ctx *h, const DomArgs &a) {
+cudaError_t launch_rpl(letkf_ctx *h, DomArgs a) {
   const LkDom &D = *h->dom;
+  if (D.series && h->cheb32) {
+    const size_t b = sizeof(float) * (size_t)dom_series_layout(8 * RPL, D.max_obs, 2 * D.max_nodes,
+                                                               D.splits).total;
+    const cudaError_t e =
+        lk_launch_pdl(domain_series_kernel<RPL>, dim3(D.n_dom, D.splits), 32 * RPL, b, h->stream,
+                      h->d_inst, a, D.sweep, (const float2 *)h->cheb32);
+    if (e != cudaSuccess) return e;
+    a.sweep = D.sweep;                 // the others, if any
+  }
   const size_t smem = (size_t)dom_layout(8 * RPL, D.max_obs, 2 * D.max_nodes).total * sizeof(float);
   return lk_launch_pdl(domain_kernel<RPL>, (unsigned)D.n_dom, 32 * RPL, smem, h->stream,
                        h->d_inst, a);
@@ -726,8 +1047,14 @@ cudaError_t launch_rpl(letkf_ctx *h, const DomArgs &a) {
 template <int RPL>
 cudaError_t setup_rpl(const LkDom &D) {
   const size_t smem = (size_t)dom_layout(8 * RPL, D.max_obs, 2 * D.max_nodes).total * sizeof(float);
-  return cudaFuncSetAttribute(domain_kernel<RPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem);
+  const cudaError_t e = cudaFuncSetAttribute(domain_kernel<RPL>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+  if (e != cudaSuccess || !D.series) return e;
+  const size_t b = sizeof(float) * (size_t)dom_series_layout(8 * RPL, D.max_obs, 2 * D.max_nodes,
+                                                             D.splits).total;
+  return cudaFuncSetAttribute(domain_series_kernel<RPL>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b);
 }
 
 // Rows per lane of the Jacobi layout (MPD = 8 RPL columns); 0: wider than the
@@ -862,6 +1189,17 @@ letkf_status lk_domains_build(letkf_ctx *h, const letkf_config &c, const std::ve
           "smaller window or fewer members)";
     return LETKF_ERR_ARG;
   }
+  // The series form, where its shared memory fits too. Systems of so few domains
+  // that half the SMs would idle give each domain's rows to two or more CTAs (at
+  // least 8 rows each): the products, most of the work, split, the Gram repeats.
+  int sms = 1;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+  if (!D->global) {
+    D->splits = std::max(1, std::min({sms / std::max(1, D->n_dom), 2 * D->max_nodes / 8, 4}));
+    const size_t b = sizeof(float) * (size_t)dom_series_layout(mpd, D->max_obs, 2 * D->max_nodes,
+                                                               D->splits).total;
+    D->series = b <= (size_t)dev_smem;
+  }
   // border edges and their incidence per domain
   std::vector<int2> edges;
   for (size_t q = 0; q < pts.size(); ++q) {
@@ -933,10 +1271,10 @@ letkf_status lk_domains_build(letkf_ctx *h, const letkf_config &c, const std::ve
     const double wd = (node_off[d + 1] - node_off[d]) / cnodes[comp[d]];
     for (int b = 0; b < Dn; ++b) wrow[(size_t)comp[d] * Dn + b] += wd * Lp[(size_t)d * Dn + b];
   }
-  std::vector<float> KT((size_t)Dn * Dn);
+  std::vector<float> K((size_t)Dn * Dn);
   for (int a = 0; a < Dn; ++a)
     for (int b = 0; b < Dn; ++b)
-      KT[(size_t)b * Dn + a] = (float)(Lp[(size_t)a * Dn + b] - wrow[(size_t)comp[a] * Dn + b]);
+      K[(size_t)a * Dn + b] = (float)(Lp[(size_t)a * Dn + b] - wrow[(size_t)comp[a] * Dn + b]);
   std::vector<float> wv(D->tau.size());
   for (size_t q = 0; q < wv.size(); ++q) wv[q] = (float)(D->tau[q] / c.sigma2);
   cudaError_t e = dup(&D->node_off, node_off);
@@ -948,9 +1286,10 @@ letkf_status lk_domains_build(letkf_ctx *h, const letkf_config &c, const std::ve
   if (e == cudaSuccess && !edges.empty()) e = dup(&D->edges, edges);
   if (e == cudaSuccess) e = dup(&D->dedge_off, dedge_off);
   if (e == cudaSuccess && !dedge.empty()) e = dup(&D->dedge, dedge);
-  if (e == cudaSuccess) e = dup(&D->KT, KT);
+  if (e == cudaSuccess) e = dup(&D->K, K);
   if (e == cudaSuccess) e = cudaMalloc((void **)&D->delta, pts.size() * 2 * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc((void **)&D->cpist, (size_t)Dn * 2 * sizeof(float));
+  if (e == cudaSuccess) e = cudaMalloc((void **)&D->bsum, (size_t)Dn * 2 * sizeof(float));
+  if (e == cudaSuccess) e = cudaMalloc((void **)&D->sweep, (size_t)Dn * sizeof(int));
   if (e == cudaSuccess && D->global) {
     const int mpt = D->rpl ? gl_mpt(mpd) : mpd;
     D->mpt = mpt;
@@ -1002,7 +1341,7 @@ void lk_domains_release(letkf_ctx *h) {
   LkDom *D = h->dom;
   if (!D) return;
   void *bufs[] = {D->node_off, D->node_ids, D->obs_off, D->obs_slot, D->obs_w, D->node_dom,
-                  D->edges,    D->dedge_off, D->dedge,   D->KT,       D->delta, D->cpist,
+                  D->edges,    D->dedge_off, D->dedge,   D->K,        D->delta, D->bsum, D->sweep,
                   D->gpart,    D->cpart,     D->T,       D->ns_ws};
   for (void *p : bufs)
     if (p) cudaFree(p);
@@ -1060,6 +1399,7 @@ cudaError_t lk_launch_domains(letkf_ctx *h, void *mean, void *spread) {
   a.spread = static_cast<float *>(spread);
   a.delta = D.delta;
   a.counters = h->counters;
+  a.sweep = nullptr;
   a.tol = (float)h->tol32;
   a.stop = (float)(h->stop32 > h->tol32 ? h->stop32 : h->tol32);
   a.kappa_thr = h->fp64_kappa > 0 ? (float)h->fp64_kappa : 0.f;
@@ -1075,12 +1415,11 @@ cudaError_t lk_launch_domains(letkf_ctx *h, void *mean, void *spread) {
     default: e = launch_rpl<16>(h, a); break;
   }
   if (e != cudaSuccess || !D.piston || D.n_dom < 2) return e;
-  e = lk_launch_pdl(piston_solve_kernel, 1, 1024, (size_t)2 * D.n_dom * sizeof(float), h->stream,
-                    D.n_dom, (const int2 *)D.edges, (const int *)D.dedge_off,
-                    (const int *)D.dedge, (const float *)D.delta, (const float *)D.KT, D.cpist);
+  e = lk_launch_pdl(piston_sum_kernel, (unsigned)((D.n_dom * 32 + LK_WARP_CTA - 1) / LK_WARP_CTA),
+                    LK_WARP_CTA, 0, h->stream, D.n_dom, (const int2 *)D.edges,
+                    (const int *)D.dedge_off, (const int *)D.dedge, (const float *)D.delta, D.bsum);
   if (e != cudaSuccess) return e;
-  const LkInst &I = h->inst[0];
-  const unsigned blocks = (unsigned)(((long long)I.n_pts * 32 + LK_WARP_CTA - 1) / LK_WARP_CTA);
-  return lk_launch_pdl(piston_apply_kernel, blocks, LK_WARP_CTA, 0, h->stream, h->d_inst,
-                       (const int *)D.node_dom, (const float *)D.cpist, static_cast<float *>(mean));
+  return lk_launch_pdl(piston_apply_kernel, (unsigned)D.n_dom, 128, 0, h->stream, h->d_inst,
+                       D.n_dom, (const int *)D.node_off, (const int *)D.node_ids,
+                       (const float *)D.K, (const float *)D.bsum, static_cast<float *>(mean));
 }

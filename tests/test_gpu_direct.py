@@ -180,3 +180,76 @@ def test_fp64_series_adjoint_matches_oracle(nsub, m, window, taper, scale):
     f.close()
     assert Jg == pytest.approx(J, rel=1e-10)
     assert np.all(np.abs(gg - g) <= 1e-8 * np.maximum(np.abs(g), 1e-6 * np.abs(g).max())), (gg, g)
+
+
+# ---------------------------------------------------------------------------
+# Multi-actuator domains (domain_series_kernel)
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("scale", [0.02, 0.08], ids=["small", "loop"])
+@pytest.mark.parametrize("nsub,m,window,parts,piston",
+                         [(8, 2, 3, 3, 1), (9, 16, 3, 3, 1), (9, 17, 3, 4, 0), (12, 32, 5, 3, 1),
+                          (12, 33, 3, 2, 1), (14, 64, 5, 4, 0), (14, 65, 3, 2, 1),
+                          (16, 101, 5, 4, 1), (20, 104, 5, 7, 1), (12, 105, 3, 3, 1),
+                          (12, 128, 5, 3, 1)])
+def test_domain_series_matches_oracle(nsub, m, window, parts, piston, scale):
+    """Every column width, one to four CTAs per domain, domains of more than one pass of
+    63 rows; the FP32 tolerances of the domain tests, and the anomalies to the series'
+    own bound (see the module docstring; the domains' kappa_hat in place of the nodes')."""
+    from oracle import letkf_domains as LD
+    mask = synth.pupil_subap_mask(nsub, 0.0)
+    dg = LD.build_domains(mask, parts, window, 1, 0.0)
+    rng = np.random.default_rng(100 * nsub + m)
+    n = dg.geom.n_pts
+    X = (3 * rng.standard_normal((n, 2, 1)) + scale * rng.standard_normal((n, 2, m)))
+    X = X.astype(np.float32)
+    y = rng.standard_normal(dg.geom.p).astype(np.float32)
+    Xb = X.astype(np.float64)
+    rXa, rmean, rspread, parts_, _ = LD.analysis_domains(dg, Xb, y.astype(np.float64), SIGMA2, RHO,
+                                                         piston=bool(piston), return_parts=True)
+    khat = max(np.trace(A) / ((m - 1) / RHO) - m + 1 for A, _, _ in parts_)
+    ratio = max(np.linalg.norm(A - (m - 1) / RHO * np.eye(m)) / ((m - 1) / RHO)
+                for A, _, _ in parts_)
+    f = Letkf(mask, m=m, window=window, taper=1, rho=RHO, sigma2=SIGMA2, partition=parts,
+              piston=piston)
+    f.set_state(torch.from_numpy(X).cuda())
+    mean, spread = f.analyze(torch.from_numpy(y).cuda())
+    f.sync()
+    st = f.stats()
+    Xa = f.get_state().cpu().numpy()
+    f.close()
+    if ratio < 99:
+        assert st[1:] == (1, dg.n_dom)
+    mean, spread = mean.cpu().numpy(), spread.cpu().numpy()
+    assert rel(mean, rmean) <= 1e-4 and rel(spread, rspread) <= 1e-3
+    step = rmean - Xb.mean(-1)
+    unit, rms = 2.0 ** -24, lambda v: float(np.sqrt(np.mean(np.square(v))))
+    if ratio < 99:
+        assert rms(Xa - rXa) <= 32 * unit * khat * (rms(anoms(Xb)) + rms(step)) \
+            + 2 * unit * rms(Xb)
+
+
+def test_domains_of_both_kinds_in_one_frame():
+    """Anomalies growing along the grid: well-conditioned domains by the series, the
+    others by the sweeps, in one frame; every domain counted once."""
+    from oracle import letkf_domains as LD
+    nsub, m, window, parts = 16, 48, 5, 5
+    mask = synth.pupil_subap_mask(nsub, 0.0)
+    dg = LD.build_domains(mask, parts, window, 1, 0.0)
+    n = dg.geom.n_pts
+    rng = np.random.default_rng(77)
+    s = 0.05 * np.geomspace(0.2, 100.0, n)
+    X = (3 * rng.standard_normal((n, 2, 1))
+         + s[:, None, None] * rng.standard_normal((n, 2, m))).astype(np.float32)
+    y = rng.standard_normal(dg.geom.p).astype(np.float32)
+    rXa, rmean, rspread = LD.analysis_domains(dg, X.astype(np.float64), y.astype(np.float64),
+                                              SIGMA2, RHO, piston=False)
+    f = Letkf(mask, m=m, window=window, taper=1, rho=RHO, sigma2=SIGMA2, partition=parts)
+    f.set_state(torch.from_numpy(X).cuda())
+    mean, spread = f.analyze(torch.from_numpy(y).cuda())
+    f.sync()
+    st = f.stats()
+    Xa = f.get_state().cpu().numpy()
+    f.close()
+    assert 1 < st[1] <= 20 and st[2] > dg.n_dom and 0 < st[0] < dg.n_dom
+    assert rel(spread.cpu().numpy(), rspread) <= 1e-3
+    assert rel(anoms(Xa), anoms(rXa)) <= 1e-3
