@@ -347,114 +347,174 @@ __global__ void __launch_bounds__(32 * RPL)
 
 // ---------------------------------------------------------------------------
 // The same update by Chebyshev series, without the eigensolve (direct_apply in
-// letkf_pair.cu describes the series): the domain's n_d anomaly rows and C d
-// as one more row form a (n_d + 1) x m block T, and a term is
+// letkf_pair.cu describes the series): with the domain's n_d anomaly rows as
+// a block T_0, a term is
 //   T_k+1 = 2 T_k X - T_k-1, X = 2 G / (alpha ratio) - I:
-// a small matrix product per term, summed with the coefficients of A^-1/2 (rows) and
-// A^-1 (the row of C d, which gives wbar). A converged loop's ratio of about 4
-// (m = 101, 128 slopes) takes 18 terms of 0.36 M FMAs, where the eigensolve's
-// eight sweeps take 14 M in rounds that each wait on two CTA barriers.
-// Domains above LK_CHEB_MAXD are left to domain_kernel (their `sweep` flag).
+// a small matrix product per term, summed with the coefficients of A^-1/2 and of
+// A^-1 (whose rows' products with C d are the rows' X'_r wbar). A converged loop's
+// ratio of about 4-7 (m = 101, 128 slopes) takes 18-21 terms of 0.35 M FMAs, where
+// the eigensolve's eight sweeps take 14 M in rounds that each wait on two CTA
+// barriers. Domains above LK_CHEB_MAXD are left to domain_kernel (their `sweep`
+// flag).
 //
-// CTA of 4 MPD threads per domain (or per part of a domain's rows, when the
-// domains are too few to fill the GPU; every part forms the same G). Products
-// in 4 x 4 register tiles: thread (row group, column group), rows fastest, so
-// that a warp's loads of T (stored [column][row]) and G are one or two
-// shared-memory wavefronts each for eight packed FMAs. T_k-1 and T_k stay in shared memory
-// (double-buffered, one barrier per term), which keeps the kernel at two CTAs
-// per SM.
+// A CTA per domain, or per part of a domain's rows when the domains are too few
+// to fill the GPU (every part forms the same G). Products in 4 x 4 register
+// tiles, eight packed FMAs per two 16-byte shared-memory loads. A 16-byte load
+// of a warp costs 2 clocks per eight different addresses (measured), so a warp's
+// tiles are 8 row groups x 4 column groups (4 x 8 for at most 16 rows): 4
+// clocks of loads against 4.3 of FMAs per column of the product and SM. T_k-1 and T_k
+// stay in shared memory ([column][row], double-buffered), G in full.
+// At most 16 rows leave half of the warps: there the two halves take half of the
+// product's columns each and add up through shared memory.
 // ---------------------------------------------------------------------------
-constexpr int DS_ROWS = 63;      // rows per pass (and the row of C d: 16 row groups)
+constexpr int DS_ROWS = 32;      // rows per pass: 8 row groups
 
 struct DomSeriesLayout {
-  int rs, g, sv, xm, wb, red, total;       // offsets in floats; rs: row stride of T
+  int g, part, sv, ow, slot, ids, xm, cv, red, total;   // offsets in 4-byte words
 };
-__host__ __device__ inline DomSeriesLayout dom_series_layout(int mpd, int max_obs, int max_rows,
-                                                             int splits) {
+__host__ __device__ inline DomSeriesLayout dom_series_layout(int mpd, int max_obs, int max_rows) {
   DomSeriesLayout L;
-  int rows = (max_rows + splits - 1) / splits;
-  rows = rows < DS_ROWS ? rows : DS_ROWS;
-  L.rs = 4 * ((rows + 1 + 3) / 4);
-  const int s = max_obs * mpd, t = 2 * mpd * L.rs;
-  L.g = s > t ? s : t;                     // S, then the two buffers of T
-  L.sv = L.g + mpd * mpd;
-  L.xm = L.sv + (max_obs + 3) / 4 * 4;
-  L.wb = L.xm + L.rs;
-  L.red = L.wb + mpd;
-  L.total = L.red + 36;
+  const int s = max_obs * mpd, t = 2 * mpd * DS_ROWS;
+  L.g = s > t ? s : t;                     // S, then the two buffers of T, then the sums
+  L.part = L.g + mpd * mpd;                // half products [warps][4][32][4], then X'_r wbar's parts
+  L.cv = L.part + (mpd + 31) / 32 * 512;
+  L.xm = L.cv + mpd;
+  L.sv = L.xm + DS_ROWS;
+  L.ow = L.sv + max_obs;
+  L.slot = L.ow + max_obs;
+  L.ids = L.slot + max_obs;
+  L.red = L.ids + max_rows / 2;
+  L.total = L.red + 32;
   return L;
 }
 
 template <int RPL>
-__global__ void __launch_bounds__(32 * RPL, RPL <= 13 ? 2 : 1)
+struct DomSeries {
+  static constexpr int MPD = 8 * RPL, CG = MPD / 4;
+  static constexpr int CB = (CG + 3) / 4;                 // column blocks of 4 groups
+  static constexpr int NW = CB < 2 ? 2 : (CB + 1) / 2 * 2;   // warps: 8 for MPD = 104
+  static constexpr int NT = 32 * NW;
+};
+
+// acc += rows (4 floats at x of each of n columns, stride xs float4) times the 4
+// columns at y (stride ys float4).
+__device__ __forceinline__ void tile_product(float2 (&acc)[4][2], const float4 *x, int xs,
+                                             const float4 *y, int ys, int n) {
+#pragma unroll 4
+  for (int q = 0; q < n; ++q) {
+    const float4 a = x[q * xs], b = y[q * ys];
+    const float bj[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 bb = make_float2(bj[j], bj[j]);
+      acc[j][0] = __ffma2_rn(make_float2(a.x, a.y), bb, acc[j][0]);
+      acc[j][1] = __ffma2_rn(make_float2(a.z, a.w), bb, acc[j][1]);
+    }
+  }
+}
+
+template <int RPL>
+__global__ void __launch_bounds__(DomSeries<RPL>::NT, 2)
     domain_series_kernel(const LkInst *__restrict__ insts, DomArgs a, int *__restrict__ sweep,
                          const float2 *__restrict__ cheb) {
-  constexpr int MPD = 8 * RPL, NT = 4 * MPD, CG = MPD / 4, TILES = CG * (CG + 1) / 2;
+  using C = DomSeries<RPL>;
+  constexpr int MPD = C::MPD, NT = C::NT, NW = C::NW, CG = C::CG, RS = DS_ROWS / 4;
+  constexpr int VQ = (MPD + 31) / 32;
   extern __shared__ __align__(16) float dsm[];
   lk_pdl_wait();
   const LkInst &I = insts[0];
   const int m = I.m, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int dom = blockIdx.x, splits = gridDim.y;
   const int o0 = a.obs_off[dom], np = a.obs_off[dom + 1] - o0;
-  const int n0 = a.node_off[dom], nd = 2 * (a.node_off[dom + 1] - n0);
-  const DomSeriesLayout Ly = dom_series_layout(MPD, a.max_obs, a.max_rows, splits);
-  float *S = dsm, *T = dsm, *G = dsm + Ly.g, *sv = dsm + Ly.sv, *xm = dsm + Ly.xm;
-  float *wb = dsm + Ly.wb, *red = dsm + Ly.red;
+  const int n0 = a.node_off[dom], nn = a.node_off[dom + 1] - n0, nd = 2 * nn;
+  const DomSeriesLayout Ly = dom_series_layout(MPD, a.max_obs, a.max_rows);
+  float *S = dsm, *T = dsm, *G = dsm + Ly.g, *part = dsm + Ly.part, *sv = dsm + Ly.sv;
+  float *ow = dsm + Ly.ow, *xm = dsm + Ly.xm, *cv = dsm + Ly.cv, *red = dsm + Ly.red;
+  int *slot = reinterpret_cast<int *>(dsm + Ly.slot), *ids = reinterpret_cast<int *>(dsm + Ly.ids);
   const float *Ybp = static_cast<const float *>(I.Ybp);
   const float *dp = static_cast<const float *>(I.dp);
   float *X = static_cast<float *>(I.X);
   const float alpha = float(I.alpha);
 
-  // ---- S = diag(sqrt(tau/sigma2)) Yb of the region and s, a warp per slope ----
-  for (int k = warp; k < np; k += NT / 32) {
-    const int slot = a.obs_slot[o0 + k];
-    const float sw = sqrtf(a.obs_w[o0 + k]);
-    for (int i = lane; i < MPD; i += 32)
-      S[k * MPD + i] = i < m ? sw * Ybp[(size_t)slot * m + i] : 0.f;
-    if (lane == 0) sv[k] = sw * dp[slot];
+  // ---- S = diag(sqrt(tau/sigma2)) Yb of the region and s: tables, then a warp per slope ----
+  for (int k = tid; k < np; k += NT) {
+    slot[k] = a.obs_slot[o0 + k];
+    ow[k] = sqrtf(a.obs_w[o0 + k]);
   }
+  for (int k = tid; k < nn; k += NT) ids[k] = a.node_ids[n0 + k];
   __syncthreads();
-  // ---- G = S^T S by 4 x 4 tiles of its lower triangle, c = S^T s, |G|_F, tr G ----
+#pragma unroll 2
+  for (int k = warp; k < np; k += NW) {
+    const float *row = Ybp + (size_t)slot[k] * m;
+    float v[VQ];
+#pragma unroll
+    for (int q = 0; q < VQ; ++q) v[q] = lane + 32 * q < m ? row[lane + 32 * q] : 0.f;
+#pragma unroll
+    for (int q = 0; q < VQ; ++q)
+      if (lane + 32 * q < MPD) S[k * MPD + lane + 32 * q] = ow[k] * v[q];
+  }
+  for (int k = tid; k < np; k += NT) sv[k] = ow[k] * dp[slot[k]];
+  __syncthreads();
+  // ---- G = S^T S: the 4 x 4 tiles that touch the lower triangle, in blocks of 8 row
+  // groups x 4 column groups per warp (a last block of fewer row groups takes
+  // more column groups); the others by symmetry. c = S^T s, |G|_F^2, tr G. ----
   float fro = 0.f, tr = 0.f;
-  for (int tile = tid; tile < TILES; tile += NT) {
-    int ti = (int)((sqrtf(8.f * tile + 1.f) - 1.f) * 0.5f);
-    while (ti * (ti + 1) / 2 > tile) --ti;
-    while ((ti + 1) * (ti + 2) / 2 <= tile) ++ti;
-    const int tj = tile - ti * (ti + 1) / 2;
-    const float4 *pa = reinterpret_cast<const float4 *>(S) + ti;
-    const float4 *pb = reinterpret_cast<const float4 *>(S) + tj;
+  constexpr int RBF = CG / 8, REM = CG % 8;          // full row blocks, row groups left
+  constexpr int RL = REM ? (REM <= 2 ? 2 : 4) : 8, CL = 32 / RL;
+  constexpr int FULL_TASKS = RBF * (RBF + 1);        // block rb: column blocks 0 .. 2 rb + 1
+  constexpr int REM_TASKS = REM ? ((CG + CL - 1) / CL) * ((REM + RL - 1) / RL) : 0;
+  for (int task = warp; task < FULL_TASKS + REM_TASKS; task += NW) {
+    int ti, tj;
+    if (task < FULL_TASKS) {
+      int rb = 0, cb = task;
+      while (cb > 2 * rb + 1) {
+        cb -= 2 * rb + 2;
+        ++rb;
+      }
+      ti = 8 * rb + (lane & 7);
+      tj = 4 * cb + (lane >> 3);
+    } else {
+      constexpr int CBR = (CG + CL - 1) / CL;
+      const int q = task - FULL_TASKS;
+      ti = 8 * RBF + RL * (q / CBR) + lane % RL;
+      tj = CL * (q % CBR) + lane / RL;
+    }
+    if (ti >= CG || tj > ti) continue;
     float2 acc[4][2];
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
-#pragma unroll 4
-    for (int k = 0; k < np; ++k) {
-      const float4 x = pa[k * CG], y = pb[k * CG];
-      const float yj[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float2 yy = make_float2(yj[j], yj[j]);
-        acc[j][0] = __ffma2_rn(make_float2(x.x, x.y), yy, acc[j][0]);
-        acc[j][1] = __ffma2_rn(make_float2(x.z, x.w), yy, acc[j][1]);
-      }
-    }
+    tile_product(acc, reinterpret_cast<const float4 *>(S) + ti, CG,
+                 reinterpret_cast<const float4 *>(S) + tj, CG, np);
     const float w2 = ti == tj ? 1.f : 2.f;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const float v[4] = {acc[j][0].x, acc[j][0].y, acc[j][1].x, acc[j][1].y};
+      reinterpret_cast<float4 *>(G + (4 * tj + j) * MPD)[ti] =
+          make_float4(v[0], v[1], v[2], v[3]);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        G[(4 * tj + j) * MPD + 4 * ti + i] = v[i];
         fro = fmaf(w2 * v[i], v[i], fro);
         if (ti == tj && i == j) tr += v[i];
       }
-      if (ti != tj)
-        for (int i = 0; i < 4; ++i) G[(4 * ti + i) * MPD + 4 * tj + j] = v[i];
+    }
+    if (ti != tj) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        reinterpret_cast<float4 *>(G + (4 * ti + i) * MPD)[tj] =
+            i & 1 ? make_float4(acc[0][i >> 1].y, acc[1][i >> 1].y, acc[2][i >> 1].y, acc[3][i >> 1].y)
+                  : make_float4(acc[0][i >> 1].x, acc[1][i >> 1].x, acc[2][i >> 1].x, acc[3][i >> 1].x);
     }
   }
-  if (tid < MPD) {
-    float c = 0.f;
-    for (int k = 0; k < np; ++k) c = fmaf(S[k * MPD + tid], sv[k], c);
-    wb[tid] = c;
+  for (int i = tid; i < MPD; i += NT) {
+    float c0 = 0.f, c1 = 0.f;
+    int k = 0;
+#pragma unroll 4
+    for (; k + 1 < np; k += 2) {
+      c0 = fmaf(S[k * MPD + i], sv[k], c0);
+      c1 = fmaf(S[(k + 1) * MPD + i], sv[k + 1], c1);
+    }
+    if (k < np) c0 = fmaf(S[k * MPD + i], sv[k], c0);
+    cv[i] = c0 + c1;
   }
   fro = lk_warp_sum(fro);
   tr = lk_warp_sum(tr);
@@ -464,7 +524,8 @@ __global__ void __launch_bounds__(32 * RPL, RPL <= 13 ? 2 : 1)
   }
   __syncthreads();
   fro = tr = 0.f;
-  for (int k = 0; k < NT / 32; ++k) {
+#pragma unroll
+  for (int k = 0; k < NW; ++k) {
     fro += red[k];
     tr += red[16 + k];
   }
@@ -479,155 +540,149 @@ __global__ void __launch_bounds__(32 * RPL, RPL <= 13 ? 2 : 1)
     }
   }
   if (!ok) return;
-  const int cls = lk_cheb_class(ratio);
-  const float2 *co = cheb + (size_t)cls * LK_CHEB_LD32;
+  const float2 *co = cheb + (size_t)lk_cheb_class(ratio) * LK_CHEB_LD32;
   const float2 head = __ldg(co++);
   const float scale = head.x / alpha;
   const int deg = (int)head.y;
-  const float inv_m = 1.f / float(m), rt = sqrtf(float(m - 1) / alpha);
+  const float inv_m = 1.f / float(m), rt = sqrtf(float(m - 1) / alpha), ia = 1.f / alpha;
   const int per = (nd + splits - 1) / splits;
   const int rbeg = blockIdx.y * per, rend = rbeg + per < nd ? rbeg + per : nd;
-  float creg = tid < MPD ? wb[tid] : 0.f;            // C d, kept across the passes
 
   for (int r0 = rbeg; r0 < rend; r0 += DS_ROWS) {
     const int nr = rend - r0 < DS_ROWS ? rend - r0 : DS_ROWS;   // rows of this pass
-    const int RT = (nr + 1 + 3) / 4, rs = 4 * RT;
     __syncthreads();
-    // ---- T_0: anomaly rows (a warp per row), C d, zero rows up to rs ----
-    for (int r = warp; r < nr; r += NT / 32) {
-      const int pid = a.node_ids[n0 + ((r0 + r) >> 1)];
-      const float *x = X + ((size_t)pid * 2 + ((r0 + r) & 1)) * m;
-      float v[(MPD + 31) / 32], sum = 0.f;
+    // ---- T_0: the anomaly rows (a warp per row), zero rows up to 32 ----
+    for (int r = warp; r < DS_ROWS; r += NW) {
+      float v[VQ], sum = 0.f;
+      const float *x = r < nr ? X + ((size_t)ids[(r0 + r) >> 1] * 2 + ((r0 + r) & 1)) * m : nullptr;
 #pragma unroll
-      for (int q = 0; q < (MPD + 31) / 32; ++q) {
-        const int j = lane + 32 * q;
-        v[q] = j < m ? x[j] : 0.f;
+      for (int q = 0; q < VQ; ++q) {
+        v[q] = x && lane + 32 * q < m ? x[lane + 32 * q] : 0.f;
         sum += v[q];
       }
       const float mu = lk_warp_sum(sum) * inv_m;
 #pragma unroll
-      for (int q = 0; q < (MPD + 31) / 32; ++q) {
+      for (int q = 0; q < VQ; ++q) {
         const int j = lane + 32 * q;
-        if (j < MPD) T[j * rs + r] = j < m ? v[q] - mu : 0.f;
+        if (j < MPD) T[j * DS_ROWS + r] = j < m ? v[q] - mu : 0.f;
       }
       if (lane == 0) xm[r] = mu;
     }
-    if (tid < MPD) {
-      T[tid * rs + nr] = creg;
-      for (int r = nr + 1; r < rs; ++r) T[tid * rs + r] = 0.f;
-    }
     __syncthreads();
-    // ---- the series on this thread's tile: rows 4 rg + i, columns 4 cg + j ----
-    const int rg = tid % RT, cg = tid / RT;
-    const bool work = cg < CG;
-    float2 u[4][2];
+    // ---- the series on this thread's tile: rows 4 rg + i, columns 4 cg + j. At most
+    // 16 rows: warps of 4 x 8 tiles, the second half of them on the second half
+    // of the product's columns ----
+    const bool narrow = nr <= 16 && NW >= 4;
+    constexpr int HW = (CG + 7) / 8;                 // warps of 4 x 8 tiles
+    const int half = narrow ? warp / HW : 0;
+    const int rg = narrow ? lane & 3 : lane & 7;
+    const int cg = narrow ? 8 * (warp - half * HW) + (lane >> 2) : 4 * warp + (lane >> 3);
+    const bool two = narrow && 2 * HW <= NW;
+    const bool work = cg < CG && half < (two ? 2 : 1);
+    const int qn = two ? MPD / 2 : MPD, q0 = half * qn;
+    float2 u[4][2], v[4][2];
     float f = scale, e = 1.f, o = 0.f;
-    const int ci = nr - 4 * rg;                      // 0..3: C d is this tile's row ci
+    float2 c = __ldg(co);
     for (int k = 0; k <= deg; ++k) {
-      float *cur = T + (k & 1) * MPD * rs, *nxt = T + ((k + 1) & 1) * MPD * rs;
-      const float2 c = __ldg(co + k);
-      const float2 c01 = make_float2(ci == 0 ? c.y : c.x, ci == 1 ? c.y : c.x);
-      const float2 c23 = make_float2(ci == 2 ? c.y : c.x, ci == 3 ? c.y : c.x);
-      if (work) {
-        float4 *ct = reinterpret_cast<float4 *>(cur) + cg * 4 * RT + rg;
-        float4 *nt = reinterpret_cast<float4 *>(nxt) + cg * 4 * RT + rg;
-        if (k == 0) {
+      float4 *cur = reinterpret_cast<float4 *>(T + (k & 1) * MPD * DS_ROWS);
+      float4 *nxt = reinterpret_cast<float4 *>(T + ((k + 1) & 1) * MPD * DS_ROWS);
+      const float2 cn = k < deg ? __ldg(co + k + 1) : c;   // in flight during the product
+      float2 acc[4][2];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float4 t = ct[j * RT];
-            u[j][0] = __fmul2_rn(c01, make_float2(t.x, t.y));
-            u[j][1] = __fmul2_rn(c23, make_float2(t.z, t.w));
-          }
-        } else {
+      for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
+      if (work && k < deg) {
+        tile_product(acc, cur + q0 * RS + rg, RS, reinterpret_cast<const float4 *>(G) + q0 * CG + cg,
+                     CG, qn);
+        if (half == 1) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float4 t = ct[j * RT];
-            u[j][0] = __ffma2_rn(c01, make_float2(t.x, t.y), u[j][0]);
-            u[j][1] = __ffma2_rn(c23, make_float2(t.z, t.w), u[j][1]);
-          }
+          for (int j = 0; j < 4; ++j)
+            reinterpret_cast<float4 *>(part)[((warp - HW) * 4 + j) * 32 + lane] =
+                make_float4(acc[j][0].x, acc[j][0].y, acc[j][1].x, acc[j][1].y);
         }
-        if (k < deg) {
-          float2 acc[4][2];
+      }
+      if (two) __syncthreads();
+      if (work && half == 0) {
+        const float2 ca = make_float2(c.x, c.x), cb = make_float2(c.y, c.y);
+        const float2 ff = make_float2(f, f), ee = make_float2(-e, -e), oo = make_float2(-o, -o);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
-          const float4 *pt = reinterpret_cast<const float4 *>(cur) + rg;
-          const float4 *pg = reinterpret_cast<const float4 *>(G) + cg;
-#pragma unroll 4
-          for (int q = 0; q < MPD; ++q) {
-            const float4 x = pt[q * RT], y = pg[q * CG];
-            const float yj[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const float2 yy = make_float2(yj[j], yj[j]);
-              acc[j][0] = __ffma2_rn(make_float2(x.x, x.y), yy, acc[j][0]);
-              acc[j][1] = __ffma2_rn(make_float2(x.z, x.w), yy, acc[j][1]);
-            }
+        for (int j = 0; j < 4; ++j) {
+          const float4 t4 = cur[(4 * cg + j) * RS + rg];
+          const float2 t0 = make_float2(t4.x, t4.y), t1 = make_float2(t4.z, t4.w);
+          if (k == 0) {
+            u[j][0] = __fmul2_rn(ca, t0);
+            u[j][1] = __fmul2_rn(ca, t1);
+            v[j][0] = __fmul2_rn(cb, t0);
+            v[j][1] = __fmul2_rn(cb, t1);
+          } else {
+            u[j][0] = __ffma2_rn(ca, t0, u[j][0]);
+            u[j][1] = __ffma2_rn(ca, t1, u[j][1]);
+            v[j][0] = __ffma2_rn(cb, t0, v[j][0]);
+            v[j][1] = __ffma2_rn(cb, t1, v[j][1]);
           }
-          // T_k+1 = f T_k G - e T_k - o T_k-1 (f, e, o = scale, 1, 0, then 2 scale, 2, 1)
-          const float2 ff = make_float2(f, f), ee = make_float2(-e, -e), oo = make_float2(-o, -o);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float4 t = ct[j * RT];
-            float4 pv = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (k) pv = nt[j * RT];
-            const float2 n0v = __ffma2_rn(ff, acc[j][0], __ffma2_rn(ee, make_float2(t.x, t.y),
-                                          __fmul2_rn(oo, make_float2(pv.x, pv.y))));
-            const float2 n1v = __ffma2_rn(ff, acc[j][1], __ffma2_rn(ee, make_float2(t.z, t.w),
-                                          __fmul2_rn(oo, make_float2(pv.z, pv.w))));
-            nt[j * RT] = make_float4(n0v.x, n0v.y, n1v.x, n1v.y);
+          if (k < deg) {
+            // T_k+1 = f T_k G - e T_k - o T_k-1 (f, e, o = scale, 1, 0, then 2 scale, 2, 1)
+            if (two) {
+              const float4 h = reinterpret_cast<const float4 *>(part)[(warp * 4 + j) * 32 + lane];
+              acc[j][0] = __fadd2_rn(acc[j][0], make_float2(h.x, h.y));
+              acc[j][1] = __fadd2_rn(acc[j][1], make_float2(h.z, h.w));
+            }
+            float4 p4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (k) p4 = nxt[(4 * cg + j) * RS + rg];
+            const float2 w0 = __ffma2_rn(ff, acc[j][0], __ffma2_rn(ee, t0,
+                                         __fmul2_rn(oo, make_float2(p4.x, p4.y))));
+            const float2 w1 = __ffma2_rn(ff, acc[j][1], __ffma2_rn(ee, t1,
+                                         __fmul2_rn(oo, make_float2(p4.z, p4.w))));
+            nxt[(4 * cg + j) * RS + rg] = make_float4(w0.x, w0.y, w1.x, w1.y);
           }
         }
       }
+      c = cn;
       f = 2.f * scale;
       e = 2.f;
       o = 1.f;
       __syncthreads();
     }
-    // ---- the sums, row-major in the first buffer; wbar ----
-    if (work) {
+    // ---- the sums of A^-1/2 row-major in T's place; the rows' parts of X'_r wbar ----
+    if (work && half == 0) {
+      const float4 c4 = reinterpret_cast<const float4 *>(cv)[cg];
+      float4 pw;
+      float *pp = reinterpret_cast<float *>(&pw);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int r = 4 * rg + i;
-        const float v[4] = {i & 1 ? u[0][i >> 1].y : u[0][i >> 1].x,
-                            i & 1 ? u[1][i >> 1].y : u[1][i >> 1].x,
-                            i & 1 ? u[2][i >> 1].y : u[2][i >> 1].x,
-                            i & 1 ? u[3][i >> 1].y : u[3][i >> 1].x};
-        if (r == nr)
-          for (int j = 0; j < 4; ++j) wb[4 * cg + j] = v[j] / alpha;
-        else if (r < nr)
-          reinterpret_cast<float4 *>(T + (size_t)r * MPD)[cg] =
-              make_float4(v[0], v[1], v[2], v[3]);
+        const float s0 = i & 1 ? v[0][i >> 1].y : v[0][i >> 1].x;
+        const float s1 = i & 1 ? v[1][i >> 1].y : v[1][i >> 1].x;
+        const float s2 = i & 1 ? v[2][i >> 1].y : v[2][i >> 1].x;
+        const float s3 = i & 1 ? v[3][i >> 1].y : v[3][i >> 1].x;
+        pp[i] = fmaf(s0, c4.x, s1 * c4.y) + fmaf(s2, c4.z, s3 * c4.w);
+        reinterpret_cast<float4 *>(T + (size_t)(4 * rg + i) * MPD)[cg] =
+            i & 1 ? make_float4(u[0][i >> 1].y, u[1][i >> 1].y, u[2][i >> 1].y, u[3][i >> 1].y)
+                  : make_float4(u[0][i >> 1].x, u[1][i >> 1].x, u[2][i >> 1].x, u[3][i >> 1].x);
       }
+      reinterpret_cast<float4 *>(part)[cg * RS + rg] = pw;
     }
     __syncthreads();
     // ---- apply, a warp per row: Xa_r = xbar_r + X'_r wbar + sqrt((m-1)/alpha) u_r ----
-    for (int r = warp; r < nr; r += NT / 32) {
-      const int pid = a.node_ids[n0 + ((r0 + r) >> 1)], comp = (r0 + r) & 1;
+    for (int r = warp; r < nr; r += NW) {
+      const int pid = ids[(r0 + r) >> 1], comp = (r0 + r) & 1;
       float *x = X + ((size_t)pid * 2 + comp) * m;
       const float mu0 = xm[r];
-      float v[(MPD + 31) / 32], w = 0.f;
+      const float w = lk_warp_sum(lane < CG ? part[lane * DS_ROWS + r] : 0.f) * ia;
+      float xa[VQ], sum = 0.f;
 #pragma unroll
-      for (int q = 0; q < (MPD + 31) / 32; ++q) {
+      for (int q = 0; q < VQ; ++q) {
         const int j = lane + 32 * q;
-        if (j < m) w = fmaf(x[j] - mu0, wb[j], w);
-      }
-      w = lk_warp_sum(w);
-      float sum = 0.f;
-#pragma unroll
-      for (int q = 0; q < (MPD + 31) / 32; ++q) {
-        const int j = lane + 32 * q;
-        v[q] = 0.f;
+        xa[q] = 0.f;
         if (j < m) {
-          v[q] = mu0 + w + rt * T[(size_t)r * MPD + j];
-          x[j] = v[q];
+          xa[q] = mu0 + w + rt * T[(size_t)r * MPD + j];
+          x[j] = xa[q];
         }
-        sum += v[q];
+        sum += xa[q];
       }
       const float mu = lk_warp_sum(sum) * inv_m;
       float sq = 0.f;
 #pragma unroll
-      for (int q = 0; q < (MPD + 31) / 32; ++q) {
-        const float d = lane + 32 * q < m ? v[q] - mu : 0.f;
+      for (int q = 0; q < VQ; ++q) {
+        const float d = lane + 32 * q < m ? xa[q] - mu : 0.f;
         sq = fmaf(d, d, sq);
       }
       const float sp = sqrtf(lk_warp_sum(sq) / float(m - 1));
@@ -670,18 +725,21 @@ __global__ void __launch_bounds__(LK_WARP_CTA)
 // c_d = (K b)_d, then every member of the domain's rows moves by it (and so does
 // the analysis mean): a CTA per domain, so that the product's n_dom^2 terms are
 // read by as many CTAs as there are rows (one CTA for all took 17 us at 75
-// domains and 53 us at 373; the two kernels take about 3 us each).
-__global__ void __launch_bounds__(128)
+// domains and 53 us at 373), and a warp per node whose values are in flight
+// while the product forms.
+constexpr int PA_WARPS = 16, PA_VALS = 4;            // nodes at a time; values per lane and row
+__global__ void __launch_bounds__(PA_WARPS * 32)
     piston_apply_kernel(const LkInst *__restrict__ insts, int n_dom,
                         const int *__restrict__ node_off, const int *__restrict__ node_ids,
                         const float *__restrict__ K, const float *__restrict__ bsum,
                         float *__restrict__ mean) {
-  __shared__ float part[2][4];
+  __shared__ float part[2][PA_WARPS];
   lk_pdl_wait();
   const LkInst &I = insts[0];
-  const int d = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int d = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, m = I.m;
+  const int q0 = node_off[d], q1 = node_off[d + 1];
   float c0 = 0.f, c1 = 0.f;
-  for (int e = threadIdx.x; e < n_dom; e += 128) {
+  for (int e = threadIdx.x; e < n_dom; e += PA_WARPS * 32) {
     const float k = K[(size_t)d * n_dom + e];
     const float2 b = reinterpret_cast<const float2 *>(bsum)[e];
     c0 = fmaf(k, b.x, c0);
@@ -693,20 +751,37 @@ __global__ void __launch_bounds__(128)
     part[0][warp] = c0;
     part[1][warp] = c1;
   }
+  int node = q0 + warp < q1 ? node_ids[q0 + warp] : -1;
+  float v0[PA_VALS], v1[PA_VALS];                    // m <= 128: all of the row
+  auto load = [&]() {
+    const float *x = static_cast<const float *>(I.X) + (size_t)node * 2 * m;
+#pragma unroll
+    for (int q = 0; q < PA_VALS; ++q) {
+      const bool in = node >= 0 && lane + 32 * q < m;
+      v0[q] = in ? x[lane + 32 * q] : 0.f;
+      v1[q] = in ? x[m + lane + 32 * q] : 0.f;
+    }
+  };
+  load();
   __syncthreads();
-  c0 = (part[0][0] + part[0][1]) + (part[0][2] + part[0][3]);
-  c1 = (part[1][0] + part[1][1]) + (part[1][2] + part[1][3]);
-  for (int q = node_off[d] + warp; q < node_off[d + 1]; q += 4) {
-    const int node = node_ids[q];
-    float *x = static_cast<float *>(I.X) + (size_t)node * 2 * I.m;
-    for (int j = lane; j < I.m; j += 32) {
-      x[j] += c0;
-      x[I.m + j] += c1;
-    }
-    if (lane == 0 && mean) {
-      mean[2 * node] += c0;
-      mean[2 * node + 1] += c1;
-    }
+  c0 = c1 = 0.f;
+#pragma unroll
+  for (int w = 0; w < PA_WARPS; ++w) {
+    c0 += part[0][w];
+    c1 += part[1][w];
+  }
+  for (int q = q0 + warp; node >= 0;) {
+    float *x = static_cast<float *>(I.X) + (size_t)node * 2 * m;
+#pragma unroll
+    for (int k = 0; k < PA_VALS; ++k)
+      if (lane + 32 * k < m) {
+        x[lane + 32 * k] = v0[k] + c0;
+        x[m + lane + 32 * k] = v1[k] + c1;
+      }
+    if (lane < 2 && mean) mean[2 * node + lane] += lane ? c1 : c0;
+    q += PA_WARPS;
+    node = q < q1 ? node_ids[q] : -1;
+    load();
   }
 }
 
@@ -1031,11 +1106,11 @@ template <int RPL>
 cudaError_t launch_rpl(letkf_ctx *h, DomArgs a) {
   const LkDom &D = *h->dom;
   if (D.series && h->cheb32) {
-    const size_t b = sizeof(float) * (size_t)dom_series_layout(8 * RPL, D.max_obs, 2 * D.max_nodes,
-                                                               D.splits).total;
+    const size_t b = sizeof(float) *
+                     (size_t)dom_series_layout(8 * RPL, D.max_obs, 2 * D.max_nodes).total;
     const cudaError_t e =
-        lk_launch_pdl(domain_series_kernel<RPL>, dim3(D.n_dom, D.splits), 32 * RPL, b, h->stream,
-                      h->d_inst, a, D.sweep, (const float2 *)h->cheb32);
+        lk_launch_pdl(domain_series_kernel<RPL>, dim3(D.n_dom, D.splits), DomSeries<RPL>::NT, b,
+                      h->stream, h->d_inst, a, D.sweep, (const float2 *)h->cheb32);
     if (e != cudaSuccess) return e;
     a.sweep = D.sweep;                 // the others, if any
   }
@@ -1051,8 +1126,8 @@ cudaError_t setup_rpl(const LkDom &D) {
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
   if (e != cudaSuccess || !D.series) return e;
-  const size_t b = sizeof(float) * (size_t)dom_series_layout(8 * RPL, D.max_obs, 2 * D.max_nodes,
-                                                             D.splits).total;
+  const size_t b = sizeof(float) *
+                   (size_t)dom_series_layout(8 * RPL, D.max_obs, 2 * D.max_nodes).total;
   return cudaFuncSetAttribute(domain_series_kernel<RPL>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b);
 }
@@ -1196,8 +1271,8 @@ letkf_status lk_domains_build(letkf_ctx *h, const letkf_config &c, const std::ve
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
   if (!D->global) {
     D->splits = std::max(1, std::min({sms / std::max(1, D->n_dom), 2 * D->max_nodes / 8, 4}));
-    const size_t b = sizeof(float) * (size_t)dom_series_layout(mpd, D->max_obs, 2 * D->max_nodes,
-                                                               D->splits).total;
+    const size_t b = sizeof(float) *
+                     (size_t)dom_series_layout(mpd, D->max_obs, 2 * D->max_nodes).total;
     D->series = b <= (size_t)dev_smem;
   }
   // border edges and their incidence per domain
@@ -1419,7 +1494,7 @@ cudaError_t lk_launch_domains(letkf_ctx *h, void *mean, void *spread) {
                     LK_WARP_CTA, 0, h->stream, D.n_dom, (const int2 *)D.edges,
                     (const int *)D.dedge_off, (const int *)D.dedge, (const float *)D.delta, D.bsum);
   if (e != cudaSuccess) return e;
-  return lk_launch_pdl(piston_apply_kernel, (unsigned)D.n_dom, 128, 0, h->stream, h->d_inst,
-                       D.n_dom, (const int *)D.node_off, (const int *)D.node_ids,
+  return lk_launch_pdl(piston_apply_kernel, (unsigned)D.n_dom, PA_WARPS * 32, 0, h->stream,
+                       h->d_inst, D.n_dom, (const int *)D.node_off, (const int *)D.node_ids,
                        (const float *)D.K, (const float *)D.bsum, static_cast<float *>(mean));
 }
