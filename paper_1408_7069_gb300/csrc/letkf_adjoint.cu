@@ -30,8 +30,8 @@
 // and applies the adjoint of the forecast. The result is bitwise reproducible.
 //
 // letkf_grad: forward over the frames storing the background and the analysis
-// eigenbases of the last segment and a checkpoint (ensemble, warm-start bases,
-// frame counters) at the start of every segment of ckpt_every frames; backward
+// eigenbases of the last segment and a checkpoint (ensemble, frame counters)
+// at the start of every segment of ckpt_every frames; backward
 // segment by segment, recomputing the segment's forward from its checkpoint.
 #include <math.h>
 #include <string.h>
@@ -48,10 +48,8 @@ struct LkAdjWork {
   void *basis_seg = nullptr;        // [ckpt][n_pts][mp][mp] analysis eigenbases of one segment
                                     // (FP32; FP64 on FP64 handles)
   void *ckpt_x = nullptr;           // [n_seg][state]
-  float *ckpt_basis = nullptr;      // [n_seg][n_pts][mp][mp] warm-start bases at segment start
   long long *ckpt_frame = nullptr;  // [n_seg][2] frame counters at segment start
   void *fin_x = nullptr;            // state after the forward pass
-  float *fin_basis = nullptr;
   long long *fin_frame = nullptr;
   double *resvar = nullptr;         // [frames]
   double *lam[2] = {nullptr, nullptr};  // [n_pts][2][m] adjoint of the analysis ensemble
@@ -710,8 +708,8 @@ cudaError_t launch_nodes(letkf_ctx *h, LkAdjWork *W, const void *bk, const LkAdj
 void free_work(LkAdjWork *W) {
   if (!W) return;
   if (W->graph) cudaGraphExecDestroy(W->graph);
-  void *bufs[] = {W->x_seg,    W->basis_seg, W->ckpt_x,   W->ckpt_basis, W->ckpt_frame, W->fin_x,
-                  W->fin_basis, W->fin_frame, W->resvar,   W->lam[0],     W->lam[1],     W->xp_bar,
+  void *bufs[] = {W->x_seg,    W->basis_seg, W->ckpt_x,   W->ckpt_frame, W->fin_x,
+                  W->fin_frame, W->resvar,   W->lam[0],     W->lam[1],     W->xp_bar,
                   W->xbar_bar,  W->ybw,       W->dbw,      W->ybar,       W->dbar,       W->theta,
                   W->acc,       W->dtap,      W->queue,    W->queue_len};
   for (void *p : bufs)
@@ -735,7 +733,6 @@ letkf_status ensure_work(letkf_ctx *h, int frames, int ckpt) {
   W->n_seg = (frames + ckpt - 1) / ckpt;
   const LkInst &I = h->inst[0];
   const size_t st = (size_t)h->state_total * h->rsz;
-  const size_t bas = (size_t)I.n_pts * I.mp * I.mp * sizeof(float);
   const size_t bas_seg = (size_t)I.n_pts * I.mp * I.mp * (h->precision == 1 ? 8 : 4);
   const size_t ns = (size_t)I.n_pts * 2 * I.m * sizeof(double);
   const size_t wc = (size_t)I.w * I.w;
@@ -743,10 +740,8 @@ letkf_status ensure_work(letkf_ctx *h, int frames, int ckpt) {
   cudaError_t e = walloc(&W->x_seg, (size_t)ckpt * st);
   if (e == cudaSuccess) e = walloc(&W->basis_seg, (size_t)ckpt * bas_seg);
   if (e == cudaSuccess) e = walloc(&W->ckpt_x, (size_t)W->n_seg * st);
-  if (e == cudaSuccess) e = walloc(&W->ckpt_basis, (size_t)W->n_seg * bas);
   if (e == cudaSuccess) e = walloc(&W->ckpt_frame, (size_t)W->n_seg * 2 * sizeof(long long));
   if (e == cudaSuccess) e = walloc(&W->fin_x, st);
-  if (e == cudaSuccess) e = walloc(&W->fin_basis, bas);
   if (e == cudaSuccess) e = walloc(&W->fin_frame, 2 * sizeof(long long));
   if (e == cudaSuccess) e = walloc(&W->resvar, (size_t)frames * sizeof(double));
   if (e == cudaSuccess) e = walloc(&W->lam[0], ns);
@@ -777,28 +772,19 @@ letkf_status ensure_work(letkf_ctx *h, int frames, int ckpt) {
   return LETKF_OK;
 }
 
-// Copies between the handle's state (ensemble, warm-start bases, frame
-// counters) and a saved copy.
-cudaError_t save_state(letkf_ctx *h, void *x, float *basis, long long *frame) {
-  const LkInst &I = h->inst[0];
+// Copies between the handle's state (ensemble, frame counters) and a saved copy.
+cudaError_t save_state(letkf_ctx *h, void *x, long long *frame) {
   cudaError_t e = cudaMemcpyAsync(x, h->X, h->state_total * h->rsz, cudaMemcpyDeviceToDevice,
                                   h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(basis, h->basis, (size_t)I.n_pts * I.mp * I.mp * sizeof(float),
-                        cudaMemcpyDeviceToDevice, h->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(frame, h->frame, 2 * sizeof(long long), cudaMemcpyDeviceToDevice,
                         h->stream);
   return e;
 }
 
-cudaError_t load_state(letkf_ctx *h, const void *x, const float *basis, const long long *frame) {
-  const LkInst &I = h->inst[0];
+cudaError_t load_state(letkf_ctx *h, const void *x, const long long *frame) {
   cudaError_t e = cudaMemcpyAsync(h->X, x, h->state_total * h->rsz, cudaMemcpyDeviceToDevice,
                                   h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(h->basis, basis, (size_t)I.n_pts * I.mp * I.mp * sizeof(float),
-                        cudaMemcpyDeviceToDevice, h->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->frame, frame, 2 * sizeof(long long), cudaMemcpyDeviceToDevice,
                         h->stream);
@@ -893,11 +879,11 @@ letkf_status enqueue_grad(letkf_ctx *h, int frames, const void *y_seq, const voi
     const int seg = k / C, slot = k % C;
     if (slot == 0)
       LK_ACUDA(h, save_state(h, static_cast<char *>(W->ckpt_x) + (size_t)seg * st,
-                             W->ckpt_basis + (size_t)seg * bas, W->ckpt_frame + 2 * seg));
+                             W->ckpt_frame + 2 * seg));
     LK_ACUDA(h, forward_frame(h, y_seq, truth_seq, W->resvar, xs + (size_t)slot * st,
                               bs + (size_t)slot * bseg, true));
   }
-  LK_ACUDA(h, save_state(h, W->fin_x, W->fin_basis, W->fin_frame));
+  LK_ACUDA(h, save_state(h, W->fin_x, W->fin_frame));
   // ---- backward ----
   LK_ACUDA(h, cudaMemsetAsync(W->lam[0], 0, (size_t)I.n_pts * 2 * I.m * sizeof(double),
                               h->stream));
@@ -907,7 +893,7 @@ letkf_status enqueue_grad(letkf_ctx *h, int frames, const void *y_seq, const voi
     const int s = seg * C, e = (s + C < frames) ? s + C : frames;
     if (seg != W->n_seg - 1) {   // the last segment is still in the segment buffers
       LK_ACUDA(h, load_state(h, static_cast<char *>(W->ckpt_x) + (size_t)seg * st,
-                             W->ckpt_basis + (size_t)seg * bas, W->ckpt_frame + 2 * seg));
+                             W->ckpt_frame + 2 * seg));
       for (int k = s; k < e; ++k)
         LK_ACUDA(h, forward_frame(h, y_seq, nullptr, nullptr, xs + (size_t)(k - s) * st,
                                   bs + (size_t)(k - s) * bseg, k + 1 < e));
@@ -920,7 +906,7 @@ letkf_status enqueue_grad(letkf_ctx *h, int frames, const void *y_seq, const voi
       cur ^= 1;
     }
   }
-  LK_ACUDA(h, load_state(h, W->fin_x, W->fin_basis, W->fin_frame));
+  LK_ACUDA(h, load_state(h, W->fin_x, W->fin_frame));
   return LETKF_OK;
 }
 

@@ -595,9 +595,9 @@ letkf_status letkf_set_state(letkf_t h, const void *X_dev) {
   if (!h) return fail(nullptr, LETKF_ERR_ARG, "handle is NULL");
   if (!X_dev) return fail(h, LETKF_ERR_ARG, "X_dev is NULL");
   DeviceGuard dg(h->device);
+  // the stored eigenbases stay: every analysis writes those it reads
   LK_CUDA(h, cudaMemcpyAsync(h->X, X_dev, h->state_total * h->rsz, cudaMemcpyDeviceToDevice,
                              h->stream));
-  LK_CUDA(h, lk_launch_basis_reset(h));
   return LETKF_OK;
 }
 
@@ -1070,6 +1070,9 @@ letkf_status letkf_set_row_split(letkf_t h, int32_t width_class, int32_t split) 
   LK_CUDA(h, cudaStreamSynchronize(h->stream));
   if (h->row_split[width_class] == split) return LETKF_OK;
   h->row_split[width_class] = split;
+  // the split form stores bases of all 32 columns, the whole-column form of at most
+  // 24 members only those of 24: the others have to be the identity's again
+  LK_CUDA(h, lk_launch_basis_reset(h));
   return rebuild_tiles(h, width_class);    // class 1 groups its tiles by width only unsplit
 }
 

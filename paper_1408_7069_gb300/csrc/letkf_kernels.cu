@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(LK_WARP_CTA)
                blockIdx.x - res_blocks - noise_blocks);
 }
 
-// Every node's warm-start eigenbasis back to the identity (grid.y = instance).
+// Every node's stored eigenbasis back to the identity (grid.y = instance).
 __global__ void basis_reset_kernel(const LkInst *__restrict__ insts) {
   const LkInst &I = insts[blockIdx.y];
   const long long mp = I.mp, n = (long long)I.n_pts * mp * mp;
