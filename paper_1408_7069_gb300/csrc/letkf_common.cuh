@@ -203,7 +203,7 @@ cudaError_t lk_launch_residual(letkf_ctx *h, const void *truth, double *resvar,
 // The same on another stream of the handle's device.
 cudaError_t lk_launch_residual_on(letkf_ctx *h, cudaStream_t stream, const void *truth,
                                   double *resvar, const long long *run_idx, double *piston);
-cudaError_t lk_launch_basis_reset(letkf_ctx *h);   // warm-start eigenbases -> identity
+cudaError_t lk_launch_basis_reset(letkf_ctx *h);   // stored eigenbases -> identity
 // Deformable mirror (letkf_dm.cu): cor = N u_{k-1} on `stream` (before a
 // residual), u_k = P pmean (after a forecast), and the simulated measurement
 // y_k = D1 (phi_prev - N u_{k-2}) + w_k of a closed loop (phi_prev NULL: zero).
@@ -271,12 +271,13 @@ int lk_domain_count(const letkf_ctx *h);
 int lk_domain_of_nodes(const letkf_ctx *h, int *node_dom_host);
 int lk_domain_obs_counts(const letkf_ctx *h, int *obs_host);
 cudaError_t lk_launch_domains(letkf_ctx *h, void *mean, void *spread);
-// The global ETKF for m > 128 (letkf_global.cu): Newton-Schulz root, refined
-// mean, matrix-product apply, from the FP64 Gram partials.
+// The global ETKF for m > 64 (letkf_global.cu): Newton-Schulz root, refined
+// mean, matrix-product apply, from the Gram's partial sums. sms: CTAs of the
+// cooperative kernel (one per SM).
 int lk_ns_tile();
 size_t lk_ns_workspace_bytes(int mpt, long long n_pad);
 cudaError_t lk_launch_ns_global(letkf_ctx *h, const double *gpart, const double *cpart,
-                                int kchunks, int mpt, int iters, void *ws, void *mean,
+                                int kchunks, int mpt, int sms, void *ws, void *mean,
                                 void *spread);
 
 // ---------------------------------------------------------------------------

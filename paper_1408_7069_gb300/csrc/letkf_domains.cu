@@ -54,7 +54,7 @@ struct LkDom {
   float *delta = nullptr;                         // [n_pts][2] mean increments
   std::vector<double> tau;                        // host: tau of each observed slope
   // one domain covering the grid (partition 1): the global ETKF pipeline
-  int global = 0, kchunks = 0, mpt = 0;
+  int global = 0, kchunks = 0, mpt = 0, sms = 1;
   void *ns_ws = nullptr;                          // Newton-Schulz workspace (global, m > 64)
   double *gpart = nullptr;                        // [kchunks][MPD][MPD] Gram partial sums
   double *cpart = nullptr;                        // [kchunks][MPD]
@@ -788,13 +788,13 @@ __global__ void __launch_bounds__(PA_WARPS * 32)
 // ---------------------------------------------------------------------------
 // One domain covering the grid (partition 1): the global ETKF (Section 3.1.1)
 // for any number of slopes and nodes, as three kernels:
-//   gram    partial sums of A = S^T S and c = S^T s over chunks of slopes, one
-//           CTA per (upper-triangle 32 x 32 tile of A, chunk): every term
-//           w_k y_ka y_kb (w = tau / sigma2, y the grid's FP32 values) formed
-//           exactly as two floats (FMA two-products) and accumulated as an
-//           unevaluated float pair (two-sum, the error carried in the low
-//           part): about 1e-11 relative to the sum of |terms| over a chunk, on
-//           the FP32 pipe, against FP64 FMAs at 1/75 of its rate
+//   gram    partial sums of A = S^T S and c = S^T s over parts of the slopes, one
+//           CTA per (upper-triangle 32 x 32 tile of A, part): every term
+//           w_k y_ka y_kb (w = tau / sigma2, y the grid's FP32 values) summed as
+//           an unevaluated float pair: about 1e-12 relative to the sum of |terms|,
+//           on the FP32 pipe, against FP64 FMAs at 1/75 of its rate. Six
+//           operations a term (gl_add_anchored) instead of the seventeen of
+//           two-products and two-sums: m = 626, 1624 slopes 183 -> 62 us
 //   solve   one CTA: A = (m-1)/rho I + the partials (FP64), its FP32 rounding
 //           diagonalised by the domain kernel's Jacobi (A = Q Lambda Q^T), then
 //           wbar = A^-1 c by mixed-precision iterative refinement (residual
@@ -822,14 +822,32 @@ __device__ __forceinline__ void gl_add_wab(float &hi, float &lo, float w, float 
   lo = __fadd_rn(lo, __fadd_rn(e, t));
 }
 
+// hi + lo += (ah + al) b, with q = the product's multiple of ulp(sigma): sigma a
+// constant 1.5 2^M with the sum of all |q| of a chunk below 2^M, so that hi sums
+// the q exactly and lo the rests, each rest one FMA (the extraction of Rump, Ogita
+// and Oishi's accurate summation): six operations, two outputs each.
+__device__ __forceinline__ void gl_add_anchored(float2 &hi, float2 &lo, float2 ah, float2 al,
+                                                float2 b, float2 sg, float2 msg) {
+  const float2 q = __fadd2_rn(__ffma2_rn(ah, b, sg), msg);
+  const float2 mq = make_float2(-q.x, -q.y);
+  const float2 r = __ffma2_rn(al, b, __ffma2_rn(ah, b, mq));
+  hi = __fadd2_rn(hi, q);
+  lo = __fadd2_rn(lo, r);
+}
+
+// Blocks: (upper-triangle tile of A, part of the slopes); a part is a run of
+// chunks of GL_KC slopes, each summed with its own anchor and then added to
+// the running pairs by two-sums.
 __global__ void __launch_bounds__(256)
     global_gram_kernel(const LkInst *__restrict__ insts, const int *__restrict__ obs_slot,
                        const float *__restrict__ obs_w, int np, int mpt,
                        double *__restrict__ gpart, double *__restrict__ cpart) {
-  __shared__ float si[GL_KC][GL_TILE + 1], sj[GL_KC][GL_TILE + 1], sw[GL_KC], sd[GL_KC];
+  constexpr int LD = GL_TILE + 2;
+  __shared__ __align__(16) float sh[GL_KC][LD], sl[GL_KC][LD], sj[GL_KC][LD];
+  __shared__ float sw[GL_KC], sd[GL_KC], mxi[8], mxj[8];
   lk_pdl_wait();
   const LkInst &I = insts[0];
-  const int m = I.m;
+  const int m = I.m, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float *Ybp = static_cast<const float *>(I.Ybp);
   const float *dp = static_cast<const float *>(I.dp);
   // upper-triangle tile (ti <= tj) from blockIdx.x
@@ -840,46 +858,95 @@ __global__ void __launch_bounds__(256)
     ++ti;
   }
   tj += ti;
-  const int kc = blockIdx.y, k0 = kc * GL_KC;
-  const int kn = np - k0 < GL_KC ? np - k0 : GL_KC;
-  for (int e = threadIdx.x; e < GL_KC * GL_TILE; e += blockDim.x) {
-    const int k = e / GL_TILE, i = e - k * GL_TILE;
-    float a = 0.f, b = 0.f;
-    if (k < kn) {
-      const int slot = obs_slot[k0 + k];
-      const int ri = ti * GL_TILE + i, rj = tj * GL_TILE + i;
-      if (ri < m) a = Ybp[(size_t)slot * m + ri];
-      if (rj < m) b = Ybp[(size_t)slot * m + rj];
-    }
-    si[k][i] = a;
-    sj[k][i] = b;
-  }
-  for (int k = threadIdx.x; k < GL_KC; k += blockDim.x) {
-    sw[k] = k < kn ? obs_w[k0 + k] : 0.f;
-    sd[k] = k < kn ? dp[obs_slot[k0 + k]] : 0.f;
-  }
-  __syncthreads();
+  const int chunks = (np + GL_KC - 1) / GL_KC;
+  const int per = (chunks + gridDim.y - 1) / gridDim.y;
+  const int c0 = blockIdx.y * per, c1 = c0 + per < chunks ? c0 + per : chunks;
   const int a0 = (threadIdx.x / 16) * 2, b0 = (threadIdx.x % 16) * 2;
-  float hi[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, lo[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-  for (int k = 0; k < GL_KC; ++k) {
-    const float w = sw[k];
+  float2 H[2], L[2];
+  H[0] = H[1] = L[0] = L[1] = make_float2(0.f, 0.f);
+  float ch = 0.f, cl = 0.f;
+  for (int kc = c0; kc < c1; ++kc) {
+    const int k0 = kc * GL_KC, kn = np - k0 < GL_KC ? np - k0 : GL_KC;
+    __syncthreads();
+    float ma = 0.f, mb = 0.f;
+    for (int k = warp; k < GL_KC; k += 8) {          // a warp per slope, a lane per column
+      float x = 0.f, y = 0.f, w = 0.f;
+      if (k < kn) {
+        const int slot = obs_slot[k0 + k];
+        const int ri = ti * GL_TILE + lane, rj = tj * GL_TILE + lane;
+        w = obs_w[k0 + k];
+        if (ri < m) x = Ybp[(size_t)slot * m + ri];
+        if (rj < m) y = Ybp[(size_t)slot * m + rj];
+        if (lane == 0) sd[k] = dp[slot];
+      } else if (lane == 0) {
+        sd[k] = 0.f;
+      }
+      const float p = __fmul_rn(w, x);               // w x as a pair
+      sh[k][lane] = p;
+      sl[k][lane] = fmaf(w, x, -p);
+      sj[k][lane] = y;
+      if (lane == 0) sw[k] = w;
+      ma = fmaxf(ma, fabsf(p));
+      mb = fmaxf(mb, fabsf(y));
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      ma = fmaxf(ma, __shfl_xor_sync(FULL, ma, o));
+      mb = fmaxf(mb, __shfl_xor_sync(FULL, mb, o));
+    }
+    if (lane == 0) {
+      mxi[warp] = ma;
+      mxj[warp] = mb;
+    }
+    __syncthreads();
+    ma = mxi[0];
+    mb = mxj[0];
 #pragma unroll
-    for (int x = 0; x < 2; ++x)
+    for (int w = 1; w < 8; ++w) {
+      ma = fmaxf(ma, mxi[w]);
+      mb = fmaxf(mb, mxj[w]);
+    }
+    // |q| < 2^(ilogb ma + ilogb mb + 2), GL_KC = 64 of them
+    int M = -100;
+    if (ma > 0.f && mb > 0.f) {
+      M = ilogbf(ma) + ilogbf(mb) + 9;
+      M = M < -100 ? -100 : M;
+    }
+    const float s = scalbnf(1.5f, M);                // infinite with infinite slopes: NaN follows
+    const float2 sg = make_float2(s, s), msg = make_float2(-s, -s);
+    float2 hi[2], lo[2];
+    hi[0] = hi[1] = lo[0] = lo[1] = make_float2(0.f, 0.f);
+#pragma unroll 8
+    for (int k = 0; k < GL_KC; ++k) {
+      const float2 x = *reinterpret_cast<const float2 *>(&sh[k][a0]);
+      const float2 xl = *reinterpret_cast<const float2 *>(&sl[k][a0]);
+      const float2 y = *reinterpret_cast<const float2 *>(&sj[k][b0]);
+      gl_add_anchored(hi[0], lo[0], make_float2(x.x, x.x), make_float2(xl.x, xl.x), y, sg, msg);
+      gl_add_anchored(hi[1], lo[1], make_float2(x.y, x.y), make_float2(xl.y, xl.y), y, sg, msg);
+    }
 #pragma unroll
-      for (int y = 0; y < 2; ++y) gl_add_wab(hi[x][y], lo[x][y], w, si[k][a0 + x], sj[k][b0 + y]);
+    for (int i = 0; i < 2; ++i) {                    // (H, L) += (hi, lo), Knuth's two-sum
+      const float2 t = __fadd2_rn(H[i], hi[i]);
+      const float2 mH = make_float2(-H[i].x, -H[i].y);
+      const float2 bb = __fadd2_rn(t, mH);
+      const float2 d = __fadd2_rn(t, make_float2(-bb.x, -bb.y));
+      const float2 e = __fadd2_rn(__fadd2_rn(H[i], make_float2(-d.x, -d.y)),
+                                  __fadd2_rn(hi[i], make_float2(-bb.x, -bb.y)));
+      H[i] = t;
+      L[i] = __fadd2_rn(L[i], __fadd2_rn(e, lo[i]));
+    }
+    if (ti == tj && threadIdx.x < GL_TILE)
+      for (int k = 0; k < GL_KC; ++k)                // w x d, x = the column's own slope
+        gl_add_wab(ch, cl, sw[k], sj[k][threadIdx.x], sd[k]);
   }
-  double *out = gpart + (size_t)kc * mpt * mpt;
+  double *out = gpart + (size_t)blockIdx.y * mpt * mpt;
 #pragma unroll
-  for (int x = 0; x < 2; ++x)
-#pragma unroll
-    for (int y = 0; y < 2; ++y)
-      out[(size_t)(ti * GL_TILE + a0 + x) * mpt + tj * GL_TILE + b0 + y] =
-          (double)hi[x][y] + (double)lo[x][y];
-  if (ti == tj && threadIdx.x < GL_TILE) {
-    float ch = 0.f, cl = 0.f;
-    for (int k = 0; k < GL_KC; ++k) gl_add_wab(ch, cl, sw[k], si[k][threadIdx.x], sd[k]);
-    cpart[(size_t)kc * mpt + ti * GL_TILE + threadIdx.x] = (double)ch + (double)cl;
+  for (int x = 0; x < 2; ++x) {
+    double *o = out + (size_t)(ti * GL_TILE + a0 + x) * mpt + tj * GL_TILE + b0;
+    o[0] = (double)H[x].x + (double)L[x].x;
+    o[1] = (double)H[x].y + (double)L[x].y;
   }
+  if (ti == tj && threadIdx.x < GL_TILE)
+    cpart[(size_t)blockIdx.y * mpt + ti * GL_TILE + threadIdx.x] = (double)ch + (double)cl;
 }
 
 // Shared memory of the solve kernel: A (FP64, [MPD][MPD+1]), c, wbar, r (FP64),
@@ -1138,9 +1205,6 @@ int rpl_of(int m) {
   return m <= 16 ? 2 : m <= 32 ? 4 : m <= 64 ? 8 : m <= 104 ? 13 : m <= 128 ? 16 : 0;
 }
 
-constexpr int NS_ITERS = 40;      // Newton-Schulz iterations of the wide global path (at most 64;
-                                  // converged iterations are skipped on the device)
-
 template <typename T>
 cudaError_t dup(T **dst, const std::vector<T> &src) {
   *dst = nullptr;
@@ -1368,8 +1432,10 @@ letkf_status lk_domains_build(letkf_ctx *h, const letkf_config &c, const std::ve
   if (e == cudaSuccess && D->global) {
     const int mpt = D->rpl ? gl_mpt(mpd) : mpd;
     D->mpt = mpt;
-    D->kchunks = (D->max_obs + GL_KC - 1) / GL_KC;
-    if (D->kchunks < 1) D->kchunks = 1;
+    // parts of the slopes: about four CTAs per SM over the tiles, at most a part per chunk
+    const int tiles = (mpt / GL_TILE) * (mpt / GL_TILE + 1) / 2;
+    D->kchunks = std::max(1, std::min((D->max_obs + GL_KC - 1) / GL_KC, (4 * sms + tiles - 1) / tiles));
+    D->sms = sms;
     e = cudaMalloc((void **)&D->gpart, (size_t)D->kchunks * mpt * mpt * sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(D->gpart, 0, (size_t)D->kchunks * mpt * mpt * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc((void **)&D->cpart, (size_t)D->kchunks * mpt * sizeof(double));
@@ -1379,6 +1445,7 @@ letkf_status lk_domains_build(letkf_ctx *h, const letkf_config &c, const std::ve
       const long long n_pad = ((2LL * (long long)pts.size() + lk_ns_tile() - 1) / lk_ns_tile()) *
                               lk_ns_tile();
       e = cudaMalloc(&D->ns_ws, lk_ns_workspace_bytes(mpt, n_pad));
+      if (e == cudaSuccess) e = cudaMemset(D->ns_ws, 0, lk_ns_workspace_bytes(mpt, n_pad));
     } else if (e == cudaSuccess) {
       switch (D->rpl) {
         case 2: e = setup_global_rpl<2>(*D, c.m); break;
@@ -1452,7 +1519,7 @@ cudaError_t lk_launch_domains(letkf_ctx *h, void *mean, void *spread) {
                                   h->stream, h->d_inst, (const int *)D.obs_slot,
                                   (const float *)D.obs_w, D.max_obs, D.mpt, D.gpart, D.cpart);
     if (e != cudaSuccess) return e;
-    return lk_launch_ns_global(h, D.gpart, D.cpart, D.kchunks, D.mpt, NS_ITERS, D.ns_ws, mean,
+    return lk_launch_ns_global(h, D.gpart, D.cpart, D.kchunks, D.mpt, D.sms, D.ns_ws, mean,
                                spread);
   }
   if (D.global) {

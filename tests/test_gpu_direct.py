@@ -253,3 +253,67 @@ def test_domains_of_both_kinds_in_one_frame():
     assert 1 < st[1] <= 20 and st[2] > dg.n_dom and 0 < st[0] < dg.n_dom
     assert rel(spread.cpu().numpy(), rspread) <= 1e-3
     assert rel(anoms(Xa), anoms(rXa)) <= 1e-3
+
+
+# ---------------------------------------------------------------------------
+# Global ETKF of more than 64 members (ns_root_kernel, global_gram_kernel)
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("scale", [0.05, 3.0], ids=["loop", "ill"])
+@pytest.mark.parametrize("nsub,m", [(3, 65), (10, 128), (12, 129), (9, 192), (16, 320), (12, 1000)])
+def test_global_root_matches_oracle(nsub, m, scale):
+    """Padding edges, fewer and more slopes than members, kappa from about 2 to 1e5, two
+    analyses in a row (the grid barrier's counters): the tolerances of the global tests."""
+    from oracle import letkf_domains as LD
+    mask = synth.pupil_subap_mask(nsub, 0.0)
+    dg = LD.build_domains(mask, 1, 3, 0, 0.0)
+    rng = np.random.default_rng(nsub + m)
+    n = dg.geom.n_pts
+    X = (3 * rng.standard_normal((n, 2, 1)) + scale * rng.standard_normal((n, 2, m)))
+    X = X.astype(np.float32)
+    f = Letkf(mask, m=m, window=3, taper=0, rho=RHO, sigma2=SIGMA2, partition=1)
+    f.set_state(torch.from_numpy(X).cuda())
+    for _ in range(2):
+        Xb = f.get_state().cpu().numpy().astype(np.float64)
+        y = rng.standard_normal(dg.geom.p).astype(np.float32)
+        rXa, rmean, rspread = LD.analysis_domains(dg, Xb, y.astype(np.float64), SIGMA2, RHO)
+        mean, spread = f.analyze(torch.from_numpy(y).cuda())
+        f.sync()
+        Xa = f.get_state().cpu().numpy()
+        assert rel(mean.cpu().numpy(), rmean) <= 1e-4
+        assert rel(spread.cpu().numpy(), rspread) <= 1e-3
+        assert rel(anoms(Xa), anoms(rXa)) <= 1e-3
+    f.close()
+
+
+def test_global_root_in_graphs_and_nonfinite_slopes():
+    from paper_1408_7069_gb300.letkf import LetkfError
+    mask = synth.pupil_subap_mask(8, 0.0)
+    rng = np.random.default_rng(5)
+    m, frames = 80, 3
+    bank = rng.standard_normal((2, 32, 32)).astype(np.float32)
+    f = Letkf(mask, m=m, window=3, taper=0, rho=RHO, sigma2=SIGMA2, partition=1, a_ar1=0.999,
+              noise_std=0.05, seed=3, bank=bank)
+    X = torch.from_numpy(rng.standard_normal((f.n_pts, 2, m)).astype(np.float32) * 0.1).cuda()
+    y = torch.from_numpy(rng.standard_normal((frames, f.p)).astype(np.float32)).cuda()
+    out = []
+    for mode in ("plain", "graph", "one"):
+        f.set_state(X)
+        f.set_frame(0)
+        if mode == "one":
+            f.run_graph(frames, y)
+        else:
+            f.run(frames, y, use_graph=mode == "graph")
+        f.sync()
+        out.append(f.get_state().cpu().numpy())
+    assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
+    bad = y[0].clone()
+    bad[7] = float("nan")
+    f.analyze(bad)
+    with pytest.raises(LetkfError, match="LETKF_ERR_NONFINITE"):
+        f.sync()
+    f.set_state(X)
+    f.set_frame(0)
+    f.run(frames, y)
+    f.sync()
+    assert np.array_equal(f.get_state().cpu().numpy(), out[0])
+    f.close()
