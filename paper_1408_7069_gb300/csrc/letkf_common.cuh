@@ -275,6 +275,7 @@ cudaError_t lk_launch_domains(letkf_ctx *h, void *mean, void *spread);
 // mean, matrix-product apply, from the Gram's partial sums. sms: CTAs of the
 // cooperative kernel (one per SM).
 int lk_ns_tile();
+cudaError_t lk_ns_setup();
 size_t lk_ns_workspace_bytes(int mpt, long long n_pad);
 cudaError_t lk_launch_ns_global(letkf_ctx *h, const double *gpart, const double *cpart,
                                 int kchunks, int mpt, int sms, void *ws, void *mean,

@@ -1432,9 +1432,9 @@ letkf_status lk_domains_build(letkf_ctx *h, const letkf_config &c, const std::ve
   if (e == cudaSuccess && D->global) {
     const int mpt = D->rpl ? gl_mpt(mpd) : mpd;
     D->mpt = mpt;
-    // parts of the slopes: about four CTAs per SM over the tiles, at most a part per chunk
+    // parts of the slopes: about four CTAs per SM over the tiles, at least two chunks each
     const int tiles = (mpt / GL_TILE) * (mpt / GL_TILE + 1) / 2;
-    D->kchunks = std::max(1, std::min((D->max_obs + GL_KC - 1) / GL_KC, (4 * sms + tiles - 1) / tiles));
+    D->kchunks = std::max(1, std::min((D->max_obs + 2 * GL_KC - 1) / (2 * GL_KC), (4 * sms + tiles - 1) / tiles));
     D->sms = sms;
     e = cudaMalloc((void **)&D->gpart, (size_t)D->kchunks * mpt * mpt * sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(D->gpart, 0, (size_t)D->kchunks * mpt * mpt * sizeof(double));
@@ -1446,6 +1446,7 @@ letkf_status lk_domains_build(letkf_ctx *h, const letkf_config &c, const std::ve
                               lk_ns_tile();
       e = cudaMalloc(&D->ns_ws, lk_ns_workspace_bytes(mpt, n_pad));
       if (e == cudaSuccess) e = cudaMemset(D->ns_ws, 0, lk_ns_workspace_bytes(mpt, n_pad));
+      if (e == cudaSuccess) e = lk_ns_setup();
     } else if (e == cudaSuccess) {
       switch (D->rpl) {
         case 2: e = setup_global_rpl<2>(*D, c.m); break;

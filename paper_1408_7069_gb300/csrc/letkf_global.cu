@@ -24,8 +24,7 @@
 //
 // Everything between the Gram and the apply is one cooperative kernel: a grid
 // barrier (about 1 us) per dependent stage instead of a launch, and the
-// number of iterations is the device's own. The products run in 32 x 32 tiles of
-// 512 threads, eight groups of 64 splitting the K dimension. (Forming only the upper triangle
+// number of iterations is the device's own. (Forming only the upper triangle
 // of these products of commuting symmetric matrices and mirroring it would
 // halve the flops, but it breaks the coupling of the iteration: in FP32 at the
 // prior draw's kappa ~ 1.5e5, m = 200, the symmetrised iteration overflows
@@ -55,7 +54,9 @@ constexpr int NS_TILE = 64, NS_KT = 32, NS_THREADS = 256;
 // threads hold 8 x 4 of these tiles (a 16-byte shared load costs 2 clocks per eight
 // different addresses: 4 clocks of loads against 4.3 of packed FMAs). The next 32-deep slice of A and B is
 // loaded into registers (float4) while the current one, in shared memory (A
-// transposed), is multiplied.
+// transposed), is multiplied; a slice's sum is formed by itself and then added (the
+// rounding of K / 32 + 32 additions instead of K: the analysis rows are much
+// smaller than the terms).
 __global__ void __launch_bounds__(NS_THREADS)
     ns_gemm_kernel(int K, const float *__restrict__ A, int lda, const float *__restrict__ B,
                    int ldb, float *__restrict__ C, int ldc) {
@@ -88,7 +89,7 @@ __global__ void __launch_bounds__(NS_THREADS)
       *reinterpret_cast<float4 *>(&Bs[bk + 16 * q][bc]) = rb[q];
     }
   };
-  float2 acc[4][2];
+  float2 acc[4][2];                                  // sums over the slices so far
 #pragma unroll
   for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
   load(0);
@@ -96,10 +97,18 @@ __global__ void __launch_bounds__(NS_THREADS)
     store();
     __syncthreads();
     if (k0 + NS_KT < K) load(k0 + NS_KT);
+    float2 part[4][2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) part[j][0] = part[j][1] = make_float2(0.f, 0.f);
 #pragma unroll 8
     for (int k = 0; k < NS_KT; ++k)
-      tile4x4(acc, *reinterpret_cast<const float4 *>(&As[k][tr * 4]),
+      tile4x4(part, *reinterpret_cast<const float4 *>(&As[k][tr * 4]),
               *reinterpret_cast<const float4 *>(&Bs[k][tc * 4]));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      acc[j][0] = __fadd2_rn(acc[j][0], part[j][0]);
+      acc[j][1] = __fadd2_rn(acc[j][1], part[j][1]);
+    }
     __syncthreads();
   }
 #pragma unroll
@@ -113,8 +122,13 @@ __global__ void __launch_bounds__(NS_THREADS)
 // ---------------------------------------------------------------------------
 // The cooperative kernel
 // ---------------------------------------------------------------------------
-constexpr int NR_THREADS = 512, NR_TILE = 32, NR_KT = 16, NR_SPLIT = 8, NR_LD = NR_TILE + 4;
-constexpr int NR_MAX_ITERS = 24, NR_REFINE = 4;
+constexpr int NR_THREADS = 512, NR_WARPS = NR_THREADS / 32;
+constexpr int NR_TILE = 32, NR_KT = 8, NR_STAGES = 3, NR_LD = NR_TILE + 4;
+constexpr int NR_SLICE = 2 * NR_KT * NR_TILE;          // floats of a slice of A and B
+constexpr int NR_PART = NR_TILE * NR_LD;               // floats of a warp's partial tile
+// shared floats: every warp's slices, every warp's partial tile, the tile's sums
+constexpr int NR_SMEM = NR_WARPS * (NR_STAGES * NR_SLICE + NR_PART) + NR_TILE * (NR_TILE + 1);
+constexpr int NR_MAX_ITERS = 24, NR_REFINE = 8;
 constexpr unsigned NR_SPIN = 1u << 21;       // polls of a grid barrier (about a second)
 
 struct NsArgs {
@@ -122,8 +136,9 @@ struct NsArgs {
   const double *gpart, *cpart;
   int kchunks, mpt;
   long long n_pad;
-  double *A64, *c64, *w64, *part, *scale;    // part [grid]: sums of squares
-  float *Y, *Z, *T, *U, *rv, *vv, *Xp, *xm;
+  double *A64, *c64, *w64, *part;            // part [grid]: sums of squares
+  float *mat;                                // eight [n][n] matrices: Y, Y^T, Z, Z^T, twice
+  float *T, *TT, *rv, *vv, *Xp, *xm;
   unsigned *sync;                            // [0] arrivals, [1] departures, [2] abort,
                                              // [4 ..] per refinement: max |r| (float bits)
   int *counters;
@@ -158,81 +173,122 @@ __device__ __forceinline__ bool grid_sync(const NsArgs &a, unsigned &target, uns
   return *flag != 0;
 }
 
-// Output tile (row0, col0) of A B, n x n: this thread's two outputs, row tid / 16,
-// columns 2 (tid % 16). Group q of 64 threads takes the 16-deep slices q, q + 8, ...;
-// the groups' partial tiles are added in group order through shared memory.
-// The operands were written by other CTAs during this launch: L2 loads only.
-__device__ __forceinline__ float2 ns_tile(int n, const float *A, const float *B, int row0,
-                                          int col0, float *smem) {
-  const int tid = threadIdx.x, q = tid >> 6, lt = tid & 63, lane = tid & 31;
-  float(*as)[NR_LD] = reinterpret_cast<float(*)[NR_LD]>(smem + q * 2 * NR_KT * NR_LD);
-  float(*bs)[NR_LD] = as + NR_KT;
-  // thread tiles 8 x 8 of 4 x 4; a warp 8 x 4 of them
-  const int tr = lane & 7, tc = (lt >> 5) * 4 + (lane >> 3);
-  const int ar = lt >> 2, ak = (lt & 3) * 4, bk = lt >> 3, bc = (lt & 7) * 4;
-  float4 ra[2], rb[2];
-  auto load = [&](int k0) {
+// ---------------------------------------------------------------------------
+// A 32 x 32 output tile of A B, n x n, by one CTA: warp w takes the 8-deep slices
+// w, w + 16, ... of the product on its own, three slices in flight (cp.async: the
+// operands were written by other CTAs of this launch, so they come from L2), each
+// lane 4 x 8 outputs (6 clocks of shared loads against 8.6 of packed FMAs per
+// column and SM); the 16 partial tiles are added in warp order. No CTA barrier
+// inside the product, and the next tile's first slices are on their way during the sums. A is read from its
+// transpose, which every product of the iteration writes beside itself, so
+// that both operands' slices are rows of 32.
+// ---------------------------------------------------------------------------
+struct NsTile {
+  const float *AT, *B;
+  int row0, col0;
+};
+
+__device__ __forceinline__ void ns_load(const NsTile &t, int n, int s, float *st) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      ra[j] = __ldcg(reinterpret_cast<const float4 *>(A + (size_t)(row0 + ar + 16 * j) * n + k0 + ak));
-      rb[j] = __ldcg(reinterpret_cast<const float4 *>(B + (size_t)(k0 + bk + 8 * j) * n + col0 + bc));
-    }
-  };
-  float2 acc[4][2];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
-  const int nk = n / NR_KT, steps = (nk + NR_SPLIT - 1) / NR_SPLIT;
-  load(q * NR_KT);                                   // n >= 128: every group has a slice
-  for (int s = 0; s < steps; ++s) {
-    const int kt = q + NR_SPLIT * s;
-    const bool valid = kt < nk;
-    if (valid) {
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int r = ar + 16 * j;
-        as[ak + 0][r] = ra[j].x;
-        as[ak + 1][r] = ra[j].y;
-        as[ak + 2][r] = ra[j].z;
-        as[ak + 3][r] = ra[j].w;
-        *reinterpret_cast<float4 *>(&bs[bk + 8 * j][bc]) = rb[j];
-      }
-    }
-    __syncthreads();
-    if (kt + NR_SPLIT < nk) load((kt + NR_SPLIT) * NR_KT);
-    if (valid) {
-#pragma unroll
-      for (int k = 0; k < NR_KT; ++k)
-        tile4x4(acc, *reinterpret_cast<const float4 *>(&as[k][tr * 4]),
-                *reinterpret_cast<const float4 *>(&bs[k][tc * 4]));
-    }
-    __syncthreads();
+  for (int j = 0; j < 2; ++j) {
+    const int e = lane + 32 * j, k = e >> 3, c = (e & 7) * 4;
+    const float *ga = t.AT + (size_t)(s * NR_KT + k) * n + t.row0 + c;
+    const float *gb = t.B + (size_t)(s * NR_KT + k) * n + t.col0 + c;
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(st + k * NR_TILE + c);
+    const unsigned sb = (unsigned)__cvta_generic_to_shared(st + (NR_KT + k) * NR_TILE + c);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(ga) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sb), "l"(gb) : "memory");
   }
-  float(*ps)[NR_LD] = reinterpret_cast<float(*)[NR_LD]>(smem + q * NR_TILE * NR_LD);
+}
+
+// The first NR_STAGES - 1 slices of the warp (a group is committed for each, empty
+// beyond the last slice).
+__device__ __forceinline__ void ns_begin(const NsTile &t, int n, float *st) {
+  const int warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < NR_STAGES - 1; ++q) {
+    const int s = warp + NR_WARPS * q;
+    if (s * NR_KT < n) ns_load(t, n, s, st + q * NR_SLICE);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+}
+
+// The product of a tile begun by ns_begin; `next` (if any) is begun before the
+// sums. Returns this thread's two outputs: row tid / 16, columns 2 (tid % 16).
+__device__ __forceinline__ float2 ns_tile(const NsTile &t, const NsTile *next, int n, float *smem) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float *st = smem + warp * NR_STAGES * NR_SLICE;
+  float *part = smem + NR_WARPS * NR_STAGES * NR_SLICE;
+  const int tr = lane & 7, tc = lane >> 3;
+  float2 acc[2][4][2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[h][j][0] = acc[h][j][1] = make_float2(0.f, 0.f);
+  int buf = 0, ld = NR_STAGES - 1;
+  for (int s = warp; s * NR_KT < n; s += NR_WARPS) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(NR_STAGES - 2) : "memory");
+    __syncwarp();
+    const int sn = s + NR_WARPS * (NR_STAGES - 1);
+    if (sn * NR_KT < n) ns_load(t, n, sn, st + ld * NR_SLICE);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const float4 *as = reinterpret_cast<const float4 *>(st + buf * NR_SLICE) + tr;
+    const float4 *bs = reinterpret_cast<const float4 *>(st + buf * NR_SLICE + NR_KT * NR_TILE) + 2 * tc;
+#pragma unroll
+    for (int k = 0; k < NR_KT; ++k) {
+      const float4 a = as[k * (NR_TILE / 4)];
+      tile4x4(acc[0], a, bs[k * (NR_TILE / 4)]);
+      tile4x4(acc[1], a, bs[k * (NR_TILE / 4) + 1]);
+    }
+    buf = buf + 1 == NR_STAGES ? 0 : buf + 1;
+    ld = ld + 1 == NR_STAGES ? 0 : ld + 1;
+  }
+  __syncwarp();
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if (next) ns_begin(*next, n, st);
+  float *p = part + warp * NR_PART;
 #pragma unroll
   for (int i = 0; i < 4; ++i)
-    *reinterpret_cast<float4 *>(&ps[tr * 4 + i][tc * 4]) =
-        i & 1 ? make_float4(acc[0][i >> 1].y, acc[1][i >> 1].y, acc[2][i >> 1].y, acc[3][i >> 1].y)
-              : make_float4(acc[0][i >> 1].x, acc[1][i >> 1].x, acc[2][i >> 1].x, acc[3][i >> 1].x);
-  __syncthreads();
-  float2 t = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int g = 0; g < NR_SPLIT; ++g) {
-    const float2 u = *reinterpret_cast<const float2 *>(smem + g * NR_TILE * NR_LD +
-                                                       (tid >> 4) * NR_LD + 2 * (tid & 15));
-    t = __fadd2_rn(t, u);
-  }
-  __syncthreads();                                   // the tile's memory is free again
-  return t;
+    for (int h = 0; h < 2; ++h)
+      *reinterpret_cast<float4 *>(p + (tr * 4 + i) * NR_LD + tc * 8 + 4 * h) =
+          i & 1 ? make_float4(acc[h][0][i >> 1].y, acc[h][1][i >> 1].y, acc[h][2][i >> 1].y, acc[h][3][i >> 1].y)
+                : make_float4(acc[h][0][i >> 1].x, acc[h][1][i >> 1].x, acc[h][2][i >> 1].x, acc[h][3][i >> 1].x);
+  __syncthreads();
+  float2 r = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int w = 0; w < NR_WARPS; ++w)
+    r = __fadd2_rn(r, *reinterpret_cast<const float2 *>(part + w * NR_PART + (tid >> 4) * NR_LD +
+                                                       2 * (tid & 15)));
+  return r;
+}
+
+// The tile's outputs (as ns_tile returned them, after the caller's epilogue) into C
+// and, transposed, into CT. Two barriers: the sums are read, the tile is complete.
+__device__ __forceinline__ void ns_write(float2 v, int n, int row0, int col0, float *C, float *CT,
+                                         float *smem) {
+  const int tid = threadIdx.x, r = tid >> 4, c = 2 * (tid & 15);
+  float *R = smem + NR_WARPS * (NR_STAGES * NR_SLICE + NR_PART);
+  R[r * (NR_TILE + 1) + c] = v.x;
+  R[r * (NR_TILE + 1) + c + 1] = v.y;
+  *reinterpret_cast<float2 *>(C + (size_t)(row0 + r) * n + col0 + c) = v;
+  __syncthreads();
+  *reinterpret_cast<float2 *>(CT + (size_t)(col0 + r) * n + row0 + c) =
+      make_float2(R[c * (NR_TILE + 1) + r], R[(c + 1) * (NR_TILE + 1) + r]);
+  __syncthreads();
 }
 
 __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
-  __shared__ __align__(16) float smem[2 * NR_SPLIT * NR_KT * NR_LD];
+  extern __shared__ __align__(16) float smem[];
   __shared__ double red[NR_THREADS / 32];
   __shared__ unsigned flag;
   const LkInst &I = a.insts[0];
   const int n = a.mpt, m = I.m, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int gw = blockIdx.x * (NR_THREADS / 32) + warp, nw = gridDim.x * (NR_THREADS / 32);
   const int nt = n / NR_TILE;
+  const size_t nn = (size_t)n * n;
+  float *st = smem + warp * NR_STAGES * NR_SLICE;
   unsigned target = 0;
   bool live = true;
   do {
@@ -241,6 +297,7 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
     for (int i = blockIdx.x; i < n; i += gridDim.x) {
       for (int j = i + tid; j < n; j += NR_THREADS) {
         double s = 0.0;
+#pragma unroll 4
         for (int k = 0; k < a.kchunks; ++k) s += a.gpart[((size_t)k * n + i) * n + j];
         // (m-1)/rho on the diagonal, the padding included: the padding's
         // eigenvalues then sit with the smallest real ones
@@ -249,12 +306,15 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
         if (j > i) a.A64[(size_t)j * n + i] = s;
         sq = fma(i == j ? s : 2.0 * s, s, sq);
       }
-      if (tid == 0) {
+      if (warp == 0) {
         double c = 0.0;
-        for (int k = 0; k < a.kchunks; ++k) c += a.cpart[(size_t)k * n + i];
-        a.c64[i] = c;
-        a.w64[i] = 0.0;
-        a.rv[i] = (float)c;
+        for (int k = lane; k < a.kchunks; k += 32) c += a.cpart[(size_t)k * n + i];
+        c = lk_warp_sum(c);
+        if (lane == 0) {
+          a.c64[i] = c;
+          a.w64[i] = 0.0;
+          a.rv[i] = (float)c;
+        }
       }
     }
     sq = lk_warp_sum(sq);
@@ -285,43 +345,60 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
     const double inv = 1.0 / fro;
     for (long long e = (long long)blockIdx.x * NR_THREADS + tid; e < (long long)n * n;
          e += (long long)gridDim.x * NR_THREADS) {
-      a.Y[e] = (float)(__ldcg(a.A64 + e) * inv);
-      a.Z[e] = e / n == e % n ? 1.f : 0.f;
+      const float y = (float)(__ldcg(a.A64 + e) * inv), z = e / n == e % n ? 1.f : 0.f;
+      a.mat[e] = a.mat[nn + e] = y;                  // symmetric
+      a.mat[2 * nn + e] = a.mat[3 * nn + e] = z;
     }
     if (!(live = grid_sync(a, target, &flag))) break;
     // ---- Newton-Schulz; x: the lower end of the interval ----
-    float *Y = a.Y, *Z = a.Z, *T = a.T, *U = a.U;
+    float *cur = a.mat, *nxt = a.mat + 4 * nn;         // Y, Y^T, Z, Z^T
     float x = (float)sqrt(I.alpha * inv);
-    int it = 0;
-    for (; x < 1.f - 1e-5f && it < NR_MAX_ITERS; ++it) {
+    for (int it = 0; x < 1.f - 1e-5f && it < NR_MAX_ITERS; ++it) {
       const float mu2 = 3.f / (1.f + x + x * x), mu = sqrtf(mu2);
       const float ca = 1.5f * mu, cb = 0.5f * mu * mu2;
+      auto first = [&](int t) {                      // Z Y
+        return NsTile{cur + 3 * nn, cur, t / nt * NR_TILE, t % nt * NR_TILE};
+      };
+      auto second = [&](int t) {                     // Y T, then T Z
+        const int u = t < nt * nt ? t : t - nt * nt;
+        return NsTile{t < nt * nt ? cur + nn : a.TT, t < nt * nt ? a.T : cur + 2 * nn,
+                      u / nt * NR_TILE, u % nt * NR_TILE};
+      };
+      NsTile now, next;
+      if ((int)blockIdx.x < nt * nt) {
+        now = first(blockIdx.x);
+        ns_begin(now, n, st);
+      }
       for (int t = blockIdx.x; t < nt * nt; t += gridDim.x) {
-        const int row0 = t / nt * NR_TILE, col0 = t % nt * NR_TILE;
-        const float2 p = ns_tile(n, Z, Y, row0, col0, smem);
-        const int r = row0 + (tid >> 4), c = col0 + 2 * (tid & 15);
-        *reinterpret_cast<float2 *>(T + (size_t)r * n + c) =
-            make_float2((r == c ? ca : 0.f) - cb * p.x, (r == c + 1 ? ca : 0.f) - cb * p.y);
+        const bool more = t + (int)gridDim.x < nt * nt;
+        if (more) next = first(t + gridDim.x);
+        const float2 p = ns_tile(now, more ? &next : nullptr, n, smem);
+        const int r = now.row0 + (tid >> 4), c = now.col0 + 2 * (tid & 15);
+        ns_write(make_float2((r == c ? ca : 0.f) - cb * p.x, (r == c + 1 ? ca : 0.f) - cb * p.y), n,
+                 now.row0, now.col0, a.T, a.TT, smem);
+        now = next;
       }
       if (!(live = grid_sync(a, target, &flag))) break;
-      // U = Y T; Z' = T Z into the old Y's place needs Y read out: a fourth buffer
-      float *V = a.Xp + a.n_pad * n;                 // [n][n], the product's place
+      if ((int)blockIdx.x < 2 * nt * nt) {
+        now = second(blockIdx.x);
+        ns_begin(now, n, st);
+      }
       for (int t = blockIdx.x; t < 2 * nt * nt; t += gridDim.x) {
-        const bool second = t >= nt * nt;
-        const int tt = second ? t - nt * nt : t;
-        const int row0 = tt / nt * NR_TILE, col0 = tt % nt * NR_TILE;
-        const float2 p = second ? ns_tile(n, T, Z, row0, col0, smem)
-                                : ns_tile(n, Y, T, row0, col0, smem);
-        const int r = row0 + (tid >> 4), c = col0 + 2 * (tid & 15);
-        *reinterpret_cast<float2 *>((second ? (it & 1 ? a.Z : V) : (it & 1 ? a.Y : U)) +
-                                    (size_t)r * n + c) = p;
+        const bool more = t + (int)gridDim.x < 2 * nt * nt;
+        if (more) next = second(t + gridDim.x);
+        const float2 p = ns_tile(now, more ? &next : nullptr, n, smem);
+        float *C = nxt + (t < nt * nt ? 0 : 2 * nn);
+        ns_write(p, n, now.row0, now.col0, C, C + nn, smem);
+        now = next;
       }
       if (!(live = grid_sync(a, target, &flag))) break;
-      Y = it & 1 ? a.Y : U;
-      Z = it & 1 ? a.Z : V;
+      float *swap = cur;
+      cur = nxt;
+      nxt = swap;
       const float y = mu * x;
       x = fminf(1.f, 0.5f * y * (3.f - y * y));
     }
+    const float *Y = cur, *Z = cur + 2 * nn, *ZT = cur + 3 * nn;
     if (!live) break;
     // ---- wbar = A^-1 c by refinement with A^-1 ~ Z Z / s_A; done when the residual
     // bounds the relative error of wbar by 1e-9 ----
@@ -368,14 +445,16 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
     const float f = (float)sqrt((m - 1) * inv);
     float mx = 0.f;
     for (int t = blockIdx.x; t < nt * nt; t += gridDim.x) {
-      const int row0 = t / nt * NR_TILE, col0 = t % nt * NR_TILE;
-      const float2 p = ns_tile(n, Z, Y, row0, col0, smem);
-      const int r = row0 + (tid >> 4), c = col0 + 2 * (tid & 15);
+      const NsTile now{ZT, Y, t / nt * NR_TILE, t % nt * NR_TILE};
+      ns_begin(now, n, st);
+      const float2 p = ns_tile(now, nullptr, n, smem);
+      __syncthreads();                               // the sums are read
+      const int r = now.row0 + (tid >> 4), c = now.col0 + 2 * (tid & 15);
       const float e0 = fabsf(p.x - (r == c ? 1.f : 0.f)), e1 = fabsf(p.y - (r == c + 1 ? 1.f : 0.f));
       if (!(e0 <= 1e-3f) || !(e1 <= 1e-3f)) mx = 1.f;
       const float2 z = __ldcg(reinterpret_cast<const float2 *>(Z + (size_t)r * n + c));
       const float w = (float)__ldcg(a.w64 + r);
-      *reinterpret_cast<float2 *>(T + (size_t)r * n + c) =
+      *reinterpret_cast<float2 *>(a.T + (size_t)r * n + c) =
           make_float2(r < m && c < m ? fmaf(f, z.x, w) : 0.f,
                       r < m && c + 1 < m ? fmaf(f, z.y, w) : 0.f);
     }
@@ -429,28 +508,30 @@ __global__ void __launch_bounds__(LK_WARP_CTA)
 
 int lk_ns_tile() { return NS_TILE; }
 
-// Workspace (one allocation, zeroed once): A64, c64, w64, part (FP64); Y, Z, T, U
-// (FP32 [mpt][mpt]); r, v (FP32 [mpt]); Xp (FP32 [n_pad][mpt]), then the product of
-// the same shape, which the iteration uses as its fifth matrix before; xm [n_pad];
-// the barrier words. (The FP32 part starts 256-byte aligned: the products load float4.)
+// Workspace (one allocation, zeroed once): A64, c64, w64, part (FP64); the
+// iteration's eight matrices, T and its transpose (FP32 [mpt][mpt]); r, v (FP32
+// [mpt]); Xp and the product (FP32 [n_pad][mpt]), xm [n_pad]; the barrier words.
+// (The FP32 part starts 256-byte aligned: the products load float4.)
 static size_t ns_fp64_bytes(int mpt) {
   return (((size_t)mpt * mpt * 8 + 2 * (size_t)mpt * 8 + 1024 * 8) + 255) & ~size_t(255);
 }
 
-static size_t ns_prod_rows(int mpt, long long n_pad) {
-  return n_pad > mpt ? (size_t)n_pad : (size_t)mpt;
+size_t lk_ns_workspace_bytes(int mpt, long long n_pad) {
+  const size_t f = 10 * (size_t)mpt * mpt + 2 * (size_t)mpt + 2 * (size_t)n_pad * mpt +
+                   (size_t)n_pad;
+  return ns_fp64_bytes(mpt) + f * 4 + 64 * sizeof(unsigned) + 1024;
 }
 
-size_t lk_ns_workspace_bytes(int mpt, long long n_pad) {
-  const size_t f = 4 * (size_t)mpt * mpt + 2 * (size_t)mpt + (size_t)n_pad * mpt +
-                   ns_prod_rows(mpt, n_pad) * mpt + (size_t)n_pad;
-  return ns_fp64_bytes(mpt) + f * 4 + 64 * sizeof(unsigned) + 1024;
+cudaError_t lk_ns_setup() {
+  return cudaFuncSetAttribute(ns_root_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              NR_SMEM * (int)sizeof(float));
 }
 
 cudaError_t lk_launch_ns_global(letkf_ctx *h, const double *gpart, const double *cpart,
                                 int kchunks, int mpt, int sms, void *ws, void *mean,
                                 void *spread) {
   const LkInst &I = h->inst[0];
+  const size_t nn = (size_t)mpt * mpt;
   NsArgs a;
   a.insts = h->d_inst;
   a.gpart = gpart;
@@ -460,23 +541,23 @@ cudaError_t lk_launch_ns_global(letkf_ctx *h, const double *gpart, const double 
   a.n_pad = ((2LL * I.n_pts + NS_TILE - 1) / NS_TILE) * NS_TILE;
   unsigned char *b = static_cast<unsigned char *>(ws);
   a.A64 = reinterpret_cast<double *>(b);
-  a.c64 = a.A64 + (size_t)mpt * mpt;
+  a.c64 = a.A64 + nn;
   a.w64 = a.c64 + mpt;
   a.part = a.w64 + mpt;
-  a.Y = reinterpret_cast<float *>(b + ns_fp64_bytes(mpt));
-  a.Z = a.Y + (size_t)mpt * mpt;
-  a.T = a.Z + (size_t)mpt * mpt;
-  a.U = a.T + (size_t)mpt * mpt;
-  a.rv = a.U + (size_t)mpt * mpt;
+  a.mat = reinterpret_cast<float *>(b + ns_fp64_bytes(mpt));
+  a.T = a.mat + 8 * nn;
+  a.TT = a.T + nn;
+  a.rv = a.TT + nn;
   a.vv = a.rv + mpt;
   a.Xp = a.vv + mpt;
   float *Pr = a.Xp + (size_t)a.n_pad * mpt;
-  a.xm = Pr + ns_prod_rows(mpt, a.n_pad) * mpt;
+  a.xm = Pr + (size_t)a.n_pad * mpt;
   a.sync = reinterpret_cast<unsigned *>(a.xm + a.n_pad);
   a.counters = h->counters;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(sms < 1024 ? sms : 1024));
   cfg.blockDim = dim3(NR_THREADS);
+  cfg.dynamicSmemBytes = NR_SMEM * sizeof(float);
   cfg.stream = h->stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
