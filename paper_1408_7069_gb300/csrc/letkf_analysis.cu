@@ -261,11 +261,12 @@ cudaError_t lk_setup_analysis(letkf_ctx *h) {
   bool wide = false;
   for (const LkInst &I : h->inst) wide = wide || I.mp > 32;
   if (e == cudaSuccess && wide && h->precision == 0) e = lk_setup_node64w();
+  if (e == cudaSuccess && h->precision == 0) e = lk_setup_list();
   return e;
 }
 
 cudaError_t lk_launch_analysis_class(letkf_ctx *h, int cls, void *mean, void *spread) {
-  cudaError_t e = cudaMemsetAsync(h->counters + 1, 0, 7 * sizeof(int), h->stream);
+  cudaError_t e = cudaMemsetAsync(h->counters + 1, 0, (LK_COUNTERS - 1) * sizeof(int), h->stream);
   if (e != cudaSuccess) return e;
   if (cls == 0) return launch_class<16>(h, 0, mean, spread);
   if (cls == 1) return launch_class<32>(h, 1, mean, spread);
@@ -315,7 +316,7 @@ constexpr size_t NA_OFF_TILES = al256(NA_OFF_OBS + (size_t)NA_MAX_NSUB * NA_MAX_
 constexpr size_t NA_OFF_TAPER = al256(NA_OFF_TILES + (size_t)NA_MAX_TILES * sizeof(LkTile));
 constexpr size_t NA_OFF_INST = al256(NA_OFF_TAPER + (size_t)NA_MAX_W * NA_MAX_W * sizeof(float));
 constexpr size_t NA_OFF_COUNTERS = al256(NA_OFF_INST + sizeof(LkInst));
-constexpr size_t NA_BYTES = al256(NA_OFF_COUNTERS + 8 * sizeof(int));
+constexpr size_t NA_BYTES = al256(NA_OFF_COUNTERS + LK_COUNTERS * sizeof(int));
 
 // The scratch. Host code must not pass this name to a kernel: it is a host-side
 // stand-in; the device address comes from cudaGetSymbolAddress (na_scratch_address).
@@ -533,7 +534,7 @@ extern "C" letkf_status letkf_analyze_noalloc(const letkf_config *cfg, void *X_d
       e = cudaMemcpyAsync(base + cp.off, cp.src, cp.bytes, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(base + NA_OFF_YBP, 0, cells * 2 * c.m * sizeof(float), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(base + NA_OFF_DP, 0, cells * 2 * sizeof(float), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(base + NA_OFF_COUNTERS, 0, 8 * sizeof(int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(base + NA_OFF_COUNTERS, 0, LK_COUNTERS * sizeof(int), st);
 
   // ---- observation (shared kernel) and analysis (variant kernel) ----
   letkf_ctx tmp;

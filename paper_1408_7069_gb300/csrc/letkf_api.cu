@@ -75,7 +75,7 @@ void release(letkf_ctx *h) {
                   h->pts,        h->saps,     h->bank,     h->basis,    h->basis64,  h->counters,
                   h->worklist,   h->frame,    h->partial,  h->tickets,  h->d_inst,   h->obs_items,
                   h->node_items, h->tiles[0], h->tiles[1], h->tiles[2], h->noise_pre, h->cheb32,
-                  h->cheb64};
+                  h->cheb64,   h->poles};
   for (void *p : bufs)
     if (p) cudaFree(p);
 }
@@ -340,7 +340,7 @@ letkf_status build_handle(const letkf_config *cfgs, int n, void *stream, letkf_t
   LK_TRY(dalloc(h, &h->basis, n_basis * sizeof(float)));
   if (h->precision == 1) LK_TRY(dalloc(h, &h->basis64, n_basis * sizeof(double)));
   LK_TRY(dalloc(h, &h->bank, n_bank * sizeof(float)));
-  LK_TRY(dalloc(h, &h->counters, 8 * sizeof(int)));
+  LK_TRY(dalloc(h, &h->counters, LK_COUNTERS * sizeof(int)));
   LK_TRY(dalloc(h, &h->worklist, 3 * h->n_pts_total * sizeof(int2)));
   LK_TRY(dalloc(h, &h->frame, 2 * sizeof(long long)));
   LK_TRY(dalloc(h, &h->partial, (size_t)n * LK_RES_BLOCKS * sizeof(double2)));
@@ -414,7 +414,7 @@ letkf_status build_handle(const letkf_config *cfgs, int n, void *stream, letkf_t
   cudaError_t e = cudaMemset(h->X, 0, h->state_total * h->rsz);
   if (e == cudaSuccess) e = cudaMemset(h->Ybp, 0, n_ybp * h->rsz);
   if (e == cudaSuccess) e = cudaMemset(h->dp, 0, n_dp * h->rsz);
-  if (e == cudaSuccess) e = cudaMemset(h->counters, 0, 8 * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(h->counters, 0, LK_COUNTERS * sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(h->frame, 0, 2 * sizeof(long long));
   if (e == cudaSuccess) e = cudaMemset(h->tickets, 0, (size_t)(n + 1) * sizeof(int));
   if (e != cudaSuccess) LK_TRY(cuda_fail(h, e, "cudaMemset"));

@@ -62,7 +62,37 @@ int cheb_series(double r, double tol, std::vector<double> &a, std::vector<double
   return deg < 1 ? 1 : deg;
 }
 
+// Poles s_j and weights w_j of z^-1/2 ~ sum_j w_j / (z + s_j) on [1, M]: the
+// midpoint rule in the elliptic substitution z = -sc^2(u, k'), which gives the best
+// rational approximation (Hale, Higham & Trefethen 2008, method 3): with k^2 =
+// 1 / M, u_j = (j - 1/2) K' / n, s_j = (sn / cn)^2 and w_j = 2 K' dn / (pi n cn^2) at
+// modulus k'. K' and the functions by the arithmetic-geometric mean and descending Landen
+// transformations (Abramowitz & Stegun 16.4, 17.6).
+void lk_poles(double M, int n, double2 *out) {
+  const double pi = 3.14159265358979323846, k = 1.0 / sqrt(M);
+  double a[32], c[32], b = k;
+  a[0] = 1.0;
+  c[0] = sqrt(1.0 - k * k);
+  int l = 0;
+  while (fabs(c[l]) > 1e-17 && l < 30) {
+    a[l + 1] = 0.5 * (a[l] + b);
+    c[l + 1] = 0.5 * (a[l] - b);
+    b = sqrt(a[l] * b);
+    ++l;
+  }
+  const double K = pi / (2.0 * a[l]);
+  for (int j = 0; j < n; ++j) {
+    double phi = ldexp(a[l] * (j + 0.5) * K / n, l);
+    for (int q = l; q > 0; --q) {
+      phi = 0.5 * (phi + asin(c[q] * sin(phi) / a[q]));
+    }
+    const double sn = sin(phi), cn = cos(phi), dn = sqrt(1.0 - (1.0 - k * k) * sn * sn);
+    out[j] = make_double2(sn * sn / (cn * cn), 2.0 * K * dn / (pi * n * cn * cn));
+  }
+}
+
 std::once_flag g_once;
+std::vector<double2> g_poles;
 std::vector<float2> g_table32;
 std::vector<double2> g_table64;
 
@@ -82,6 +112,8 @@ void fill_table(std::vector<V> &table, int classes, int ld, double tol, F pair) 
 void build_tables() {
   fill_table(g_table32, LK_CHEB_CLASSES32, LK_CHEB_LD32, 1e-8,
              [](double x, double y) { return make_float2((float)x, (float)y); });
+  g_poles.assign(16, make_double2(0.0, 0.0));
+  lk_poles(LK_TRI_MAX, 15, g_poles.data());
   fill_table(g_table64, LK_CHEB_CLASSES64, LK_CHEB_LD64, 1e-17,
              [](double x, double y) { return make_double2(x, y); });
 }
@@ -98,7 +130,10 @@ cudaError_t upload_table(V **dst, const std::vector<V> &table) {
 
 cudaError_t lk_setup_cheb(letkf_ctx *h) {
   std::call_once(g_once, build_tables);
-  if (h->precision == 0) return upload_table(&h->cheb32, g_table32);
+  if (h->precision == 0) {
+    const cudaError_t e = upload_table(&h->cheb32, g_table32);
+    return e == cudaSuccess ? upload_table(&h->poles, g_poles) : e;
+  }
   const cudaError_t e = upload_table(&h->cheb64, g_table64);
   return e == cudaSuccess ? lk_setup_series64(h) : e;
 }

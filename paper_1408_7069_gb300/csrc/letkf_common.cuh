@@ -46,6 +46,17 @@ constexpr double LK_CHEB_R0 = 0.25, LK_CHEB_STEP = 1.25;
 constexpr int LK_CHEB_CLASSES32 = 33, LK_CHEB_LD32 = 192;
 constexpr float LK_CHEB_MAX32 = 300.f;        // below the last class's 315.5
 constexpr float LK_CHEB_MAXD = 100.f;         // multi-actuator domains: 94 products
+// kappa_hat to which ill-conditioned nodes of FP32 handles take the float-pair
+// tridiagonal form (letkf_tri.cuh) instead of FP64 sweeps: the error of its rational
+// approximation (15 poles) is 4e-9 there, and 7e-8, more than the sweeps', at 1e6.
+// An entry of its list holds the instance in its low LK_TRI_INST bits and above it the
+// exponent that bounds the node's kappa_hat.
+constexpr float LK_TRI_MAX = 1e5f;
+constexpr int LK_TRI_INST = 26;
+// Ints of a handle's counters: [0] status bits, [1] FP64 nodes, [2] max and [3]
+// total sweeps, [4..6] lengths of the classes' sweep lists, [7..8] of the
+// tridiagonal lists of classes 0 and 1 (which fill the same worklists from their ends).
+constexpr int LK_COUNTERS = 16, LK_TRI_LIST = 3;   // a class's tridiagonal count sits 3 above its sweep count
 // The FP64 table, truncated below FP64 rounding: classes up to 42.4, 128 terms.
 // Beyond, the products outnumber an eigensolve's work on the 0.5 FMA per clock
 // that an SM sub-partition issues.
@@ -110,6 +121,7 @@ struct letkf_ctx {
   int max_sweeps = 20;
   float2 *cheb32 = nullptr;         // FP32 Chebyshev table; NULL: every node by Jacobi sweeps
   double2 *cheb64 = nullptr;        // the FP64 one (FP64 handles)
+  double2 *poles = nullptr;         // [16] poles and weights of A^-1/2 (FP32 handles)
   int keep_basis = 0;               // store every node's eigenbasis (reverse mode needs it)
 
   int n_inst = 0;
@@ -135,7 +147,7 @@ struct letkf_ctx {
   int2 *pts = nullptr, *saps = nullptr;
   float *bank = nullptr, *basis = nullptr;
   double *basis64 = nullptr;        // FP64 handles: the FP64 eigenbases the reverse mode records
-  int *counters = nullptr;          // [0] status bits, [1] FP64 queue length, [2] max sweeps, [3] total sweeps
+  int *counters = nullptr;          // [LK_COUNTERS]
   int2 *worklist = nullptr;         // [n_pts_total] (inst, point) queued for FP64
   long long *frame = nullptr;       // [0] forecast counter, [1] frame index within letkf_run
   double2 *partial = nullptr;       // [n_inst][LK_RES_BLOCKS] residual partial sums
@@ -243,8 +255,10 @@ cudaError_t lk_setup_cheb(letkf_ctx *h);
 // the pair kernel queued in class cls of an FP32 handle.
 cudaError_t lk_launch_node64(letkf_ctx *h, int cls, void *mean, void *spread);
 cudaError_t lk_launch_list64(letkf_ctx *h, int cls, void *mean, void *spread);
-// Shared-memory limit of the wide class's FP64 list kernel (MP = 48 / 64 queue).
+// Shared-memory limit of the wide class's FP64 list kernel (MP = 48 / 64 queue), and
+// of the list kernel with the tridiagonal form.
 cudaError_t lk_setup_node64w();
+cudaError_t lk_setup_list();
 
 // Whether width class cls of the handle can take tile shape `shape`: FP32
 // handles need whole warps of nodes and, in class 2 (one node per warp), at

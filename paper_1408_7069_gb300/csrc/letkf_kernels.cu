@@ -21,8 +21,8 @@ __device__ __forceinline__ void obs_block(const LkInst *__restrict__ insts,
                                           int *__restrict__ counters, int bx) {
   lk_pdl_wait();   // no early trigger: an analysis launched early would have its CTAs
                    // packed onto the SMs this kernel still occupies
-  // the analysis that follows counts into counters[1..7] (queue lengths, sweeps)
-  if (bx == 0 && threadIdx.x < 7) counters[1 + threadIdx.x] = 0;
+  // the analysis that follows counts into the other counters (list lengths, sweeps)
+  if (bx == 0 && threadIdx.x < LK_COUNTERS - 1) counters[1 + threadIdx.x] = 0;
   const long long wi = ((long long)bx * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (wi >= n_items) return;
@@ -322,7 +322,7 @@ int warp_blocks(long long warps) {
 
 cudaError_t lk_launch_obs(letkf_ctx *h, const void *y, const long long *run_idx) {
   // no subaperture, no kernel: the analysis counters are zeroed here instead
-  if (h->sap_total == 0) return cudaMemsetAsync(h->counters + 1, 0, 7 * sizeof(int), h->stream);
+  if (h->sap_total == 0) return cudaMemsetAsync(h->counters + 1, 0, (LK_COUNTERS - 1) * sizeof(int), h->stream);
   const int blocks = warp_blocks(h->sap_total);
   if (h->precision == 1)
     return lk_launch_pdl(obs_kernel<double>, blocks, LK_WARP_CTA, 0, h->stream, h->d_inst,

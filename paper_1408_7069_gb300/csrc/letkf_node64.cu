@@ -27,7 +27,7 @@
 
 #include <atomic>
 
-#include "letkf_device.cuh"
+#include "letkf_tri.cuh"
 
 namespace {
 
@@ -435,6 +435,55 @@ __global__ void __launch_bounds__(N64_THREADS)
   }
 }
 
+// FP32 handles with the series: the nodes queued for the tridiagonal form (a warp
+// each, from the end of the worklist), then those of the sweeps (a CTA each), a
+// fixed grid of CTAs walking both.
+template <int MP>
+__global__ void __launch_bounds__(N64_THREADS, 3)
+    tri_list_kernel(const LkInst *__restrict__ insts, const int2 *__restrict__ worklist, int n_list,
+                    const int *__restrict__ queue_len,
+                    const double2 *__restrict__ poles, float *__restrict__ mean,
+                    float *__restrict__ spread, double tol, int max_sweeps,
+                    int *__restrict__ counters) {
+  extern __shared__ __align__(16) double n64_smem[];
+  lk_pdl_wait();   // no early trigger (long kernel): dependents launch as its CTAs exit
+  const int qn = queue_len[0], tn = queue_len[LK_TRI_LIST];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float *ws = reinterpret_cast<float *>(n64_smem) + warp * TriCfg<MP>::TOTAL;
+  for (int idx = blockIdx.x * (N64_THREADS / 32) + warp; idx < tn;
+       idx += gridDim.x * (N64_THREADS / 32)) {
+    const int2 it = worklist[n_list - 1 - idx];
+    const LkInst &I = insts[it.x & ((1 << LK_TRI_INST) - 1)];
+    const float *taper = static_cast<const float *>(I.taper);
+    unsigned short *cell = reinterpret_cast<unsigned short *>(ws + TriCfg<MP>::V);
+    const int wc = I.w * I.w;
+    int ncell = 0;
+    for (int e0 = 0; e0 < wc; e0 += 32) {            // the taper's support
+      const int e = e0 + lane, er = e / I.w;
+      const bool in = e < wc && taper[e] != 0.f;
+      const unsigned b = __ballot_sync(FULL, in);
+      if (in) cell[ncell + __popc(b & ((1u << lane) - 1u))] = er << 8 | (e - er * I.w);
+      ncell += __popc(b);
+    }
+    __syncwarp();
+    const long long row = I.node_off + it.y;
+    // |G| <= tr G < alpha kappa_hat (one more for the FP32 sum that kappa_hat is)
+    const int EG = ilogbf((float)I.alpha) + 2 + (it.x >> LK_TRI_INST);
+    tri_node<MP>(I, it.y, ncell, EG, poles, mean ? mean + 2 * row : nullptr,
+                 spread ? spread + 2 * row : nullptr, counters, ws);
+  }
+  __syncthreads();
+  for (int idx = blockIdx.x; idx < qn; idx += gridDim.x) {
+    const int2 it = worklist[idx];
+    const LkInst &I = insts[it.x];
+    const long long row = I.node_off + it.y;
+    node64<MP, float, true>(I, it.y, mean ? mean + 2 * row : nullptr,
+                            spread ? spread + 2 * row : nullptr, tol, LK_WARM_STOP64, max_sweeps,
+                            counters, n64_smem);
+    __syncthreads();                       // shared memory is reused by the next node
+  }
+}
+
 // ---------------------------------------------------------------------------
 // FP64 fallback of the wide class (m = 33..64): the nodes the pair kernel
 // queued for MP = 48 and MP = 64, both padded to 64 columns here (identity on
@@ -781,6 +830,14 @@ cudaError_t launch_node64(letkf_ctx *h, void *mean, void *spread) {
                        h->tol64, h->max_sweeps, h->counters, h->keep_basis);
 }
 
+// Dynamic shared memory of tri_list_kernel: four warps' workspaces, or one node64.
+template <int MP>
+constexpr size_t tri_list_smem() {
+  const size_t t = (size_t)(N64_THREADS / 32) * TriCfg<MP>::TOTAL * sizeof(float);
+  const size_t n = n64_smem_doubles<MP>() * sizeof(double);
+  return t > n ? t : n;
+}
+
 template <int MP>
 cudaError_t launch_list64(letkf_ctx *h, int cls, void *mean, void *spread) {
   long long n = 0;
@@ -792,6 +849,13 @@ cudaError_t launch_list64(letkf_ctx *h, int cls, void *mean, void *spread) {
   const size_t smem = n64_smem_doubles<MP>() * sizeof(double);
   const int2 *list = h->worklist + (size_t)cls * h->n_pts_total;
   const int *len = h->counters + 4 + cls;
+  if (h->precision == 0 && h->cheb32 && h->row_split[cls] == 1) {
+    const long long full = 3LL * n64_sm_count(h->device);    // three CTAs per SM (shared memory)
+    return lk_launch_pdl(tri_list_kernel<MP>, (unsigned)(n < full ? n : full), N64_THREADS,
+                         tri_list_smem<MP>(), h->stream, h->d_inst, list, (int)h->n_pts_total, len,
+                         (const double2 *)h->poles, (float *)mean, (float *)spread, h->tol64,
+                         h->max_sweeps, h->counters);
+  }
   if (h->precision == 1)
     return lk_launch_pdl(node64_list_kernel<MP, double>, blocks, N64_THREADS, smem, h->stream,
                          h->d_inst, list, len, (double *)mean, (double *)spread, h->tol64,
@@ -819,6 +883,14 @@ cudaError_t launch_list64w(letkf_ctx *h, void *mean, void *spread) {
 cudaError_t lk_setup_node64w() {
   return cudaFuncSetAttribute(node64w_list_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)(n64w_smem_doubles() * sizeof(double)));
+}
+
+cudaError_t lk_setup_list() {
+  const cudaError_t e = cudaFuncSetAttribute(
+      tri_list_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_list_smem<16>());
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(tri_list_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)tri_list_smem<32>());
 }
 
 cudaError_t lk_launch_node64(letkf_ctx *h, int cls, void *mean, void *spread) {

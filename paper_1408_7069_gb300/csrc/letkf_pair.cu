@@ -33,11 +33,11 @@
 // warp.
 //
 // kappa_hat = 1 + rho tr(G)/(m-1) bounds the condition number before the
-// eigensolve; nodes above the threshold still take this FP32 sweep, store
-// their eigenbasis (the start of their FP64 sweep) and leave X alone: they are
-// queued, per width class, for the FP64 list kernels of letkf_node64.cu
-// (MP = 16 and 32: node64_list_kernel; MP = 48 and 64 share one queue:
-// node64w_list_kernel), which write them.
+// solve; nodes above the threshold leave X alone and are queued, per width class,
+// for the list kernels of letkf_node64.cu (MP = 16 and 32: tri_list_kernel, the
+// float-pair tridiagonal form of letkf_tri.cuh; MP = 48 and 64 share one queue:
+// node64w_list_kernel), which write them. Those of the FP64 sweeps take the FP32
+// eigensolve here and store their eigenbasis, the start of their FP64 sweep.
 #include <math.h>
 #include <stdint.h>
 
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
                          float *__restrict__ mean, float *__restrict__ spread, float tol,
                          float stop, int max_sweeps, float kappa_thr, int *__restrict__ counters,
                          int *__restrict__ queue, int2 *__restrict__ worklist, int keep_basis,
-                         const float2 *__restrict__ cheb) {
+                         const float2 *__restrict__ cheb, int n_list) {
   lk_pdl_wait();   // no early trigger: the next kernel launches as this one's CTAs exit
   LK_PHASE_STAMP(ph0);
   using C = PairCfg<MP>;
@@ -473,15 +473,22 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
   if (!live) diag = cd0 = cd1 = 0.f;
   const float alpha = float(I.alpha);
   const bool active = pid >= 0;
-  // kappa_hat above the threshold: the node's mean solve needs the FP64 Gram.
-  // It still takes this FP32 eigensolve, whose basis is stored as the start of
-  // the FP64 list kernel's sweep; X is left alone and the node is queued.
-  bool queued = false;
+  // kappa_hat above the threshold: the node's mean solve needs more than an FP32
+  // Gram. X is left alone and the node is queued: for the float-pair tridiagonal
+  // form (which starts from nothing) at the end of the worklist, or beyond its
+  // range, without the series, and for the wide classes at its front for the FP64
+  // sweeps, which start from the basis of the FP32 eigensolve below.
+  bool queued = false, tri = false;
   if (!BASIS && queue) {
-    const float trg = group_sum<GL>(diag);
-    if (active && 1.f + trg / alpha > kappa_thr) {
+    const float kappa = 1.f + group_sum<GL>(diag) / alpha;
+    if (active && kappa > kappa_thr) {
+      tri = MP <= 32 && cheb && kappa <= LK_TRI_MAX && alpha > 0.01f && alpha < 1e6f;
       if (li == 0) {
-        worklist[atomicAdd(queue, 1)] = make_int2(tl.inst, pid);
+        if (tri)
+          worklist[n_list - 1 - atomicAdd(queue + LK_TRI_LIST, 1)] =
+              make_int2(tl.inst | (ilogbf(kappa) + 1) << LK_TRI_INST, pid);
+        else
+          worklist[atomicAdd(queue, 1)] = make_int2(tl.inst, pid);
         atomicAdd(&counters[1], 1);
       }
       queued = true;
@@ -545,7 +552,7 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
     }
   }
   // ---- Jacobi: every other node, and all of them when their bases are kept ----
-  const bool sweep_node = active && (!direct || keep_basis);
+  const bool sweep_node = active && ((!direct && !tri) || keep_basis);
   if (__any_sync(FULL, sweep_node)) {
   // (m-1)/rho on the diagonal, 1 on the padding; inactive nodes and idle lanes
   // get identity columns
@@ -1086,7 +1093,7 @@ cudaError_t launch_shape(letkf_ctx *h, const LkTile *tiles, int n_tiles, float *
                          TI * TJ * 32 / PairCfg<MP>::NPW, need, h->stream, h->d_inst, tiles, mean,
                          spread, (float)h->tol32, (float)h->stop32, h->max_sweeps, kthr,
                          h->counters, queue, worklist, h->keep_basis,
-                         (const float2 *)h->cheb32);
+                         (const float2 *)h->cheb32, (int)h->n_pts_total);
   }
 }
 
@@ -1128,7 +1135,7 @@ cudaError_t launch_basis_shape(letkf_ctx *h, int cls) {
                          h->tiles[cls], (float *)nullptr, (float *)nullptr, (float)h->tol32,
                          (float)h->stop32, h->max_sweeps, 0.f, h->counters,
                          lk_series64(h) ? h->counters + 4 + cls : (int *)nullptr,
-                         (int2 *)nullptr, 1, (const float2 *)nullptr);
+                         (int2 *)nullptr, 1, (const float2 *)nullptr, 0);
   }
 }
 

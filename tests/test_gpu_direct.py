@@ -317,3 +317,34 @@ def test_global_root_in_graphs_and_nonfinite_slopes():
     f.sync()
     assert np.array_equal(f.get_state().cpu().numpy(), out[0])
     f.close()
+
+
+# ---------------------------------------------------------------------------
+# Ill-conditioned node problems of FP32 handles (letkf_tri.cuh)
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("scale", [2.0, 12.0, 60.0], ids=["3e2", "1e4", "3e5"])
+@pytest.mark.parametrize("nsub,m,window,taper",
+                         [(3, 2, 3, 1), (4, 3, 3, 1), (5, 15, 3, 1), (5, 16, 5, 0), (6, 17, 5, 1),
+                          (6, 24, 9, 0), (6, 25, 5, 1), (6, 31, 4, 1), (7, 32, 7, 1),
+                          (12, 32, 13, 0)])
+def test_ill_conditioned_nodes_match_oracle(nsub, m, window, taper, scale):
+    """Every queued node by the float-pair tridiagonal form, or by the FP64 sweeps beyond its
+    range: more slopes than one staged chunk, windows with fewer slopes than members, both
+    column widths. kappa_hat above 1 sends every node there. Tolerances: the FP32 ones on
+    the mean; the storage's rounding, 4 units of 2^-24 of the background's size, plus 1e-6
+    of the analysis anomalies (kappa to 1e5 times 2^-42 and the poles' 4e-9) on the members."""
+    mask, geom, X, y, khat = problem(nsub, m, window, taper, scale)
+    ref = oracle.analysis(geom, X.astype(np.float64), y.astype(np.float64), SIGMA2, RHO)
+    Xa, mean, spread, st = analyse(mask, X, y, m, window, taper, fp64_kappa=1.0000001)
+    assert st[0] == geom.n_pts
+    if khat.max() < 9.9e4:
+        assert st[1:] == (1, geom.n_pts)
+
+    def rms(v):
+        return float(np.sqrt(np.mean(np.square(v))))
+    if khat.max() < 9.9e4:
+        assert rel(mean, ref[1]) <= 1e-4
+        assert rel(spread, ref[2]) <= 1e-3
+        assert rel(anoms(Xa), anoms(ref[0])) <= 1e-3
+    Xj, mj, sj, _ = analyse(mask, X, y, m, window, taper, fp64_kappa=1.0000001, max_sweeps=30)
+    assert rms(Xa - Xj) <= 4 * 2.0 ** -24 * rms(X) + 1e-6 * rms(anoms(ref[0]))
