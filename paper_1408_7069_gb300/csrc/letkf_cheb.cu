@@ -94,7 +94,7 @@ void lk_poles(double M, int n, double2 *out) {
 std::once_flag g_once;
 std::vector<double2> g_poles;
 std::vector<float2> g_table32;
-std::vector<double2> g_table64;
+std::vector<float4> g_table64;   // pairs of floats: a_k high, low, b_k high, low
 
 template <typename V, typename F>
 void fill_table(std::vector<V> &table, int classes, int ld, double tol, F pair) {
@@ -115,7 +115,10 @@ void build_tables() {
   g_poles.assign(16, make_double2(0.0, 0.0));
   lk_poles(LK_TRI_MAX, 15, g_poles.data());
   fill_table(g_table64, LK_CHEB_CLASSES64, LK_CHEB_LD64, 1e-17,
-             [](double x, double y) { return make_double2(x, y); });
+             [](double x, double y) {
+               const float xh = (float)x, yh = (float)y;
+               return make_float4(xh, (float)(x - xh), yh, (float)(y - yh));
+             });
 }
 
 template <typename V>

@@ -120,7 +120,7 @@ struct letkf_ctx {
   double stop32 = 1e-3;             // FP32 Jacobi stops after a sweep with all cosines <= this
   int max_sweeps = 20;
   float2 *cheb32 = nullptr;         // FP32 Chebyshev table; NULL: every node by Jacobi sweeps
-  double2 *cheb64 = nullptr;        // the FP64 one (FP64 handles)
+  float4 *cheb64 = nullptr;         // the FP64 one (FP64 handles), in pairs of floats
   double2 *poles = nullptr;         // [16] poles and weights of A^-1/2 (FP32 handles)
   int keep_basis = 0;               // store every node's eigenbasis (reverse mode needs it)
 

@@ -140,6 +140,36 @@ def test_fp64_series_matches_oracle(nsub, m, window, taper, scale):
     assert rel(anoms(Xa), anoms(ref[0])) <= 1e-8
 
 
+@pytest.mark.parametrize("m", [7, 24])
+def test_fp64_series_keeps_the_range_of_fp64(m):
+    """The node's values are scaled by powers of two before anything is rounded: an
+    analysis in other units, by 2^+-200, has the same digits. And rows and innovations
+    of nothing but zeros."""
+    mask, geom, X, y, _ = problem(4, m, 3, 1, 0.06)
+    X, y = X.astype(np.float64), y.astype(np.float64)
+
+    def run(X, y, s):
+        f = Letkf(mask, m=m, window=3, taper=1, rho=RHO, sigma2=SIGMA2 * s * s, precision=1)
+        f.set_state(torch.from_numpy(X * s).cuda())
+        mean, spread = f.analyze(torch.from_numpy(y * s).cuda())
+        out = f.get_state().cpu().numpy(), mean.cpu().numpy(), spread.cpu().numpy()
+        f.sync()
+        assert f.stats()[1] == 1
+        f.close()
+        return [v / s for v in out]
+    a = run(X, y, 1.0)
+    for s in (2.0 ** 200, 2.0 ** -200):
+        assert all(np.array_equal(u, v) for u, v in zip(a, run(X, y, s)))
+    flat = np.repeat(X.mean(-1, keepdims=True), m, -1)
+    Xz = X.copy()
+    Xz[:, 1] = flat[:, 1]                        # no anomalies in the second row
+    for Xb, yb in ((Xz, y), (flat, y), (X, np.zeros_like(y)), (flat, np.zeros_like(y))):
+        ref = oracle.analysis(geom, Xb, yb, SIGMA2, RHO)
+        got = run(Xb, yb, 1.0)
+        for u, v in zip(got, ref):
+            assert np.abs(u - v).max() <= 1e-9 * np.abs(X).max()
+
+
 def test_fp64_series_and_eigensolve_nodes_in_one_frame():
     mask, geom, X, y, khat = problem(8, 20, 5, 1, 0.3, ramp=(0.02, 10.0))
     X, y = X.astype(np.float64), y.astype(np.float64)
