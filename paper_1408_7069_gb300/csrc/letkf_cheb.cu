@@ -96,6 +96,20 @@ std::vector<double2> g_poles;
 std::vector<float2> g_table32;
 std::vector<float4> g_table64;   // pairs of floats: a_k high, low, b_k high, low
 
+// The term up to which a series needs more than floats: from low + 1 on the coefficients,
+// weighted by the growth of the recurrences' rounding (the number of steps since), add up
+// to less than 2^-27, and so the rounding of these terms in FP32 to less than 2^-51.
+int last_in_pairs(const std::vector<double> &a, const std::vector<double> &b, int deg) {
+  double s = 0.0, tail = 0.0;
+  int k = deg;
+  for (; k > 1; --k) {
+    s += fmax(fabs(a[k]), fabs(b[k]));
+    tail += s;
+    if (tail > ldexp(1.0, -27)) break;
+  }
+  return k;
+}
+
 template <typename V, typename F>
 void fill_table(std::vector<V> &table, int classes, int ld, double tol, F pair) {
   table.assign((size_t)classes * ld, pair(0.0, 0.0));
@@ -105,6 +119,7 @@ void fill_table(std::vector<V> &table, int classes, int ld, double tol, F pair) 
     const int deg = cheb_series(r, tol, a, b);
     V *row = table.data() + (size_t)c * ld;
     row[0] = pair(2.0 / r, deg);
+    if constexpr (sizeof(V) == sizeof(float4)) row[0].w = (float)last_in_pairs(a, b, deg);
     for (int k = 0; k <= deg && k + 1 < ld; ++k) row[k + 1] = pair(a[k], b[k]);
   }
 }

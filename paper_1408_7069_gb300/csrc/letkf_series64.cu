@@ -14,7 +14,9 @@
 // fast; the condition of I + G, at most 1 + ratio, is small here. Values enter by their
 // bits, scaled by powers of two to about 1: slopes by sqrt(tau / (sigma2 alpha)) and the
 // innovations, rows and adjoints by their largest exponent, so the range is FP64's. Means
-// and what is added to them stay FP64.
+// and what is added to them stay FP64. About the second half of a series, whose
+// coefficients are below 2^-27 (letkf_cheb.cu: last_in_pairs), runs in floats: its
+// rounding is then below that of the pairs.
 //
 // One CTA per node, MPD = m padded to 8, 16, 24 or 32 columns: thread
 // (row, vector, segment) holds a segment of L columns of its row of 2 X in
@@ -23,9 +25,11 @@
 // through shared memory, double-buffered: one barrier per product. Segment 0
 // sums the series of A^-1/2, segment 1 that of A^-1, in one instruction.
 // Measured on one GB300: 8 x 8, m = 10, 16 frames: eigensolve 1971 us, series in FP64 557,
-// in pairs 424; gradient of ten frames at 16 m, m = 24: 32.7, 7.2, 3.1 ms. Errors against
-// FP64 of four seeds: the eigensolve's X 1e-15 to 5e-15 and gradient 8e-15 to 1.4e-12, the
-// pairs' 9e-16 to 4e-15 and 8e-15 to 1.1e-13.
+// in pairs 424, with the second half in floats 400; gradient of ten frames at 16 m,
+// m = 24: 32.7, 7.2, 3.1, 2.45 ms (861 nodes: forward 116, 40, 33 us, adjoint 449, 161, 104,
+// 45% of the issue slots used: bound by the products' chains at 12 to 15 warps per SM).
+// Errors against FP64 of four seeds: the eigensolve's X 1e-15 to 5e-15 and gradient 8e-15 to
+// 1.4e-12, now 9e-16 to 4e-15 and 1e-14 to 4e-14.
 #include <math.h>
 
 #include "letkf_df.cuh"
@@ -102,58 +106,57 @@ struct Alpha64 {
   }
 };
 
-// The cells of the node's window inside the taper's support: offsets ds * w + dt with the
-// exponent of sqrt(tau / (sigma2 alpha)) above them, and that root's significand (0 where
-// rounding left tau below it at the edge of the support). redi: their number, and the largest
-// exponent of the innovations times the root. One barrier.
+// The cells of the node's window inside the taper's support, by one warp: row and column (5
+// bits each: windows are up to 31 wide) with the exponent of sqrt(tau / (sigma2 alpha)) above
+// them, and that root's significand (0 where rounding left tau below it at the edge of the
+// support). redi: their number, and the largest exponent of the innovations times the root.
 constexpr int CELL_BITS = 10, CELL_EXP = 1 << 14;
+__device__ __forceinline__ int cell_row(int c) { return (c >> 5) & 31; }
+__device__ __forceinline__ int cell_col(int c) { return c & 31; }
 constexpr int NO_EXP = -4000;                        // the exponent of nothing but zeros
 template <int MPD>
-__device__ __forceinline__ int support(const LkInst &I, int2 ij, const Smem64<MPD> &sm) {
+__device__ __forceinline__ void support(const LkInst &I, int2 ij, const Smem64<MPD> &sm) {
   const double *__restrict__ taper = static_cast<const double *>(I.taper);
   const double2 *__restrict__ dp = static_cast<const double2 *>(I.dp);
   const int w = I.w, wc = w * w;
-  if (threadIdx.x < 32) {
-    const int ea = exponent64(I.alpha);
-    const Df ia = df_rcp(df_split(I.alpha, -ea));
-    int n = 0, ed = NO_EXP;
-    constexpr int U = 3;                             // loads in flight
-    for (int e0 = 0; e0 < wc; e0 += 32 * U) {
-      double t[U];
-      double2 d[U];
+  const int ea = exponent64(I.alpha), lane = threadIdx.x & 31;
+  const Df ia = df_rcp(df_split(I.alpha, -ea));
+  int n = 0, ed = NO_EXP;
+  constexpr int U = 3;                               // loads in flight
+  for (int e0 = 0; e0 < wc; e0 += 32 * U) {
+    double t[U];
+    double2 d[U];
+    int c[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int e = e0 + 32 * u + threadIdx.x, cs = e / w;
-        t[u] = e < wc ? taper[e] : 0.0;
-        d[u] = e < wc ? dp[(size_t)(ij.x + cs) * I.gs_cols + ij.y + e - cs * w] : make_double2(0.0, 0.0);
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const bool in = t[u] != 0.0;
-        const unsigned b = __ballot_sync(FULL, in);
-        if (in) {
-          const int q = n + __popc(b & ((1u << threadIdx.x) - 1u));
-          const int et = exponent64(t[u]), x = et - ea, odd = x & 1;
-          Df s = df(0.f);
-          if (t[u] > 0.0) s = df_sqrt(df_mul(df_split(t[u], odd - et), ia));
-          const int es = (x - odd) / 2;
-          sm.cell[q] = (es + CELL_EXP) << CELL_BITS | (e0 + 32 * u + (int)threadIdx.x);
-          sm.st[q] = st_df(s);
-          const int e1 = exponent64(d[u].x), e2 = exponent64(d[u].y);
-          const int em = e1 > e2 ? e1 : e2;
-          if (em > -1022) ed = max(ed, em + es);
-        }
-        n += __popc(b);
-      }
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + 32 * u + lane, cs = e / w, ct = e - cs * w;
+      c[u] = cs << 5 | ct;
+      t[u] = e < wc ? taper[e] : 0.0;
+      d[u] = e < wc ? dp[(size_t)(ij.x + cs) * I.gs_cols + ij.y + ct] : make_double2(0.0, 0.0);
     }
-    ed = __reduce_max_sync(FULL, ed);
-    if (threadIdx.x == 0) {
-      sm.redi()[0] = n;
-      sm.redi()[1] = ed;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool in = t[u] != 0.0;
+      const unsigned b = __ballot_sync(FULL, in);
+      if (in) {
+        const int q = n + __popc(b & ((1u << lane) - 1u));
+        const int et = exponent64(t[u]), x = et - ea, odd = x & 1;
+        Df s = df(0.f);
+        if (t[u] > 0.0) s = df_sqrt(df_mul(df_split(t[u], odd - et), ia));
+        const int es = (x - odd) / 2;
+        sm.cell[q] = (es + CELL_EXP) << CELL_BITS | c[u];
+        sm.st[q] = st_df(s);
+        const int em = max(exponent64(d[u].x), exponent64(d[u].y));
+        if (em > -1022) ed = max(ed, em + es);
+      }
+      n += __popc(b);
     }
   }
-  __syncthreads();
-  return sm.redi()[0];
+  ed = __reduce_max_sync(FULL, ed);
+  if (lane == 0) {
+    sm.redi()[0] = n;
+    sm.redi()[1] = ed;
+  }
 }
 
 // Slopes q0 .. q0 + nq - 1 of the support list into Yh, Yl (zero on the padding): SCALE:
@@ -165,14 +168,13 @@ __device__ __forceinline__ void stage_slopes(const LkInst &I, int2 ij, const Sme
   using C = S64<MPD>;
   const double *__restrict__ Ybp = static_cast<const double *>(I.Ybp);
   const double *__restrict__ dp = static_cast<const double *>(I.dp);
-  const int m = I.m, w = I.w;
+  const int m = I.m;
 #pragma unroll 4
   for (int e = threadIdx.x; e < nq * MPD; e += C::NT) {
     const int q = e / MPD, i = e - q * MPD;
     const int k = (q0 + q) >> 1, cc = (q0 + q) & 1;
-    const int ce = sm.cell[k] & ((1 << CELL_BITS) - 1), cs = ce / w;
-    const int es = (sm.cell[k] >> CELL_BITS) - CELL_EXP;
-    const size_t src = (size_t)(ij.x + cs) * I.gs_cols + (ij.y + ce - cs * w);
+    const int ce = sm.cell[k], es = (ce >> CELL_BITS) - CELL_EXP;
+    const size_t src = (size_t)(ij.x + cell_row(ce)) * I.gs_cols + (ij.y + cell_col(ce));
     const double v = i < m ? Ybp[(src * 2 + cc) * m + i] : 0.0;
     Df z = df_split(v, SCALE ? es : ey);
     if (SCALE) z = df_mul(z, ld_df(sm.st[k]));
@@ -337,6 +339,20 @@ __device__ __forceinline__ Df product(const Seg64<MPD> &g, const float *b, int v
   return s;
 }
 
+// The same of the high parts alone.
+template <int MPD>
+__device__ __forceinline__ float product32(const Seg64<MPD> &g, const float *b, int vec, int seg) {
+  using C = S64<MPD>;
+  const float2 *ph = reinterpret_cast<const float2 *>(b + (vec * C::KS + seg) * C::TS);
+  float2 S = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int j = 0; j < C::L / 2; ++j) S = __ffma2_rn(g.h[j], ph[j], S);
+  float s = S.x + S.y;
+#pragma unroll
+  for (int o = 1; o < C::KS; o <<= 1) s += __shfl_xor_sync(FULL, s, o);
+  return s;
+}
+
 template <int MPD>
 __device__ __forceinline__ int slot64(int vec, int row) {
   using C = S64<MPD>;
@@ -348,29 +364,31 @@ __device__ __forceinline__ void put64(float *buf, int slot, Df v) {
   buf[S64<MPD>::VEC + slot] = v.l;
 }
 
-// The two rows of X at the node: their means (red64[8..9]), exponents (redi[2..3]) and
-// anomalies times 2^-exponent (xs and the term buffer 0). Ends with a barrier.
+// Row r of X at the node, by one warp: its mean (red64[8 + r]), exponent (redi[2 + r]) and
+// anomalies times 2^-exponent (xs and the term buffer 0).
 template <int MPD>
-__device__ __forceinline__ void rows64(const double *__restrict__ xrow, int m,
-                                       const Smem64<MPD> &sm) {
-  const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
-  if (wv < 2) {                                      // NT >= 64: two warps at least
-    const double x = lane < m ? xrow[(size_t)wv * m + lane] : 0.0;
-    const double mu = lk_warp_sum(x) / m;
-    const double xa = lane < m ? x - mu : 0.0;
-    const int ex = __reduce_max_sync(FULL, exponent64(xa));
-    const int sh = ex == -1022 ? NO_EXP : ex;
-    if (lane < MPD) {
-      const Df v = df_split(xa, -sh);
-      sm.xs[wv * MPD + lane] = st_df(v);
-      put64<MPD>(sm.tb, slot64<MPD>(wv, lane), v);
-    }
-    if (lane == 0) {
-      sm.red64()[8 + wv] = mu;
-      sm.redi()[2 + wv] = sh;
-    }
+__device__ __forceinline__ void row64(const double *__restrict__ xrow, int m, int r,
+                                      const Smem64<MPD> &sm) {
+  const int lane = threadIdx.x & 31;
+  const double x = lane < m ? xrow[(size_t)r * m + lane] : 0.0;
+  const double mu = lk_warp_sum(x) / m;
+  const double xa = lane < m ? x - mu : 0.0;
+  const int ex = __reduce_max_sync(FULL, exponent64(xa));
+  const int sh = ex == -1022 ? NO_EXP : ex;
+  if (lane < MPD) {
+    const Df v = df_split(xa, -sh);
+    sm.xs[r * MPD + lane] = st_df(v);
+    put64<MPD>(sm.tb, slot64<MPD>(r, lane), v);
   }
-  __syncthreads();
+  if (lane == 0) {
+    sm.red64()[8 + r] = mu;
+    sm.redi()[2 + r] = sh;
+  }
+}
+// The warp that looks after row r while warp 0 lists the support (two warps at least).
+template <int MPD>
+__device__ __forceinline__ bool row_warp(int wv, int r) {
+  return wv == (S64<MPD>::NW >= 3 ? 1 + r : 1);
 }
 
 template <int MPD>
@@ -389,9 +407,16 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
   const Smem64<MPD> sm(sm64, w);
   const int pid = it.y;
   const int2 ij = I.pts[pid];
-  const int nsl = 2 * support<MPD>(I, ij, sm), ed = sm.redi()[1];
-  gram64<MPD>(I, ij, sm, nsl, ed);
   const int t = threadIdx.x, seg = t % C::KS, vec = (t / C::KS) & 1, row = t / (2 * C::KS);
+  const int lane = t & 31, wv = t >> 5;
+  double *xrow = static_cast<double *>(I.X) + (size_t)pid * 2 * m;
+  if (wv == 0) support<MPD>(I, ij, sm);
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+    if (row_warp<MPD>(wv, r)) row64<MPD>(xrow, m, r, sm);
+  __syncthreads();
+  const int nsl = 2 * sm.redi()[0], ed = sm.redi()[1];
+  gram64<MPD>(I, ij, sm, nsl, ed);
   Seg64<MPD> g;
   const float f2 = seg_load<MPD>(g, sm, row, seg);
   // both vectors' threads hold G: half the sum of squares is |G|_F^2
@@ -400,18 +425,16 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
     if (t == 0) worklist[atomicAdd(queue, 1)] = make_int2(it.x, pid);
     return;
   }
-  double *xrow = static_cast<double *>(I.X) + (size_t)pid * 2 * m;
-  rows64<MPD>(xrow, m, sm);
-  // ---- the series ----
+  // ---- the series: terms up to `low` in pairs, then in floats ----
   const float4 *co = cheb + (size_t)lk_cheb_class(ratio) * LK_CHEB_LD64;
   const float4 c0 = co[0];
-  const int deg = (int)c0.z;
+  const int deg = (int)c0.z, low = (int)c0.w;
   seg_scale<MPD>(g, Df{c0.x, c0.y}, row, seg);
   const float2 *ck = reinterpret_cast<const float2 *>(co + 1) + (seg & 1);
   Df tp = df(0.f), tc = ld_df(sm.xs[vec * MPD + row]);
   Df acc = df_mul(ld_df(__ldg(ck)), tc);
   const int sl = slot64<MPD>(vec, row);
-  for (int k = 1; k <= deg; ++k) {
+  for (int k = 1; k <= low; ++k) {
     const Df c = ld_df(__ldg(ck + 2 * k));
     const Df gt = product<MPD>(g, sm.tb + ((k - 1) & 1) * 2 * C::VEC, vec, seg);
     // T_k = 2 X T_k-1 - T_k-2, T_1 = X T_0
@@ -422,6 +445,19 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
     __syncthreads();
     acc = df_add(acc, df_mul(c, tc));
   }
+  {
+    float ah = 0.f, pf = tp.h, cf = tc.h;
+    for (int k = low + 1; k <= deg; ++k) {
+      const float c = __ldg(ck + 2 * k).x;
+      const float tn = product32<MPD>(g, sm.tb + ((k - 1) & 1) * 2 * C::VEC, vec, seg) - pf;
+      if (seg == 0) sm.tb[(k & 1) * 2 * C::VEC + sl] = tn;
+      pf = cf;
+      cf = tn;
+      __syncthreads();
+      ah = fmaf(c, tn, ah);
+    }
+    acc = df_add(acc, df(ah));
+  }
   // ---- X'_r wbar = (A^-1 x'_r) . C d, X'_r W, and the outputs ----
   // (the lanes of the two vectors alternate every KS: each sums its own)
   Df pr = seg == 1 ? df_mul(acc, ld_df(sm.cv[row])) : df(0.f);
@@ -431,7 +467,6 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
   if ((t & 31) == vec * C::KS) sm.red[2 * (t >> 5) + vec] = st_df(pr);
   if (seg == 0) sm.xs[vec * MPD + row] = st_df(acc);
   __syncthreads();
-  const int lane = t & 31, wv = t >> 5;
   if (wv < 2) {                                      // a warp per row of X
     const Alpha64 al(I.alpha, m);
     Df p = ld_df(sm.red[wv]);
@@ -513,10 +548,31 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
   float2 *qs = gv + 2 * MPD, *qc = qs + 2 * C::QC, *qd = qc + C::QC, *qf = qd + C::QC;
   int *qe = reinterpret_cast<int *>(qf + C::QC);
   const int2 ij = I.pts[pid];
-  const int nsl = 2 * support<MPD>(I, ij, sm), ed = sm.redi()[1];
-  gram64<MPD>(I, ij, sm, nsl, ed);
   const int t = threadIdx.x, seg = t % C::KS, vec = (t / C::KS) & 1, row = t / (2 * C::KS);
   const int lane = t & 31, wv = t >> 5;
+  int *ri = sm.redi();
+  if (wv == 0) support<MPD>(I, ij, sm);
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+    if (row_warp<MPD>(wv, r)) {
+      row64<MPD>(static_cast<const double *>(I.X) + (size_t)pid * 2 * m, m, r, sm);
+      // g_r and s_r = g_r . 1
+      const double x = lane < m ? a.lam_a[((size_t)pid * 2 + r) * m + lane] : 0.0;
+      const double s = lk_warp_sum(x);
+      const int ex = __reduce_max_sync(FULL, exponent64(x)), sh = ex == -1022 ? NO_EXP : ex;
+      if (lane < MPD) {
+        const Df v = df_split(x, -sh);
+        gv[r * MPD + lane] = st_df(v);
+        put64<MPD>(terms, slot64<MPD>(r, lane), v);
+      }
+      if (lane == 0) {
+        sm.red64()[10 + r] = s;
+        ri[4 + r] = sh;
+      }
+    }
+  __syncthreads();
+  const int nsl = 2 * ri[0], ed = ri[1];
+  gram64<MPD>(I, ij, sm, nsl, ed);
   Seg64<MPD> g;
   const float f2 = seg_load<MPD>(g, sm, row, seg);
   const float ratio = sqrtf(0.5f * cta_sum<C::NW>(f2, sm.red));
@@ -524,24 +580,7 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
     if (t == 0) a.queue[atomicAdd(a.queue_len, 1)] = make_int2(0, pid);
     return;
   }
-  rows64<MPD>(static_cast<const double *>(I.X) + (size_t)pid * 2 * m, m, sm);
-  int *ri = sm.redi();
-  if (wv < 2) {                                      // g_r and s_r = g_r . 1
-    const double x = lane < m ? a.lam_a[((size_t)pid * 2 + wv) * m + lane] : 0.0;
-    const double s = lk_warp_sum(x);
-    const int ex = __reduce_max_sync(FULL, exponent64(x)), sh = ex == -1022 ? NO_EXP : ex;
-    if (lane < MPD) {
-      const Df v = df_split(x, -sh);
-      gv[wv * MPD + lane] = st_df(v);
-      put64<MPD>(terms, slot64<MPD>(wv, lane), v);
-    }
-    if (lane == 0) {
-      sm.red64()[10 + wv] = s;
-      ri[4 + wv] = sh;
-      a.xbar_bar[(size_t)pid * 2 + wv] = s;
-    }
-  }
-  __syncthreads();
+  if (t < 2) a.xbar_bar[(size_t)pid * 2 + t] = sm.red64()[10 + t];
   // s_0 x'_0 + s_1 x'_1 times 2^-eb
   const int ex0 = ri[2], ex1 = ri[3], eg0 = ri[4], eg1 = ri[5];
   const double s0 = sm.red64()[10], s1 = sm.red64()[11];
@@ -564,6 +603,7 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
   const Df scale = Df{c0.x, c0.y};
   const int deg = (int)c0.z;
   const bool keep = deg <= ADJ_KEEP;
+  const int low = keep ? (int)c0.w : deg;            // (run backwards the terms stay pairs)
   seg_scale<MPD>(g, scale, row, seg);
   ++co;
   Df tc = ld_df(gv[vec * MPD + row]), tp = df(0.f), yp = df(0.f), ga, ya;
@@ -572,7 +612,7 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
     ga = df_mul(Df{c.x, c.y}, tc);
     ya = df_mul(Df{c.z, c.w}, yc);
   }
-  for (int k = 1; k <= deg; ++k) {
+  for (int k = 1; k <= low; ++k) {
     const float4 c = __ldg(co + k);
     const Df gt = product<MPD>(g, terms + (keep ? k - 1 : (k - 1) & 1) * 2 * C::VEC, vec, seg);
     const Df gy = product<MPD>(g, sb + ((k - 1) & 1) * 2 * C::VEC, vec, seg);
@@ -590,6 +630,27 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
     ga = df_add(ga, df_mul(Df{c.x, c.y}, tc));
     ya = df_add(ya, df_mul(Df{c.z, c.w}, yc));
   }
+  {
+    float gs = 0.f, ys = 0.f, tq = tp.h, tf = tc.h, yq = yp.h, yf = yc.h;
+    for (int k = low + 1; k <= deg; ++k) {
+      const float4 c = __ldg(co + k);
+      const float tn = product32<MPD>(g, terms + (k - 1) * 2 * C::VEC, vec, seg) - tq;
+      const float yn = product32<MPD>(g, sb + ((k - 1) & 1) * 2 * C::VEC, vec, seg) - yq;
+      tq = tf;
+      tf = tn;
+      yq = yf;
+      yf = yn;
+      if (seg == 0) {
+        terms[k * 2 * C::VEC + sl] = tn;
+        sb[(k & 1) * 2 * C::VEC + sl] = yn;
+      }
+      __syncthreads();
+      gs = fmaf(c.x, tn, gs);
+      ys = fmaf(c.z, yn, ys);
+    }
+    ga = df_add(ga, df(gs));
+    ya = df_add(ya, df(ys));
+  }
   const Alpha64 al(I.alpha, m);
   // wbar times 2^-ed, then b_bar times 2^-ebb
   const int ebb = eb - al.e;
@@ -598,10 +659,12 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
   float2 S[C::L / 2], F[C::L / 2];
 #pragma unroll
   for (int j = 0; j < C::L / 2; ++j) S[j] = F[j] = make_float2(0.f, 0.f);
-  Df p, pn = df(0.f);                                // P_{deg-1}, P_deg
+  // P_{deg-1} and P_deg; down to P_low in floats (with a zero low part in the buffer)
+  Df p, pn = df(0.f);
   {
     const float4 c = __ldg(co + deg);
     p = df_mul(Df{c.x, c.y}, x);
+    if (deg - 1 >= low) p.l = 0.f;
   }
   if (seg == 0) put64<MPD>(sm.tb + ((deg - 1) & 1) * 2 * C::VEC, sl, p);
   __syncthreads();
@@ -610,7 +673,34 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
     a.xp_bar[((size_t)pid * 2 + vec) * m + row] =
         u + df_to_double(df_mul(al.rt, ga), al.re + (vec ? eg1 : eg0));
   }
-  for (int j = deg - 1; j >= 0; --j) {
+  {
+    float2 SF[C::L / 2];
+#pragma unroll
+    for (int c = 0; c < C::L / 2; ++c) SF[c] = make_float2(0.f, 0.f);
+    for (int j = deg - 1; j >= low; --j) {           // (low >= 1)
+      const float2 *qh = reinterpret_cast<const float2 *>(
+          terms + j * 2 * C::VEC + (vec * C::KS + seg) * C::TS);
+      const float2 ph = dup2(2.f * p.h);
+#pragma unroll
+      for (int c = 0; c < C::L / 2; ++c) SF[c] = __ffma2_rn(ph, qh[c], SF[c]);
+      const float gp = product32<MPD>(g, sm.tb + (j & 1) * 2 * C::VEC, vec, seg);
+      float pm = fmaf(__ldg(co + j).x, x.h, gp - pn.h), pl = 0.f;
+      if (j == low) {                                // P_{low-1} in pairs again
+        const float4 c = __ldg(co + j);
+        const Df gd = product<MPD>(g, sm.tb + (j & 1) * 2 * C::VEC, vec, seg);
+        const Df pd = df_add(df_add(gd, df_neg(pn)), df_mul(Df{c.x, c.y}, x));
+        pm = pd.h;
+        pl = pd.l;
+      }
+      pn = p;
+      p = Df{pm, pl};
+      if (seg == 0) put64<MPD>(sm.tb + ((j - 1) & 1) * 2 * C::VEC, sl, p);
+      __syncthreads();
+    }
+#pragma unroll
+    for (int c = 0; c < C::L / 2; ++c) S[c] = SF[c];
+  }
+  for (int j = low - 1 < deg - 1 ? low - 1 : deg - 1; j >= 0; --j) {
     // the terms' own recurrence run backwards holds T_{j+1} = tc, T_j = tp
     const float2 *qh = reinterpret_cast<const float2 *>(
         terms + (keep ? j : j & 1) * 2 * C::VEC + (vec * C::KS + seg) * C::TS);
@@ -705,10 +795,10 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
     double cj = 0.0, dj = 0.0;                       // the slope of warp 0's lane
     int ce = 0;
     if (wv == 0 && lane < nq) {
-      ce = sm.cell[(q0 + lane) >> 1] & ((1 << CELL_BITS) - 1);
-      const int cs = ce / w;
+      const int c = sm.cell[(q0 + lane) >> 1];
+      ce = cell_row(c) * w + cell_col(c);
       cj = tap[ce];
-      dj = dp[((size_t)(ij.x + cs) * I.gs_cols + (ij.y + ce - cs * w)) * 2 + (lane & 1)];
+      dj = dp[((size_t)(ij.x + cell_row(c)) * I.gs_cols + (ij.y + cell_col(c))) * 2 + (lane & 1)];
       // y_bar = c 2^ec (2 (A_bar y) 2^(eA - ey) + d 2^el b_bar 2^ebb)
       const int ec = exponent64(cj), el = dj == 0.0 ? NO_EXP : exponent64(dj);
       const int ea = eA - ey + 1, eb2 = el + ebb, eo = max(ea, eb2);
@@ -772,7 +862,7 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
     for (int q = t; q < nq * MPD; q += C::NT) {
       const int k = q / MPD, i = q - k * MPD;
       if (i >= m) continue;
-      const int cell = sm.cell[(q0 + k) >> 1] & ((1 << CELL_BITS) - 1);
+      const int c = sm.cell[(q0 + k) >> 1], cell = cell_row(c) * w + cell_col(c);
       const float2 f = qf[k];
       const Df u = df_mul(Df{f.y * qd[k].x, f.y * qd[k].y}, ld_df(bb[i]));
       const Df v = df_add(Df{f.x * ayh[k * C::LDY + i], f.x * ayl[k * C::LDY + i]}, u);
