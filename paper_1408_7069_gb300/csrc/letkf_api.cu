@@ -467,7 +467,12 @@ letkf_status enqueue_head(letkf_ctx *h, const void *y, const void *truth, double
   } else if (res) {
     LK_CUDA(h, lk_launch_residual(h, truth, resvar, ridx));
   }
-  LK_CUDA(h, lk_launch_obs(h, y, ridx));
+  if (h->sap_total > 0) {
+    *drawn = all_have_banks(h);
+    LK_CUDA(h, lk_launch_obs_residual(h, y, nullptr, nullptr, ridx, *drawn ? h->noise_pre : nullptr));
+  } else {
+    LK_CUDA(h, lk_launch_obs(h, y, ridx));
+  }
   if (fork) LK_CUDA(h, cudaStreamWaitEvent(h->stream, h->ev_join, 0));
   return LETKF_OK;
 }
@@ -478,6 +483,9 @@ letkf_status enqueue_frame(letkf_ctx *h, const void *y_seq, const void *truth_se
   bool drawn;
   letkf_status st = enqueue_head(h, y_seq, truth_seq, resvar, ridx, &drawn);
   if (st != LETKF_OK) return st;
+  bool done;
+  LK_CUDA(h, lk_launch_cycle(h, drawn ? h->noise_pre : nullptr, &done));
+  if (done) return LETKF_OK;
   LK_CUDA(h, lk_launch_analysis(h, nullptr, nullptr));
   LK_CUDA(h, lk_launch_forecast(h, drawn ? h->noise_pre : nullptr));
   return LETKF_OK;
@@ -486,7 +494,8 @@ letkf_status enqueue_frame(letkf_ctx *h, const void *y_seq, const void *truth_se
 // One frame from the step staging buffers: upload, (residual beside the)
 // observation, analysis (mean into staging), download, then the forecast.
 // ev_out is recorded after the downloads (an event node of the step graph),
-// so that the caller can return its outputs while the forecast still runs.
+// so that the caller can return its outputs while the forecast still runs (the
+// form of lk_launch_cycle, no faster here, would put it before them).
 letkf_status enqueue_step(letkf_ctx *h, bool with_truth) {
   unsigned char *yd = h->step_dev + h->step_off[0], *td = h->step_dev + h->step_off[1];
   unsigned char *md = h->step_dev + h->step_off[2], *rd = h->step_dev + h->step_off[3];
@@ -518,9 +527,16 @@ letkf_status enqueue_frame_dm(letkf_ctx *h, const void *truth_seq, const void *w
   const long long *ridx = h->frame + 1;
   if (resvar) LK_CUDA(h, lk_launch_residual(h, truth_seq, resvar, ridx));
   LK_CUDA(h, lk_launch_dm_wfs(h, truth_seq, wnoise_seq, ridx, h->dm_wfs_y));
-  LK_CUDA(h, lk_launch_obs(h, h->dm_wfs_y, nullptr));
+  void *noise = h->sap_total > 0 && all_have_banks(h) ? h->noise_pre : nullptr;
+  if (noise)
+    LK_CUDA(h, lk_launch_obs_residual(h, h->dm_wfs_y, nullptr, nullptr, nullptr, noise));
+  else
+    LK_CUDA(h, lk_launch_obs(h, h->dm_wfs_y, nullptr));
+  bool done;
+  LK_CUDA(h, lk_launch_cycle(h, noise, &done));
+  if (done) return LETKF_OK;
   LK_CUDA(h, lk_launch_analysis(h, nullptr, nullptr));
-  LK_CUDA(h, lk_launch_forecast(h, nullptr));
+  LK_CUDA(h, lk_launch_forecast(h, noise));
   return LETKF_OK;
 }
 

@@ -202,11 +202,22 @@ struct letkf_ctx {
 cudaError_t lk_launch_obs(letkf_ctx *h, const void *y, const long long *run_idx);
 // Observation of one frame with, in the same launch, its residual (truth and
 // resvar given) and the model noise of the frame's forecast (noise_out given,
-// [n_pts][m] at each instance's noise_off). Not with a deformable mirror, whose
-// residual needs N u first, nor without subapertures.
+// [n_pts][m] at each instance's noise_off). No residual with a deformable mirror, whose
+// residual needs N u first; not without subapertures.
 cudaError_t lk_launch_obs_residual(letkf_ctx *h, const void *y, const void *truth,
                                    double *resvar, const long long *run_idx, void *noise_out);
 cudaError_t lk_launch_analysis(letkf_ctx *h, void *mean, void *spread);
+// The forecast inside the analysis (it is local to a node): with the noise already drawn,
+// every kernel that writes a node's analysis writes its forecast instead, phi_k to row 1 and
+// a phi_k + v to row 0, and the last list kernel advances the counters. `noise` NULL: no.
+struct LkCycle {
+  const void *noise = nullptr;   // [n_pts][m] at each instance's noise_off
+  long long *frame = nullptr;    // the counters to advance, or NULL
+};
+// Analysis and forecast of a frame in the analysis kernels; *done is false, and nothing
+// launched, where the handle's analysis has no such form (domains, row-split or
+// FP64-sweep analyses, no list kernels) or no noise is given.
+cudaError_t lk_launch_cycle(letkf_ctx *h, const void *noise, bool *done);
 cudaError_t lk_launch_analysis_class(letkf_ctx *h, int cls, void *mean, void *spread);
 // The forecast also advances the forecast counter and the run index (frame[0..1]).
 cudaError_t lk_launch_forecast(letkf_ctx *h, const void *noise);
@@ -228,7 +239,7 @@ cudaError_t lk_launch_dm_get(letkf_ctx *h, void *out);
 cudaError_t lk_launch_stamp(letkf_ctx *h, unsigned long long *dst);
 cudaError_t lk_setup_analysis(letkf_ctx *h);
 // FP32 analysis of width class cls, two columns per lane (letkf_pair.cu).
-cudaError_t lk_launch_pair(letkf_ctx *h, int cls, void *mean, void *spread);
+cudaError_t lk_launch_pair(letkf_ctx *h, int cls, void *mean, void *spread, const LkCycle &cy = {});
 cudaError_t lk_setup_pair(letkf_ctx *h);
 // Inputs and outputs of the reverse mode's node kernels (letkf_adjoint.cu).
 struct LkAdjArgs {
@@ -245,7 +256,8 @@ struct LkAdjArgs {
 // width class cls of an FP64 handle, those above LK_CHEB_MAX64 queued in the
 // class's worklist; and the adjoint of every node, likewise queued in a.queue.
 bool lk_series64(const letkf_ctx *h);     // whether the handle takes this form
-cudaError_t lk_launch_series64(letkf_ctx *h, int cls, void *mean, void *spread);
+cudaError_t lk_launch_series64(letkf_ctx *h, int cls, void *mean, void *spread,
+                               const LkCycle &cy = {});
 cudaError_t lk_launch_adj_series64(letkf_ctx *h, const LkAdjArgs &a);
 cudaError_t lk_setup_series64(letkf_ctx *h);
 // Allocates and fills the handle's Chebyshev tables (letkf_cheb.cu).
@@ -254,7 +266,8 @@ cudaError_t lk_setup_cheb(letkf_ctx *h);
 // node of width class cls (0: MP 16, 1: MP 32) of an FP64 handle, or the nodes
 // the pair kernel queued in class cls of an FP32 handle.
 cudaError_t lk_launch_node64(letkf_ctx *h, int cls, void *mean, void *spread);
-cudaError_t lk_launch_list64(letkf_ctx *h, int cls, void *mean, void *spread);
+cudaError_t lk_launch_list64(letkf_ctx *h, int cls, void *mean, void *spread,
+                             const LkCycle &cy = {});
 // Shared-memory limit of the wide class's FP64 list kernel (MP = 48 / 64 queue), and
 // of the list kernel with the tridiagonal form.
 cudaError_t lk_setup_node64w();
@@ -353,5 +366,37 @@ __device__ __forceinline__ unsigned long long lk_splitmix64(unsigned long long s
   z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
   z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
   return z ^ (z >> 31);
+}
+
+// The AR(1) forecast of member i at node gpt (Section 2.2): a x + v, v the drawn noise.
+template <typename S>
+__device__ __forceinline__ S lk_ar1(const LkInst &I, const S *__restrict__ noise, int gpt, int i,
+                                    S x) {
+  return fma(S(I.a_ar1), x, noise[I.noise_off + (long long)gpt * I.m + i]);
+}
+// The forecast of a node in place, by one warp (lane = member): phi_k to row 1, a phi_k + v
+// to row 0; with a deformable mirror the predicted phase, for the command u = P phihat.
+template <typename S>
+__device__ __forceinline__ void lk_forecast_warp(const LkInst &I, const S *__restrict__ noise,
+                                                 int gpt, int lane) {
+  S *row0 = static_cast<S *>(I.X) + (size_t)gpt * 2 * I.m;
+  S psum = S(0);
+  for (int i = lane; i < I.m; i += 32) {
+    const S x = row0[i], f = lk_ar1<S>(I, noise, gpt, i, x);
+    row0[I.m + i] = x;
+    row0[i] = f;
+    psum += f;
+  }
+  if (I.dm) {
+    psum = lk_warp_sum(psum);
+    if (lane == 0) static_cast<S *>(I.pmean)[gpt] = psum / S(I.m);
+  }
+}
+// Counters of the forecast, by the last list kernel of a frame (nothing in it reads them).
+__device__ __forceinline__ void lk_advance(long long *__restrict__ frame) {
+  if (frame && blockIdx.x == 0 && threadIdx.x == 0) {
+    frame[0] += 1;
+    frame[1] += 1;
+  }
 }
 #endif

@@ -121,7 +121,7 @@ __device__ __forceinline__ void forecast_node(const LkInst *__restrict__ insts, 
     const S x0 = row0[i];
     const S v = noise ? noise[I.noise_off + (long long)gpt * m + i] : bank_draw<S>(I, ij, i, frame[0]);
     row0[m + i] = x0;
-    row0[i] = a * x0 + v;
+    row0[i] = fma(a, x0, v);
     psum += row0[i];
   }
   if (I.dm) {                       // the predicted phase, for the command u = P phihat
@@ -335,8 +335,8 @@ cudaError_t lk_launch_obs(letkf_ctx *h, const void *y, const long long *run_idx)
 
 cudaError_t lk_launch_obs_residual(letkf_ctx *h, const void *y, const void *truth,
                                    double *resvar, const long long *run_idx, void *noise_out) {
-  if (h->sap_total == 0 || h->inst[0].dm) return cudaErrorInvalidValue;
   const int rblocks = (truth && resvar) ? LK_RES_BLOCKS * h->n_inst : 0;
+  if (h->sap_total == 0 || (rblocks && h->inst[0].dm)) return cudaErrorInvalidValue;
   const int nblocks = noise_out ? warp_blocks(h->n_pts_total) : 0;
   const int blocks = rblocks + nblocks + warp_blocks(h->sap_total);
   if (h->precision == 1)

@@ -402,7 +402,8 @@ __global__ void __launch_bounds__(N64_THREADS)
                   S *__restrict__ mean, S *__restrict__ spread, double tol, int max_sweeps,
                   int *__restrict__ counters, int keep_basis) {
   extern __shared__ __align__(16) double n64_smem[];
-  lk_pdl_wait();   // no early trigger (long kernel): dependents launch as its CTAs exit
+  lk_pdl_wait();
+  lk_pdl_trigger();
   const int2 it = items[blockIdx.x];
   const LkInst &I = insts[it.x];
   if (I.mp != MP) return;
@@ -420,9 +421,12 @@ __global__ void __launch_bounds__(N64_THREADS)
     node64_list_kernel(const LkInst *__restrict__ insts, const int2 *__restrict__ worklist,
                        const int *__restrict__ queue_len, S *__restrict__ mean,
                        S *__restrict__ spread, double tol, int max_sweeps,
-                       int *__restrict__ counters, int keep_basis) {
+                       int *__restrict__ counters, int keep_basis, const S *__restrict__ noise,
+                       long long *__restrict__ frame) {
   extern __shared__ __align__(16) double n64_smem[];
-  lk_pdl_wait();   // no early trigger (long kernel): dependents launch as its CTAs exit
+  lk_pdl_wait();
+  lk_pdl_trigger();
+  lk_advance(frame);
   const int qn = *queue_len;
   for (int idx = blockIdx.x; idx < qn; idx += gridDim.x) {
     const int2 it = worklist[idx];
@@ -432,6 +436,7 @@ __global__ void __launch_bounds__(N64_THREADS)
                         spread ? spread + 2 * row : nullptr, tol, LK_WARM_STOP64, max_sweeps,
                         counters, n64_smem, keep_basis != 0, sizeof(S) == 8 ? 2 : 1);
     __syncthreads();                       // shared memory is reused by the next node
+    if (noise && threadIdx.x < 32) lk_forecast_warp<S>(I, noise, it.y, threadIdx.x);
   }
 }
 
@@ -444,10 +449,12 @@ __global__ void __launch_bounds__(N64_THREADS, 3)
                     const int *__restrict__ queue_len,
                     const double2 *__restrict__ poles, float *__restrict__ mean,
                     float *__restrict__ spread, double tol, int max_sweeps,
-                    int *__restrict__ counters) {
+                    int *__restrict__ counters, const float *__restrict__ noise,
+                    long long *__restrict__ frame) {
   extern __shared__ __align__(16) double n64_smem[];
-  lk_pdl_wait();   // no early trigger (long kernel): dependents launch as its CTAs exit
-  const int qn = queue_len[0], tn = queue_len[LK_TRI_LIST];
+  lk_pdl_wait();
+  lk_advance(frame);
+  const int tn = queue_len[LK_TRI_LIST];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float *ws = reinterpret_cast<float *>(n64_smem) + warp * TriCfg<MP>::TOTAL;
   for (int idx = blockIdx.x * (N64_THREADS / 32) + warp; idx < tn;
@@ -473,6 +480,7 @@ __global__ void __launch_bounds__(N64_THREADS, 3)
                  spread ? spread + 2 * row : nullptr, counters, ws);
   }
   __syncthreads();
+  const int qn = queue_len[0];
   for (int idx = blockIdx.x; idx < qn; idx += gridDim.x) {
     const int2 it = worklist[idx];
     const LkInst &I = insts[it.x];
@@ -481,6 +489,18 @@ __global__ void __launch_bounds__(N64_THREADS, 3)
                             spread ? spread + 2 * row : nullptr, tol, LK_WARM_STOP64, max_sweeps,
                             counters, n64_smem);
     __syncthreads();                       // shared memory is reused by the next node
+  }
+  if (noise) {                             // the same nodes' forecasts (a lane its own members)
+    for (int idx = blockIdx.x * (N64_THREADS / 32) + warp; idx < queue_len[LK_TRI_LIST];
+         idx += gridDim.x * (N64_THREADS / 32)) {
+      const int2 it = worklist[n_list - 1 - idx];
+      const LkInst &I = insts[it.x & ((1 << LK_TRI_INST) - 1)];
+      lk_forecast_warp<float>(I, noise, it.y, lane);
+    }
+    for (int idx = blockIdx.x; idx < queue_len[0] && warp == 0; idx += gridDim.x) {
+      const int2 it = worklist[idx];
+      lk_forecast_warp<float>(insts[it.x], noise, it.y, lane);
+    }
   }
 }
 
@@ -790,9 +810,12 @@ __global__ void __launch_bounds__(N64W_THREADS)
     node64w_list_kernel(const LkInst *__restrict__ insts, const int2 *__restrict__ worklist,
                         const int *__restrict__ queue_len, float *__restrict__ mean,
                         float *__restrict__ spread, double tol, int max_sweeps,
-                        int *__restrict__ counters) {
+                        int *__restrict__ counters, const float *__restrict__ noise,
+                        long long *__restrict__ frame) {
   extern __shared__ __align__(16) double n64_smem[];
-  lk_pdl_wait();   // no early trigger (long kernel): dependents launch as its CTAs exit
+  lk_pdl_wait();
+  lk_pdl_trigger();
+  lk_advance(frame);
   const int qn = *queue_len;
   for (int idx = blockIdx.x; idx < qn; idx += gridDim.x) {
     const int2 it = worklist[idx];
@@ -801,6 +824,7 @@ __global__ void __launch_bounds__(N64W_THREADS)
     node64w(I, it.y, mean ? mean + 2 * row : nullptr, spread ? spread + 2 * row : nullptr, tol,
             LK_WARM_STOP64, max_sweeps, counters, n64_smem);
     __syncthreads();                       // shared memory is reused by the next node
+    if (noise && threadIdx.x < 32) lk_forecast_warp<float>(I, noise, it.y, threadIdx.x);
   }
 }
 
@@ -839,7 +863,7 @@ constexpr size_t tri_list_smem() {
 }
 
 template <int MP>
-cudaError_t launch_list64(letkf_ctx *h, int cls, void *mean, void *spread) {
+cudaError_t launch_list64(letkf_ctx *h, int cls, void *mean, void *spread, const LkCycle &cy) {
   long long n = 0;
   for (const LkInst &I : h->inst)
     if (I.mp == MP) n += I.n_pts;
@@ -854,18 +878,19 @@ cudaError_t launch_list64(letkf_ctx *h, int cls, void *mean, void *spread) {
     return lk_launch_pdl(tri_list_kernel<MP>, (unsigned)(n < full ? n : full), N64_THREADS,
                          tri_list_smem<MP>(), h->stream, h->d_inst, list, (int)h->n_pts_total, len,
                          (const double2 *)h->poles, (float *)mean, (float *)spread, h->tol64,
-                         h->max_sweeps, h->counters);
+                         h->max_sweeps, h->counters, (const float *)cy.noise, cy.frame);
   }
   if (h->precision == 1)
     return lk_launch_pdl(node64_list_kernel<MP, double>, blocks, N64_THREADS, smem, h->stream,
                          h->d_inst, list, len, (double *)mean, (double *)spread, h->tol64,
-                         h->max_sweeps, h->counters, h->keep_basis);
+                         h->max_sweeps, h->counters, h->keep_basis, (const double *)cy.noise,
+                         cy.frame);
   return lk_launch_pdl(node64_list_kernel<MP, float>, blocks, N64_THREADS, smem, h->stream,
                        h->d_inst, list, len, (float *)mean, (float *)spread, h->tol64,
-                       h->max_sweeps, h->counters, 0);
+                       h->max_sweeps, h->counters, 0, (const float *)cy.noise, cy.frame);
 }
 
-cudaError_t launch_list64w(letkf_ctx *h, void *mean, void *spread) {
+cudaError_t launch_list64w(letkf_ctx *h, void *mean, void *spread, const LkCycle &cy) {
   long long n = 0;
   for (const LkInst &I : h->inst)
     if (I.mp > 32) n += I.n_pts;
@@ -875,7 +900,8 @@ cudaError_t launch_list64w(letkf_ctx *h, void *mean, void *spread) {
   return lk_launch_pdl(node64w_list_kernel, blocks, N64W_THREADS,
                        n64w_smem_doubles() * sizeof(double), h->stream, h->d_inst,
                        h->worklist + (size_t)2 * h->n_pts_total, h->counters + 6, (float *)mean,
-                       (float *)spread, h->tol64, h->max_sweeps, h->counters);
+                       (float *)spread, h->tol64, h->max_sweeps, h->counters,
+                       (const float *)cy.noise, cy.frame);
 }
 
 }  // namespace
@@ -897,8 +923,8 @@ cudaError_t lk_launch_node64(letkf_ctx *h, int cls, void *mean, void *spread) {
   return cls == 0 ? launch_node64<16>(h, mean, spread) : launch_node64<32>(h, mean, spread);
 }
 
-cudaError_t lk_launch_list64(letkf_ctx *h, int cls, void *mean, void *spread) {
-  if (cls == 2) return launch_list64w(h, mean, spread);
-  return cls == 0 ? launch_list64<16>(h, cls, mean, spread)
-                  : launch_list64<32>(h, cls, mean, spread);
+cudaError_t lk_launch_list64(letkf_ctx *h, int cls, void *mean, void *spread, const LkCycle &cy) {
+  if (cls == 2) return launch_list64w(h, mean, spread, cy);
+  return cls == 0 ? launch_list64<16>(h, cls, mean, spread, cy)
+                  : launch_list64<32>(h, cls, mean, spread, cy);
 }

@@ -402,7 +402,8 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
                          float *__restrict__ mean, float *__restrict__ spread, float tol,
                          float stop, int max_sweeps, float kappa_thr, int *__restrict__ counters,
                          int *__restrict__ queue, int2 *__restrict__ worklist, int keep_basis,
-                         const float2 *__restrict__ cheb, int n_list) {
+                         const float2 *__restrict__ cheb, int n_list,
+                         const float *__restrict__ noise) {
   lk_pdl_wait();   // no early trigger: the next kernel launches as this one's CTAs exit
   LK_PHASE_STAMP(ph0);
   using C = PairCfg<MP>;
@@ -705,15 +706,15 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
   LK_PHASE_STAMP(ph3);
   const float xa00 = xb0 + w0 + xa0.x, xa01 = xb0 + w0 + xa0.y;
   const float xa10 = xb1 + w1 + xa1.x, xa11 = xb1 + w1 + xa1.y;
-  if (wr) {
-    if (in0) {
-      xrow[m0] = xa00;
-      xrow[m + m0] = xa10;
-    }
-    if (in1) {
-      xrow[m1] = xa01;
-      xrow[m + m1] = xa11;
-    }
+  // with noise, the forecast is written instead (the sums below cover its loads)
+  float f0 = xa00, f1 = xa01;
+  if (noise && wr) {
+    if (in0) f0 = lk_ar1<float>(I, noise, pid, m0, xa00);
+    if (in1) f1 = lk_ar1<float>(I, noise, pid, m1, xa01);
+  }
+  if (noise && I.dm) {                               // the predicted phase
+    const float ps = group_sum<GL>((in0 ? f0 : 0.f) + (in1 ? f1 : 0.f));
+    if (wr && li == 0) static_cast<float *>(I.pmean)[pid] = ps / float(m);
   }
   const float e00 = in0 ? xa00 : 0.f, e01 = in1 ? xa01 : 0.f;
   const float e10 = in0 ? xa10 : 0.f, e11 = in1 ? xa11 : 0.f;
@@ -723,6 +724,16 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
   const float d10 = in0 ? xa10 - mu1 : 0.f, d11 = in1 ? xa11 - mu1 : 0.f;
   const float sp0 = sqrtf(group_sum<GL>(d00 * d00 + d01 * d01) / float(m - 1));
   const float sp1 = sqrtf(group_sum<GL>(d10 * d10 + d11 * d11) / float(m - 1));
+  if (wr) {
+    if (in0) {
+      xrow[m0] = f0;
+      xrow[m + m0] = noise ? xa00 : xa10;
+    }
+    if (in1) {
+      xrow[m1] = f1;
+      xrow[m + m1] = noise ? xa01 : xa11;
+    }
+  }
   if (wr && li == 0) {
     const long long row = I.node_off + pid;
     if (mean) {
@@ -1072,7 +1083,7 @@ bool serves(const LkInst &I) {
 
 template <int MP, int TI, int TJ, bool SPLIT>
 cudaError_t launch_shape(letkf_ctx *h, const LkTile *tiles, int n_tiles, float *mean,
-                         float *spread, float kthr, int *queue, int2 *worklist) {
+                         float *spread, float kthr, int *queue, int2 *worklist, const float *noise) {
   if (n_tiles == 0) return cudaSuccess;
   if constexpr (SPLIT ? !split_shape_ok<MP, TI, TJ>() : !shape_ok<MP, TI, TJ>()) {
     return cudaErrorInvalidConfiguration;
@@ -1093,13 +1104,13 @@ cudaError_t launch_shape(letkf_ctx *h, const LkTile *tiles, int n_tiles, float *
                          TI * TJ * 32 / PairCfg<MP>::NPW, need, h->stream, h->d_inst, tiles, mean,
                          spread, (float)h->tol32, (float)h->stop32, h->max_sweeps, kthr,
                          h->counters, queue, worklist, h->keep_basis,
-                         (const float2 *)h->cheb32, (int)h->n_pts_total);
+                         (const float2 *)h->cheb32, (int)h->n_pts_total, noise);
   }
 }
 
 template <int MP>
 cudaError_t launch_mp(letkf_ctx *h, int cls, const LkTile *tiles, int n_tiles, float *mean,
-                      float *spread) {
+                      float *spread, const float *noise) {
   const float kthr = h->fp64_kappa > 0 ? (float)h->fp64_kappa : 0.f;
   int *queue = kthr > 0.f ? h->counters + 4 + cls : nullptr;
   int2 *wl = h->worklist + (size_t)cls * h->n_pts_total;
@@ -1108,9 +1119,9 @@ cudaError_t launch_mp(letkf_ctx *h, int cls, const LkTile *tiles, int n_tiles, f
 #define LK_CASE(id, ti, tj)                                                                   \
   case id:                                                                                    \
     return split ? launch_shape<MP, ti, tj, true>(h, tiles, n_tiles, mean, spread, kthr, queue, \
-                                                  wl)                                         \
+                                                  wl, noise)                                  \
                  : launch_shape<MP, ti, tj, false>(h, tiles, n_tiles, mean, spread, kthr, queue, \
-                                                   wl);
+                                                   wl, noise);
     LK_FOR_SHAPES(LK_CASE)
 #undef LK_CASE
   }
@@ -1135,7 +1146,7 @@ cudaError_t launch_basis_shape(letkf_ctx *h, int cls) {
                          h->tiles[cls], (float *)nullptr, (float *)nullptr, (float)h->tol32,
                          (float)h->stop32, h->max_sweeps, 0.f, h->counters,
                          lk_series64(h) ? h->counters + 4 + cls : (int *)nullptr,
-                         (int2 *)nullptr, 1, (const float2 *)nullptr, 0);
+                         (int2 *)nullptr, 1, (const float2 *)nullptr, 0, (const float *)nullptr);
   }
 }
 
@@ -1191,20 +1202,21 @@ cudaError_t setup_mp(letkf_ctx *h) {
 // Class 0: MP = 16; class 1: tiles of instances with m <= 24 first (tile_split
 // of them, none in the row-split form) on MP = 24, then MP = 32; class 2: tiles
 // of MP = 64 instances first, then MP = 48.
-cudaError_t lk_launch_pair(letkf_ctx *h, int cls, void *mean, void *spread) {
+cudaError_t lk_launch_pair(letkf_ctx *h, int cls, void *mean, void *spread, const LkCycle &cy) {
+  const float *nz = static_cast<const float *>(cy.noise);
   float *mo = static_cast<float *>(mean), *so = static_cast<float *>(spread);
-  if (cls == 0) return launch_mp<16>(h, 0, h->tiles[0], h->n_tiles[0], mo, so);
+  if (cls == 0) return launch_mp<16>(h, 0, h->tiles[0], h->n_tiles[0], mo, so, nz);
   if (cls == 1) {
     const int n24 = h->tile_split[1];
-    cudaError_t e = launch_mp<24>(h, 1, h->tiles[1], n24, mo, so);
+    cudaError_t e = launch_mp<24>(h, 1, h->tiles[1], n24, mo, so, nz);
     if (e == cudaSuccess)
-      e = launch_mp<32>(h, 1, h->tiles[1] + n24, h->n_tiles[1] - n24, mo, so);
+      e = launch_mp<32>(h, 1, h->tiles[1] + n24, h->n_tiles[1] - n24, mo, so, nz);
     return e;
   }
   const int split = h->tile_split[2];
-  cudaError_t e = launch_mp<64>(h, 2, h->tiles[2], split, mo, so);
+  cudaError_t e = launch_mp<64>(h, 2, h->tiles[2], split, mo, so, nz);
   if (e == cudaSuccess)
-    e = launch_mp<48>(h, 2, h->tiles[2] + split, h->n_tiles[2] - split, mo, so);
+    e = launch_mp<48>(h, 2, h->tiles[2] + split, h->n_tiles[2] - split, mo, so, nz);
   return e;
 }
 

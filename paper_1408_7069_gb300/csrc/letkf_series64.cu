@@ -396,10 +396,12 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
     series64_kernel(const LkInst *__restrict__ insts, const int2 *__restrict__ items,
                     double *__restrict__ mean, double *__restrict__ spread,
                     const float4 *__restrict__ cheb, int *__restrict__ counters,
-                    int *__restrict__ queue, int2 *__restrict__ worklist) {
+                    int *__restrict__ queue, int2 *__restrict__ worklist,
+                    const double *__restrict__ noise) {
   using C = S64<MPD>;
   extern __shared__ __align__(16) double sm64[];
   lk_pdl_wait();
+  lk_pdl_trigger();
   const int2 it = items[blockIdx.x];
   const LkInst &I = insts[it.x];
   const int m = I.m, w = I.w;
@@ -475,7 +477,20 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
     const int ex = sm.redi()[2 + wv];
     const Df a = lane < m ? ld_df(sm.xs[wv * MPD + lane]) : df(0.f);
     const double y = sm.red64()[8 + wv] + df_to_double(p, ex + ed);
-    if (lane < m) xrow[(size_t)wv * m + lane] = y + df_to_double(df_mul(al.rt, a), ex + al.re);
+    double fc = 0.0;
+    if (lane < m) {                                  // with noise, the forecast instead
+      const double xa = y + df_to_double(df_mul(al.rt, a), ex + al.re);
+      if (!noise) xrow[(size_t)wv * m + lane] = xa;
+      if (noise && wv == 0) {
+        xrow[m + lane] = xa;
+        fc = lk_ar1<double>(I, noise, pid, lane, xa);
+        xrow[lane] = fc;
+      }
+    }
+    if (noise && wv == 0 && I.dm) {
+      fc = lk_warp_sum(fc);
+      if (lane == 0) static_cast<double *>(I.pmean)[pid] = fc / m;
+    }
     // their mean and spread (|a| < 8: at most that of the anomalies, below 1 each)
     const Df rm = df_rcp(df((float)m));
     const Df am = df_mul(df_redux(a, 3), rm);
@@ -891,7 +906,7 @@ cudaError_t launch_adj64(letkf_ctx *h, const LkAdjArgs &a) {
 }
 
 template <int MPD>
-cudaError_t launch_series64(letkf_ctx *h, int cls, void *mean, void *spread) {
+cudaError_t launch_series64(letkf_ctx *h, int cls, void *mean, void *spread, const void *noise) {
   size_t need = 0;
   for (const LkInst &I : h->inst)
     if (I.m <= MPD && I.m > MPD - 8) {
@@ -902,7 +917,7 @@ cudaError_t launch_series64(letkf_ctx *h, int cls, void *mean, void *spread) {
   return lk_launch_pdl(series64_kernel<MPD>, (unsigned)h->n_pts_total, S64<MPD>::NT, need,
                        h->stream, h->d_inst, h->node_items, (double *)mean, (double *)spread,
                        (const float4 *)h->cheb64, h->counters, h->counters + 4 + cls,
-                       h->worklist + (size_t)cls * h->n_pts_total);
+                       h->worklist + (size_t)cls * h->n_pts_total, (const double *)noise);
 }
 
 template <int MPD>
@@ -919,13 +934,13 @@ cudaError_t setup_series64(int w) {
 
 }  // namespace
 
-cudaError_t lk_launch_series64(letkf_ctx *h, int cls, void *mean, void *spread) {
+cudaError_t lk_launch_series64(letkf_ctx *h, int cls, void *mean, void *spread, const LkCycle &cy) {
   if (cls == 0) {
-    cudaError_t e = launch_series64<8>(h, 0, mean, spread);
-    return e == cudaSuccess ? launch_series64<16>(h, 0, mean, spread) : e;
+    cudaError_t e = launch_series64<8>(h, 0, mean, spread, cy.noise);
+    return e == cudaSuccess ? launch_series64<16>(h, 0, mean, spread, cy.noise) : e;
   }
-  cudaError_t e = launch_series64<24>(h, 1, mean, spread);
-  return e == cudaSuccess ? launch_series64<32>(h, 1, mean, spread) : e;
+  cudaError_t e = launch_series64<24>(h, 1, mean, spread, cy.noise);
+  return e == cudaSuccess ? launch_series64<32>(h, 1, mean, spread, cy.noise) : e;
 }
 
 cudaError_t lk_launch_adj_series64(letkf_ctx *h, const LkAdjArgs &a) {

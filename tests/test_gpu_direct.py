@@ -378,3 +378,36 @@ def test_ill_conditioned_nodes_match_oracle(nsub, m, window, taper, scale):
         assert rel(anoms(Xa), anoms(ref[0])) <= 1e-3
     Xj, mj, sj, _ = analyse(mask, X, y, m, window, taper, fp64_kappa=1.0000001, max_sweeps=30)
     assert rms(Xa - Xj) <= 4 * 2.0 ** -24 * rms(X) + 1e-6 * rms(anoms(ref[0]))
+
+
+# ---------------------------------------------------------------------------
+# The forecast inside the analysis (lk_launch_cycle): letkf_run against the same frames
+# by letkf_analyze and letkf_forecast, whose kernels are separate. The same bits.
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("use_graph", [True, False], ids=["graph", "stream"])
+@pytest.mark.parametrize("m,precision,scale,kw",
+                         [(10, 0, 0.1, {}), (20, 0, 0.1, {}), (32, 0, 3.0, {}),
+                          (17, 0, 30.0, {}), (20, 0, 3.0, dict(max_sweeps=20)), (40, 0, 3.0, {}),
+                          (64, 0, 0.1, {}), (24, 0, 0.1, dict(fp64_kappa=-1.0)),
+                          (10, 1, 0.1, {}), (24, 1, 3.0, {})])
+def test_run_equals_analyses_and_forecasts(m, precision, scale, kw, use_graph):
+    mask, geom, X, y, _ = problem(6, m, 3, 1, scale)
+    dt = np.float64 if precision else np.float32
+    frames, rng = 3, np.random.default_rng(m)
+    ys = torch.from_numpy(rng.standard_normal((frames, geom.p)).astype(dt)).cuda()
+    bank = rng.standard_normal((2, 16, 16)).astype(np.float32)
+    f = Letkf(mask, m=m, window=3, taper=1, rho=RHO, sigma2=SIGMA2, a_ar1=0.99, noise_std=0.1,
+              precision=precision, seed=3, bank=bank, **kw)
+    X = torch.from_numpy(X.astype(dt)).cuda()
+    f.set_state(X)
+    f.run(frames, ys, use_graph=use_graph)
+    f.sync()
+    a = f.get_state()
+    f.set_state(X)
+    f.set_frame(0)
+    for k in range(frames):
+        f.analyze(ys[k], outputs=False)
+        f.forecast()
+    f.sync()
+    assert torch.equal(a, f.get_state())
+    f.close()
