@@ -319,7 +319,7 @@ letkf_status letkf_grad(letkf_t h, int32_t frames, const void *y_seq_dev, const 
  * warp, tiles of at most 8 nodes). On FP32 handles a tile
  * holds whole warps of nodes (a multiple of 4 nodes in class 0, of 2 in class
  * 1); a shape a class cannot take gives LETKF_ERR_ARG. New handles start at
- * shape 0 (2 x 4). letkf_set_tile_shape
+ * shape 0 (2 x 4) in classes 0 and 1 and at shape 2 (2 x 2) in class 2. letkf_set_tile_shape
  * selects a shape for one class; letkf_autotune times every allowed shape for every class
  * present on the handle's current ensemble with slopes y_dev (reps timed
  * analyses of that class's nodes each, state restored afterwards; tune on a

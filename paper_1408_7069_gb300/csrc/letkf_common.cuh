@@ -16,8 +16,13 @@ enum : int {
   LK_BIT_TIMEOUT = 4,
 };
 
-// Default node tile of one analysis CTA (TI x TJ nodes, one warp each); the
-// autotuner may choose another of the compiled shapes.
+// Default node tile of one analysis CTA (TI x TJ nodes); the autotuner may choose
+// another of the compiled shapes. The wide class, a warp per node and 170 to 240 registers
+// per thread, takes 2 x 2 (shape 2): eight warps of a 2 x 4 tile fill an SM's registers
+// alone, of 2 x 2 tiles three fit for 48 columns. Measured on one GB300, four frames
+// 2 x 4 -> 2 x 2: 80 x 80, m = 48 417 -> 355 us, m = 40 417 -> 351, m = 64 474 -> 440; 16 x 16,
+// m = 56 104 -> 94; 48 systems 2.68 -> 2.36 ms. (The halo cells a node stages grow with it, which
+// at a window of 13 still costs less than it gives: 40 x 40, m = 64 517 -> 442.)
 constexpr int LK_TILE_I = 2;
 constexpr int LK_TILE_J = 4;
 // Padding of the slope-anomaly grid: tiles up to this many nodes per side keep
@@ -135,7 +140,7 @@ struct letkf_ctx {
   int2 *node_items = nullptr;       // [n_pts_total] (inst, point)
   LkTile *tiles[3] = {nullptr, nullptr, nullptr};   // per width class 16 / 32 / 64
   int n_tiles[3] = {0, 0, 0};
-  int tile_shape[3] = {0, 0, 0};    // index into the compiled tile shapes, per class
+  int tile_shape[3] = {0, 0, 2};    // index into the compiled tile shapes, per class
   int tile_split[3] = {0, 0, 0};    // class 2: leading tiles of MP = 64 instances (MP = 48 after)
   int row_split[3] = {1, 1, 1};     // 2: each column's rows on two lanes (classes 0 and 1, FP32)
   int fp64_warm = 1;                // FP64 handles: FP32 basis pass, then the FP64 sweep from it
