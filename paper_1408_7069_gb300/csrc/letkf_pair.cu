@@ -85,7 +85,7 @@ __host__ __device__ PairLayout pair_layout(int w) {
   const size_t ncell = (size_t)(TI + w - 1) * (TJ + w - 1);
   L.dh = align16(ncell * C::CELLF * sizeof(float));
   L.tap = align16(L.dh + ncell * 2 * sizeof(float));
-  L.scr = align16(L.tap + (size_t)w * w * sizeof(float));
+  L.scr = align16(L.tap + ((size_t)w * w + 1) * sizeof(float2));
   L.total = L.scr + (size_t)TI * TJ * C::NODE_SCR * sizeof(float);
   return L;
 }
@@ -243,7 +243,33 @@ __device__ __forceinline__ float2 reduce_scatter(float2 (&v)[GL], int li) {
   return v[0];
 }
 
-// Stages the tile's halo (slope anomalies and innovations) and the taper table.
+// The window's cells inside the taper's support, by the CTA's last warp: (weight, cell of the
+// halo from the node's corner), their number in front.
+template <typename S>
+__device__ __forceinline__ void support_list(const S *__restrict__ taper, int w, int HJ, float *tap) {
+  if ((threadIdx.x >> 5) != (blockDim.x >> 5) - 1) return;
+  float2 *list = reinterpret_cast<float2 *>(tap) + 1;
+  const int lane = threadIdx.x & 31, wc = w * w;
+  int n = 0;
+  for (int e0 = 0; e0 < wc; e0 += 64) {
+    float t[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) t[u] = e0 + 32 * u + lane < wc ? (float)taper[e0 + 32 * u + lane] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = e0 + 32 * u + lane, ds = e / w;
+      const unsigned b = __ballot_sync(FULL, t[u] != 0.f);
+      if (t[u] != 0.f)
+        list[n + __popc(b & ((1u << lane) - 1u))] =
+            make_float2(t[u], __int_as_float(ds * HJ + e - ds * w));
+      n += __popc(b);
+    }
+  }
+  if (lane == 0) reinterpret_cast<int *>(tap)[0] = n;
+}
+
+// Stages the tile's halo (slope anomalies and innovations) and the taper table, or (LIST) the
+// list of the cells of its support.
 // S: the handle's storage type (double on FP64 handles, whose FP32 basis pass
 // rounds the window to float here). FP32 goes by cp.async, every copy of a CTA in flight
 // at once, a power of two of lanes per slope row so that no index is divided by the
@@ -260,7 +286,7 @@ __device__ __forceinline__ void cp_async4(float *dst, const float *src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
                "l"(src) : "memory");
 }
-template <int MP, int TI, int TJ, typename S = float>
+template <int MP, int TI, int TJ, typename S = float, bool LIST = true>
 __device__ __forceinline__ void stage_pair_tile(const LkInst &I, int i0, int j0, float *halo,
                                                 float *dh, float *tap) {
   using C = PairCfg<MP>;
@@ -306,7 +332,10 @@ __device__ __forceinline__ void stage_pair_tile(const LkInst &I, int i0, int j0,
     }
     for (int e = threadIdx.x; e < ncell * 2; e += blockDim.x)
       cp_async4(dh + e, dp + source(e >> 1) * 2 + (e & 1));
-    for (int e = threadIdx.x; e < w * w; e += blockDim.x) cp_async4(tap + e, taper + e);
+    if constexpr (LIST)
+      support_list(taper, w, HJ, tap);
+    else
+      for (int e = threadIdx.x; e < w * w; e += blockDim.x) cp_async4(tap + e, taper + e);
     asm volatile("cp.async.wait_all;" ::: "memory");
   } else {
     for (int e = threadIdx.x; e < ncell * C::CELLF; e += blockDim.x) {
@@ -328,7 +357,10 @@ __device__ __forceinline__ void stage_pair_tile(const LkInst &I, int i0, int j0,
       const size_t src = (size_t)(i0 + hi) * I.gs_cols + (j0 + hj);
       dh[e] = (float)dp[src * 2 + (e & 1)];
     }
-    for (int e = threadIdx.x; e < w * w; e += blockDim.x) tap[e] = (float)taper[e];
+    if constexpr (LIST)
+      support_list(taper, w, HJ, tap);
+    else
+      for (int e = threadIdx.x; e < w * w; e += blockDim.x) tap[e] = (float)taper[e];
   }
 }
 
@@ -486,30 +518,30 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
   const float *hwin = halo + (size_t)(ti * HJ + tj) * C::CELLF;
   const float *dwin = dh + (size_t)(ti * HJ + tj) * 2;
   const int lr = live ? li : 0;                      // idle lanes read row pair 0, then drop it
-  for (int ds = 0; ds < w; ++ds) {
-    for (int dt = 0; dt < w; ++dt) {
-      const int cell = ds * HJ + dt;
-      const float tw = tap[ds * w + dt];
-      if (tw == 0.f) continue;                       // outside the taper's support
+  const int n_cell = reinterpret_cast<const int *>(tap)[0];
+  const float2 *list = reinterpret_cast<const float2 *>(tap) + 1;
+  for (int q = 0; q < n_cell; ++q) {
+    const float2 wc = list[q];
+    const float tw = wc.x;
+    const int cell = __float_as_int(wc.y);
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const float *yv = hwin + (size_t)cell * C::CELLF + c * MP;
-        const float2 yl = reinterpret_cast<const float2 *>(yv)[lr];
-        const float cy0 = tw * yl.x, cy1 = tw * yl.y;
-        diag = fmaf(cy0, yl.x, fmaf(cy1, yl.y, diag));
-        const float dj = dwin[cell * 2 + c];
-        cd0 = fmaf(cy0, dj, cd0);
-        cd1 = fmaf(cy1, dj, cd1);
-        const float2 c0 = f2(cy0), c1 = f2(cy1);
+    for (int c = 0; c < 2; ++c) {
+      const float *yv = hwin + (size_t)cell * C::CELLF + c * MP;
+      const float2 yl = reinterpret_cast<const float2 *>(yv)[lr];
+      const float cy0 = tw * yl.x, cy1 = tw * yl.y;
+      diag = fmaf(cy0, yl.x, fmaf(cy1, yl.y, diag));
+      const float dj = dwin[cell * 2 + c];
+      cd0 = fmaf(cy0, dj, cd0);
+      cd1 = fmaf(cy1, dj, cd1);
+      const float2 c0 = f2(cy0), c1 = f2(cy1);
 #pragma unroll
-        for (int k = 0; k < K2 / 2; ++k) {
-          const float4 y4 = reinterpret_cast<const float4 *>(yv)[k];
-          const float2 ya = make_float2(y4.x, y4.y), yb = make_float2(y4.z, y4.w);
-          P[2 * k] = fma2(c0, ya, P[2 * k]);
-          P[2 * k + 1] = fma2(c0, yb, P[2 * k + 1]);
-          Q[2 * k] = fma2(c1, ya, Q[2 * k]);
-          Q[2 * k + 1] = fma2(c1, yb, Q[2 * k + 1]);
-        }
+      for (int k = 0; k < K2 / 2; ++k) {
+        const float4 y4 = reinterpret_cast<const float4 *>(yv)[k];
+        const float2 ya = make_float2(y4.x, y4.y), yb = make_float2(y4.z, y4.w);
+        P[2 * k] = fma2(c0, ya, P[2 * k]);
+        P[2 * k + 1] = fma2(c0, yb, P[2 * k + 1]);
+        Q[2 * k] = fma2(c1, ya, Q[2 * k]);
+        Q[2 * k + 1] = fma2(c1, yb, Q[2 * k + 1]);
       }
     }
   }
@@ -847,7 +879,7 @@ __global__ void __launch_bounds__(SplitLaunch<MP, TI, TJ>::threads, SplitLaunch<
   float *halo = reinterpret_cast<float *>(smem);
   float *dh = reinterpret_cast<float *>(smem + Ly.dh);
   float *tap = reinterpret_cast<float *>(smem + Ly.tap);
-  stage_pair_tile<MP, TI, TJ>(I, tl.i0, tl.j0, halo, dh, tap);
+  stage_pair_tile<MP, TI, TJ, float, false>(I, tl.i0, tl.j0, halo, dh, tap);
   __syncthreads();
   LK_PHASE_STAMP(ph1);
 
