@@ -85,7 +85,7 @@ __host__ __device__ PairLayout pair_layout(int w) {
   const size_t ncell = (size_t)(TI + w - 1) * (TJ + w - 1);
   L.dh = align16(ncell * C::CELLF * sizeof(float));
   L.tap = align16(L.dh + ncell * 2 * sizeof(float));
-  L.scr = align16(L.tap + ((size_t)w * w + 1) * sizeof(float2));
+  L.scr = align16(L.tap + ((size_t)w * w + 2) * sizeof(float2));
   L.total = L.scr + (size_t)TI * TJ * C::NODE_SCR * sizeof(float);
   return L;
 }
@@ -520,8 +520,10 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
   const int lr = live ? li : 0;                      // idle lanes read row pair 0, then drop it
   const int n_cell = reinterpret_cast<const int *>(tap)[0];
   const float2 *list = reinterpret_cast<const float2 *>(tap) + 1;
+  float2 next = list[0];                             // (read a cell ahead; one pair of slack)
   for (int q = 0; q < n_cell; ++q) {
-    const float2 wc = list[q];
+    const float2 wc = next;
+    next = list[q + 1];
     const float tw = wc.x;
     const int cell = __float_as_int(wc.y);
 #pragma unroll
