@@ -338,7 +338,7 @@ constexpr size_t NA_OFF_PID = al256(NA_OFF_DP + NA_CELLS * 2 * sizeof(float));
 constexpr size_t NA_OFF_SAPS = al256(NA_OFF_PID + (size_t)NA_NN * NA_NN * sizeof(int));
 constexpr size_t NA_OFF_PTS = al256(NA_OFF_SAPS + (size_t)NA_MAX_NSUB * NA_MAX_NSUB * sizeof(int2));
 constexpr size_t NA_OFF_OBS = al256(NA_OFF_PTS + (size_t)NA_NN * NA_NN * sizeof(int2));
-constexpr size_t NA_OFF_TILES = al256(NA_OFF_OBS + (size_t)NA_MAX_NSUB * NA_MAX_NSUB * sizeof(int2));
+constexpr size_t NA_OFF_TILES = al256(NA_OFF_OBS + (size_t)NA_MAX_NSUB * NA_MAX_NSUB * sizeof(LkObsItem));
 constexpr size_t NA_OFF_TAPER = al256(NA_OFF_TILES + (size_t)NA_MAX_TILES * sizeof(LkTile));
 constexpr size_t NA_OFF_INST = al256(NA_OFF_TAPER + (size_t)NA_MAX_W * NA_MAX_W * sizeof(float));
 constexpr size_t NA_OFF_COUNTERS = al256(NA_OFF_INST + sizeof(LkInst));
@@ -353,7 +353,7 @@ std::mutex g_na_mutex;
 int g_na_pid[NA_NN * NA_NN];
 int2 g_na_saps[NA_MAX_NSUB * NA_MAX_NSUB];
 int2 g_na_pts[NA_NN * NA_NN];
-int2 g_na_obs[NA_MAX_NSUB * NA_MAX_NSUB];
+LkObsItem g_na_obs[NA_MAX_NSUB * NA_MAX_NSUB];
 LkTile g_na_tiles[NA_MAX_TILES];
 float g_na_taper[NA_MAX_W * NA_MAX_W];
 void *g_na_addr[256];          // scratch address per device, set once
@@ -483,7 +483,6 @@ extern "C" letkf_status letkf_analyze_noalloc(const letkf_config *cfg, void *X_d
   for (int s = 0; s < ns; ++s)
     for (int t = 0; t < ns; ++t)
       if (c.subap_mask[(size_t)s * ns + t]) {
-        g_na_obs[n_sap] = make_int2(0, n_sap);
         g_na_saps[n_sap++] = make_int2(s, t);
         g_na_pid[s * nn + t] = g_na_pid[(s + 1) * nn + t] = 0;
         g_na_pid[s * nn + t + 1] = g_na_pid[(s + 1) * nn + t + 1] = 0;
@@ -518,6 +517,11 @@ extern "C" letkf_status letkf_analyze_noalloc(const letkf_config *cfg, void *X_d
       g_na_taper[ds * w + dt] = (float)(tau / c.sigma2);
     }
   const int gs = ((nn + LK_TILE_MAX - 1) / LK_TILE_MAX) * LK_TILE_MAX + w;
+  for (int q = 0; q < n_sap; ++q) {
+    const int s = g_na_saps[q].x, t = g_na_saps[q].y;
+    const int *p = g_na_pid + s * nn + t;
+    g_na_obs[q] = LkObsItem{0, q, (s + hw) * gs + t + hw, 0, p[0], p[nn], p[1], p[nn + 1]};
+  }
   LkInst inst;
   memset(&inst, 0, sizeof(inst));
   inst.nsub = ns;
@@ -551,7 +555,7 @@ extern "C" letkf_status letkf_analyze_noalloc(const letkf_config *cfg, void *X_d
   } copies[] = {{NA_OFF_PID, g_na_pid, (size_t)nn * nn * sizeof(int)},
                 {NA_OFF_SAPS, g_na_saps, (size_t)n_sap * sizeof(int2)},
                 {NA_OFF_PTS, g_na_pts, (size_t)n_pts * sizeof(int2)},
-                {NA_OFF_OBS, g_na_obs, (size_t)n_sap * sizeof(int2)},
+                {NA_OFF_OBS, g_na_obs, (size_t)n_sap * sizeof(LkObsItem)},
                 {NA_OFF_TILES, g_na_tiles, (size_t)n_tiles * sizeof(LkTile)},
                 {NA_OFF_TAPER, g_na_taper, (size_t)w * w * sizeof(float)},
                 {NA_OFF_INST, &inst, sizeof(LkInst)}};
@@ -568,7 +572,7 @@ extern "C" letkf_status letkf_analyze_noalloc(const letkf_config *cfg, void *X_d
   tmp.precision = 0;
   tmp.n_inst = 1;
   tmp.d_inst = reinterpret_cast<LkInst *>(base + NA_OFF_INST);
-  tmp.obs_items = reinterpret_cast<int2 *>(base + NA_OFF_OBS);
+  tmp.obs_items = reinterpret_cast<LkObsItem *>(base + NA_OFF_OBS);
   tmp.sap_total = n_sap;
   tmp.p_total = 2 * n_sap;
   tmp.counters = reinterpret_cast<int *>(base + NA_OFF_COUNTERS);

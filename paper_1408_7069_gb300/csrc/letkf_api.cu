@@ -347,7 +347,7 @@ letkf_status build_handle(const letkf_config *cfgs, int n, void *stream, letkf_t
   LK_TRY(dalloc(h, &h->noise_pre, (size_t)h->noise_total * h->rsz));
   LK_TRY(dalloc(h, &h->tickets, (size_t)(n + 1) * sizeof(int)));
   LK_TRY(dalloc(h, &h->d_inst, (size_t)n * sizeof(LkInst)));
-  LK_TRY(dalloc(h, &h->obs_items, h->sap_total * sizeof(int2)));
+  LK_TRY(dalloc(h, &h->obs_items, h->sap_total * sizeof(LkObsItem)));
   LK_TRY(dalloc(h, &h->node_items, h->n_pts_total * sizeof(int2)));
   if (h->stream) {
     cudaError_t es = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking);
@@ -358,7 +358,8 @@ letkf_status build_handle(const letkf_config *cfgs, int n, void *stream, letkf_t
   }
   // ---- slice buffers, upload tables ----
   size_t o_ybp = 0, o_dp = 0, o_tap = 0, o_pid = 0, o_basis = 0, o_bank = 0, o_pts = 0, o_sap = 0;
-  std::vector<int2> obs_items, node_items;
+  std::vector<LkObsItem> obs_items;
+  std::vector<int2> node_items;
   std::vector<std::vector<int>> pids(n);
   for (int k = 0; k < n; ++k) {
     const letkf_config &c = cfgs[k];
@@ -392,7 +393,11 @@ letkf_status build_handle(const letkf_config *cfgs, int n, void *stream, letkf_t
                     (size_t)c.bank_B * c.bank_G * c.bank_G * sizeof(float)));
       o_bank += (size_t)c.bank_B * c.bank_G * c.bank_G;
     }
-    for (int q = 0; q < I.n_sap; ++q) obs_items.push_back(make_int2(k, q));
+    for (int q = 0; q < I.n_sap; ++q) {
+      const int s = G.saps[q].x, t = G.saps[q].y, nn = c.nsub + 1;
+      const int *p = G.pid.data() + (size_t)s * nn + t;
+      obs_items.push_back(LkObsItem{k, q, (s + I.h) * I.gs_cols + t + I.h, 0, p[0], p[nn], p[1], p[nn + 1]});
+    }
     for (int q = 0; q < I.n_pts; ++q) node_items.push_back(make_int2(k, q));
     for (size_t q = 0; q < G.pts.size(); ++q) {
       h->pts_host.push_back(G.pts[q].x);
@@ -409,7 +414,7 @@ letkf_status build_handle(const letkf_config *cfgs, int n, void *stream, letkf_t
     o_sap += G.saps.size();
   }
   LK_TRY(upload(h, h->d_inst, h->inst.data(), (size_t)n * sizeof(LkInst)));
-  LK_TRY(upload(h, h->obs_items, obs_items.data(), obs_items.size() * sizeof(int2)));
+  LK_TRY(upload(h, h->obs_items, obs_items.data(), obs_items.size() * sizeof(LkObsItem)));
   LK_TRY(upload(h, h->node_items, node_items.data(), node_items.size() * sizeof(int2)));
   cudaError_t e = cudaMemset(h->X, 0, h->state_total * h->rsz);
   if (e == cudaSuccess) e = cudaMemset(h->Ybp, 0, n_ybp * h->rsz);

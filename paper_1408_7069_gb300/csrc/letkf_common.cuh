@@ -107,6 +107,13 @@ struct LkInst {
 };
 
 // Work items.
+// One subaperture of the observation kernel: instance, index, cell of the padded grid, node
+// ids of its corners (0,0), (1,0), (0,1), (1,1).
+struct alignas(16) LkObsItem {
+  int inst, k, cell, pad;
+  int q00, q10, q01, q11;
+};
+
 struct LkTile {             // one analysis CTA: instance, tile origin (node coordinates)
   int inst, i0, j0, cost;
 };
@@ -136,7 +143,7 @@ struct letkf_ctx {
   long long sap_total = 0;
 
   // work lists (device)
-  int2 *obs_items = nullptr;        // [sap_total] (inst, subap)
+  LkObsItem *obs_items = nullptr;   // [sap_total]
   int2 *node_items = nullptr;       // [n_pts_total] (inst, point)
   LkTile *tiles[3] = {nullptr, nullptr, nullptr};   // per width class 16 / 32 / 64
   int n_tiles[3] = {0, 0, 0};
