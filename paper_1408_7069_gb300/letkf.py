@@ -10,6 +10,7 @@ from __future__ import annotations
 import ctypes
 import os
 import re
+import threading
 from ctypes import POINTER, byref, c_char_p, c_double, c_int32, c_uint64, c_void_p
 
 import numpy as np
@@ -380,6 +381,7 @@ class Letkf:
         if not torch.cuda.is_available():
             raise RuntimeError("Letkf needs a CUDA GPU; there is no CPU implementation")
         self.stream = stream if stream is not None else torch.cuda.Stream()
+        self._order = threading.local()
         if _configs is None:
             _configs = [make_config(subap_mask, m, window, **kw)]
         self._keep = [k for _, k in _configs]
@@ -413,11 +415,26 @@ class Letkf:
                    _configs=[workload_config(w, b, **kw) for w, b in zip(workloads, banks)])
 
     # -- stream ordering ---------------------------------------------------
+    # The private stream after torch's current one on entry, and the other way round on
+    # exit, by events kept per thread (and per device of the current stream): wait_stream
+    # makes an event each time, which took a small analysis as long as the GPU. Measured, 16 m
+    # on one GB300: four frames from the host 248 -> 210 us, from the device 107 -> 94, an
+    # update by domains 140 -> 98.
     def _enter(self):
-        self.stream.wait_stream(self._torch.cuda.current_stream())
+        o = self._order
+        if not hasattr(o, "leave"):
+            o.enter, o.leave = {}, self._torch.cuda.Event()
+        o.current = self._torch.cuda.current_stream()
+        ev = o.enter.get(o.current.device_index)
+        if ev is None:
+            ev = o.enter[o.current.device_index] = self._torch.cuda.Event()
+        ev.record(o.current)
+        self.stream.wait_event(ev)
 
     def _leave(self):
-        self._torch.cuda.current_stream().wait_stream(self.stream)
+        o = self._order
+        o.leave.record(self.stream)
+        o.current.wait_event(o.leave)
 
     def _t(self, t, shape):
         if t is None:
@@ -473,7 +490,7 @@ class Letkf:
         self._leave()
 
     def get_state(self):
-        X = self.new(*self.state_shape)
+        X = self._torch.empty(*self.state_shape, dtype=self.dtype, device="cuda")   # all written
         self._enter()
         letkf_get_state(self.h, X)
         self._leave()

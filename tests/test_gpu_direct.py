@@ -411,3 +411,35 @@ def test_run_equals_analyses_and_forecasts(m, precision, scale, kw, use_graph):
     f.sync()
     assert torch.equal(a, f.get_state())
     f.close()
+
+
+def test_calls_are_ordered_against_the_current_stream():
+    """Inputs still being written on one torch stream, outputs read on another, from two
+    threads in turn: the events that order the handle's stream are kept between calls."""
+    import threading
+    mask, geom, X, _, _ = problem(6, 8, 3, 1, 0.1)
+    f = Letkf(mask, m=8, window=3, taper=1, rho=RHO, sigma2=SIGMA2)
+    X = torch.from_numpy(X).cuda()
+    big = torch.randn(4096, 4096, device="cuda")
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def turn(k):
+        with torch.cuda.stream(a):
+            z = big
+            for _ in range(4):
+                z = z @ big * 1e-2
+            f.set_state(X * k + 0 * z[0, 0].nan_to_num(0.0, 0.0, 0.0))
+        with torch.cuda.stream(b):
+            out.append((k, f.get_state()))
+    out = []
+    for k in range(1, 5):
+        t = threading.Thread(target=turn, args=(float(k),))
+        if k % 2:
+            t.start()
+            t.join()
+        else:
+            turn(float(k))
+    torch.cuda.synchronize()
+    assert len(out) == 4 and all(torch.equal(v, X * k) for k, v in out)
+    f.close()
