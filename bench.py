@@ -370,7 +370,7 @@ def domains_arm(torch, L, K: int = 200, Wm: int = 20):
     21 x 21 partition (373 domains), m = 101, n_d <= 32, p_d <= 128, with the
     differential-piston least squares; and the global ETKF (Section 3.1.1:
     partition 1, all 1624 slopes) of the 16 m telescope at m = 101. Per frame:
-    the update (one CTA per domain and the piston kernels, or the global
+    the update (the domains' series and the piston kernels, or the global
     pipeline) timed with CUDA events; for the partitions also the whole
     closed-loop frame (residual, observation, update, forecast) as one launch
     of K frames with in-graph stamps. The global update (m = 101 and 626) is
@@ -438,7 +438,7 @@ def domains_arm(torch, L, K: int = 200, Wm: int = 20):
                           "frame_us_p99": percentile(list(fus), 99),
                           "frames_per_s": 1e6 / float(np.mean(fus)),
                           "resvar_last": float(resv[-1].item())})
-            entry["launch"] = ("update: one CTA per domain + piston solve + piston apply; "
+            entry["launch"] = ("update: series over the domains' row parts + piston sums + piston apply; "
                                "frames: letkf_run_graph (one launch, in-graph stamps)")
         elif w.m <= 64:
             entry["launch"] = ("update: compensated-FP32 Gram (split over slope chunks), one-CTA FP32 "
@@ -446,8 +446,8 @@ def domains_arm(torch, L, K: int = 200, Wm: int = 20):
                                "timed on the prior draw")
         else:
             entry["launch"] = ("update: compensated-FP32 Gram (split over slope chunks), coupled "
-                               "Newton-Schulz iterations on FP32 matrix products (at most 40, "
-                               "converged ones skipped), FP64-refined mean solve, "
+                               "Newton-Schulz iterations, scaled, on FP32 matrix products in one "
+                               "cooperative kernel, FP64-refined mean solve, "
                                "matrix-product apply; timed on the prior draw")
         entry["paper_context"] = ("Section 5.3, Table 2 (2 x Xeon E5-2680 v2): update of one "
                                   "domain 0.94 ms on one core; full 16 m cycle 1.18 ms with "
@@ -582,7 +582,7 @@ def phase_worker(args):
     L.letkf_sync(h)
     c = L.letkf_phase_clocks()
     f.close()
-    names = ["halo_staging", "gram_and_kappa", "jacobi_sweeps", "transform_and_apply"]
+    names = ["halo_staging", "gram_and_kappa", "series_or_sweeps", "apply"]
     tot = sum(c[:4])
     print(json.dumps({"workload": w.name, "analyses": K, "warps_per_analysis": c[4] / K,
                       "cycles_per_warp": {n: c[i] / c[4] for i, n in enumerate(names)},
@@ -643,6 +643,22 @@ def phase_split(args):
     r = subprocess.run([sys.executable, os.path.abspath(__file__), worker, "--steps",
                         str(args.steps), "--warmup", str(args.warmup)], env=env, timeout=900)
     return r.returncode
+
+
+def mean_products(w, inp, X, n=64):
+    """Mean number of series products per node (opcount.chebyshev_products) over n nodes of
+    the ensemble X, from the oracle's window Grams."""
+    import numpy as np
+    import oracle
+    from paper_1408_7069_gb300 import opcount
+    geom = oracle.build_geometry(inp.subap_mask, w.window, w.taper, w.loc_len)
+    _, _, Yb, _ = oracle.observe(geom, X.astype(np.float64))
+    alpha, out = (w.m - 1) / w.rho, []
+    for q in np.linspace(0, geom.n_pts - 1, n).astype(int):
+        y = Yb[geom.win_idx[q]]
+        G = (y * (np.asarray(geom.win_tau[q]) / w.sigma2)[:, None]).T @ y
+        out.append(opcount.chebyshev_products(float(np.linalg.norm(G)) / alpha))
+    return float(np.mean(out))
 
 
 # --------------------------------------------------------------------------- CPU oracle
@@ -891,6 +907,7 @@ def gpu_arm(args):
     torch.cuda.synchronize()
     L.letkf_sync(h)
     nfp64, sweeps, total_sweeps = L.letkf_stats(h)
+    X_last = f.get_state().cpu().numpy()
     ana_ms = [e[0].elapsed_time(e[1]) for e in eva]
 
     reduce_max = make_reduce_max(world, "cuda")
@@ -960,18 +977,20 @@ def gpu_arm(args):
     ana_mean_s = statistics.mean(ana_ms) / 1e3
     achieved = flops / ana_mean_s / 1e12
     fallback = 1 if f.precision == 0 else 0
-    launches_per_frame = 1 + (1 + fallback) + 1   # observation with the residual, pair (+ FP64 list), forecast
-    # the Jacobi executes several times the paper's m^3 for the EVD: the kernel's
-    # own flops, from its loop counts and the measured mean sweeps
+    # observation with residual and noise, pair, list; the forecast inside them, or its own
+    launches_per_frame = 3
+    # the kernel's own flops, from its loop counts and the products its series take on a
+    # sample of the last frame's nodes
     mp = next(c for c in (16, 24, 32, 48, 64) if w.m <= c)
     n_sup = opcount.taper_support_cells(w.window, w.taper, w.loc_len)
-    ex_flops = opcount.frame_executed_flops(mp, f.n_pts, n_sup,
-                                            total_sweeps / max(1, f.n_pts - nfp64))
+    products = mean_products(w, inp, X_last)
+    ex_flops = opcount.frame_executed_flops(mp, f.n_pts, n_sup, products)
     executed = {"flops_per_launch": ex_flops, "achieved": ex_flops / ana_mean_s / 1e12,
                 "frac": ex_flops / ana_mean_s / 1e12 / fp32_peak,
                 "count": f"per node: Gram 2 mp^2 over the 2 x {n_sup} slopes of the window "
-                         "cells inside the taper's support, Jacobi 3.5 mp^3 per sweep x the "
-                         "measured mean sweeps, transform and apply 10 mp^2 (an FMA counts as two)"}
+                         "cells inside the taper's support, 4 mp^2 per product of the "
+                         f"Chebyshev series x {products:.1f} products (mean of 64 nodes' "
+                         "ratios at the last frame; an FMA counts as two)"}
     line = {
         "metric": METRIC, "value": agg["value"], "unit": UNIT, "n_gpus": world, "steps": K,
         "warmup": Wm, "ms_per_step": agg["ms_per_step"], "higher_is_better": True,
@@ -1006,6 +1025,7 @@ def gpu_arm(args):
                      "launch_us": 1e6 * ana_mean_s,
                      "executed": executed},
         "gpu_launches": launches_per_frame * K,
+        # a node analysed by the Chebyshev series or the tridiagonal form counts one
         "jacobi_sweeps_max": sweeps, "jacobi_sweeps_mean": total_sweeps / max(1, f.n_pts - nfp64),
         "fp64_nodes_last_frame": nfp64,
         "wall_s_timed": t_wall,

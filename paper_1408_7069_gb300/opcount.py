@@ -9,6 +9,8 @@ for m = 101, n = 32, p = 128). Appendix B.2 counts the prediction step,
 """
 from __future__ import annotations
 
+import math
+
 
 def update_mults(m: int, n: int, p: int, gamma: int = 1) -> int:
     """Multiplications of one (local) update with state size n and p observations."""
@@ -44,16 +46,23 @@ def taper_support_cells(window: int, taper: int, loc_len: float = 0.0) -> int:
                if ((ds - hw + 0.5) ** 2 + (dt - hw + 0.5) ** 2) ** 0.5 / c < 2.0)
 
 
-def frame_executed_flops(mp: int, n_nodes: int, support_cells: int, mean_sweeps: float) -> float:
+def chebyshev_products(ratio: float, tol: float = 1e-8) -> int:
+    """Products with G that the Chebyshev series of the FP32 analysis takes at a node of
+    ratio |G|_F / alpha: the degree at which the tail of the series of (1 + g)^-1 on
+    [0, r] (coefficients 2 q^k, the slower of the two) falls below tol, r the node's
+    class of the kernel's table (0.25 x 1.25^c)."""
+    r = 0.25 * 1.25 ** max(0, math.ceil(math.log(max(ratio, 1e-30) / 0.25) / math.log(1.25)))
+    chi = 1.0 + 2.0 / r
+    q = chi - math.sqrt(chi * chi - 1.0)
+    return max(1, math.ceil(math.log(tol * (1.0 + q) / 2.0) / math.log(q)) - 1)
+
+
+def frame_executed_flops(mp: int, n_nodes: int, support_cells: int, mean_products: float) -> float:
     """Flops the FP32 analysis kernel executes per frame (an FMA counts as two),
     from its loop structure, beside the paper's count. Per node: the Gram over
     the window cells inside the taper's support (two slopes each, 2 mp^2 flops
-    per slope, both triangles of the mp x mp matrix, pupil or not); per Jacobi
-    sweep mp rounds of mp/2 column pairs, each a dot product (2 mp) and a
-    rotation of both columns, 4 mp in the even rounds (one FMA per element)
-    and 6 mp in the odd ones (a multiply and an FMA), 3.5 mp^3 in all; the
-    eigenvector normalisation, transform and apply (about 10 mp^2).
-    mean_sweeps: the measured mean sweep count per node."""
-    per_sweep = 3.5 * mp ** 3
-    per_node = 2.0 * mp * mp * 2 * support_cells + mean_sweeps * per_sweep + 10.0 * mp * mp
+    per slope, both triangles of the mp x mp matrix, pupil or not); per product of
+    the Chebyshev series with the two anomaly rows 4 mp^2.
+    mean_products: the mean number of products per node (chebyshev_products)."""
+    per_node = 2.0 * mp * mp * 2 * support_cells + mean_products * 4.0 * mp * mp
     return float(n_nodes * per_node)
