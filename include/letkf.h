@@ -380,7 +380,7 @@ letkf_status letkf_stats(letkf_t h, int32_t *fp64_points, int32_t *max_sweeps,
  * start-up, or code where cudaMalloc is not allowed). It needs no handle and
  * calls no cudaMalloc, cudaFree or other allocating routine: its scratch (the
  * slope-anomaly and innovation grids, node tables, counters) is one static
- * device array of about 6 MB that every GPU loading this library keeps until
+ * device array of about 7 MB that every GPU loading this library keeps until
  * the process exits. The paper has no counterpart; it computes the same
  * analysis as letkf_analyze in FP32, with eigenvectors accumulated from the
  * identity and without the FP64 fallback.

@@ -62,9 +62,9 @@ constexpr int LK_TRI_INST = 26;
 // total sweeps, [4..6] lengths of the classes' sweep lists, [7..8] of the
 // tridiagonal lists of classes 0 and 1 (which fill the same worklists from their ends).
 constexpr int LK_COUNTERS = 16, LK_TRI_LIST = 3;   // a class's tridiagonal count sits 3 above its sweep count
-// The FP64 table, truncated below FP64 rounding: classes up to 42.4, 128 terms.
-// Beyond, the products outnumber an eigensolve's work on the 0.5 FMA per clock
-// that an SM sub-partition issues.
+// The FP64 table, truncated below FP64 rounding: classes up to 42.4, 128 terms. Beyond,
+// the recurrences' rounding in pairs of floats (it grows with the terms' number) is no longer
+// below the eigensolve's.
 constexpr int LK_CHEB_CLASSES64 = 24, LK_CHEB_LD64 = 136;
 constexpr float LK_CHEB_MAX64 = 42.f;
 
