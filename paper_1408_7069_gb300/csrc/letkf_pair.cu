@@ -69,22 +69,24 @@ struct PairCfg {
   static constexpr int GL = MP <= 32 ? pow2_ceil(LPN) : 32;    // lanes of a node's group (power of 2)
   static constexpr int NPW = 32 / GL;                          // nodes per warp
   static constexpr int K2 = MP / 2;                            // float2 per column
-  static constexpr int CELLF = 2 * MP + 4;                     // floats per halo cell (+4: bank shift)
+  static constexpr int CELLF = 2 * MP + 4;                     // floats per halo cell: its slopes, its two
+                                                               // innovations (at 2 MP), two unused (bank shift)
   static constexpr int NODE_SCR = 4 * MP + 4;                  // scratch floats per node
   static constexpr int MPS = MP == 24 ? 32 : MP;               // columns of the stored basis
 };
 
-// Shared-memory layout of one CTA (bytes).
+// Shared-memory layout of one CTA (bytes). The innovations stand in the halo cells' padding:
+// as an array of their own they would, beside the support list and the series' terms, take
+// the 4 x 4 tile past an SM's 227 KB at a window of 25 and 17 to 32 members.
 struct PairLayout {
-  size_t dh, tap, scr, total;
+  size_t tap, scr, total;
 };
 template <int MP, int TI, int TJ>
 __host__ __device__ PairLayout pair_layout(int w) {
   using C = PairCfg<MP>;
   PairLayout L;
   const size_t ncell = (size_t)(TI + w - 1) * (TJ + w - 1);
-  L.dh = align16(ncell * C::CELLF * sizeof(float));
-  L.tap = align16(L.dh + ncell * 2 * sizeof(float));
+  L.tap = align16(ncell * C::CELLF * sizeof(float));
   L.scr = align16(L.tap + ((size_t)w * w + 2) * sizeof(float2));
   L.total = L.scr + (size_t)TI * TJ * C::NODE_SCR * sizeof(float);
   return L;
@@ -288,7 +290,7 @@ __device__ __forceinline__ void cp_async4(float *dst, const float *src) {
 }
 template <int MP, int TI, int TJ, typename S = float, bool LIST = true>
 __device__ __forceinline__ void stage_pair_tile(const LkInst &I, int i0, int j0, float *halo,
-                                                float *dh, float *tap) {
+                                                float *tap) {
   using C = PairCfg<MP>;
   const int w = I.w, m = I.m;
   const int HJ = TJ + w - 1;
@@ -331,7 +333,7 @@ __device__ __forceinline__ void stage_pair_tile(const LkInst &I, int i0, int j0,
       }
     }
     for (int e = threadIdx.x; e < ncell * 2; e += blockDim.x)
-      cp_async4(dh + e, dp + source(e >> 1) * 2 + (e & 1));
+      cp_async4(halo + (size_t)(e >> 1) * C::CELLF + 2 * MP + (e & 1), dp + source(e >> 1) * 2 + (e & 1));
     if constexpr (LIST)
       support_list(taper, w, HJ, tap);
     else
@@ -341,21 +343,17 @@ __device__ __forceinline__ void stage_pair_tile(const LkInst &I, int i0, int j0,
     for (int e = threadIdx.x; e < ncell * C::CELLF; e += blockDim.x) {
       const int cell = e / C::CELLF;
       const int r = e - cell * C::CELLF;
+      const int hi = cell / HJ, hj = cell - hi * HJ;
+      const size_t src = (size_t)(i0 + hi) * I.gs_cols + (j0 + hj);
       float v = 0.f;
       if (r < 2 * MP) {
         const int c = r / MP;
         const int mm = r - c * MP;
-        const int hi = cell / HJ, hj = cell - hi * HJ;
-        const size_t src = (size_t)(i0 + hi) * I.gs_cols + (j0 + hj);
         if (mm < m) v = (float)Ybp[(src * 2 + c) * m + mm];
+      } else if (r < 2 * MP + 2) {
+        v = (float)dp[src * 2 + r - 2 * MP];
       }
       halo[e] = v;
-    }
-    for (int e = threadIdx.x; e < ncell * 2; e += blockDim.x) {
-      const int cell = e >> 1;
-      const int hi = cell / HJ, hj = cell - hi * HJ;
-      const size_t src = (size_t)(i0 + hi) * I.gs_cols + (j0 + hj);
-      dh[e] = (float)dp[src * 2 + (e & 1)];
     }
     if constexpr (LIST)
       support_list(taper, w, HJ, tap);
@@ -491,9 +489,8 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
   const PairLayout Ly = pair_layout<MP, TI, TJ>(w);
   const int HJ = TJ + w - 1;
   float *halo = reinterpret_cast<float *>(smem);
-  float *dh = reinterpret_cast<float *>(smem + Ly.dh);
   float *tap = reinterpret_cast<float *>(smem + Ly.tap);
-  stage_pair_tile<MP, TI, TJ, S>(I, tl.i0, tl.j0, halo, dh, tap);
+  stage_pair_tile<MP, TI, TJ, S>(I, tl.i0, tl.j0, halo, tap);
   __syncthreads();
   LK_PHASE_STAMP(ph1);
 
@@ -516,7 +513,6 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
   }
   float diag = 0.f, cd0 = 0.f, cd1 = 0.f;
   const float *hwin = halo + (size_t)(ti * HJ + tj) * C::CELLF;
-  const float *dwin = dh + (size_t)(ti * HJ + tj) * 2;
   const int lr = live ? li : 0;                      // idle lanes read row pair 0, then drop it
   const int n_cell = reinterpret_cast<const int *>(tap)[0];
   const float2 *list = reinterpret_cast<const float2 *>(tap) + 1;
@@ -532,7 +528,7 @@ __global__ void __launch_bounds__(PairLaunch<MP, TI, TJ>::threads, PairLaunch<MP
       const float2 yl = reinterpret_cast<const float2 *>(yv)[lr];
       const float cy0 = tw * yl.x, cy1 = tw * yl.y;
       diag = fmaf(cy0, yl.x, fmaf(cy1, yl.y, diag));
-      const float dj = dwin[cell * 2 + c];
+      const float dj = hwin[(size_t)cell * C::CELLF + 2 * MP + c];
       cd0 = fmaf(cy0, dj, cd0);
       cd1 = fmaf(cy1, dj, cd1);
       const float2 c0 = f2(cy0), c1 = f2(cy1);
@@ -879,9 +875,8 @@ __global__ void __launch_bounds__(SplitLaunch<MP, TI, TJ>::threads, SplitLaunch<
   const PairLayout Ly = pair_layout<MP, TI, TJ>(w);
   const int HJ = TJ + w - 1;
   float *halo = reinterpret_cast<float *>(smem);
-  float *dh = reinterpret_cast<float *>(smem + Ly.dh);
   float *tap = reinterpret_cast<float *>(smem + Ly.tap);
-  stage_pair_tile<MP, TI, TJ, float, false>(I, tl.i0, tl.j0, halo, dh, tap);
+  stage_pair_tile<MP, TI, TJ, float, false>(I, tl.i0, tl.j0, halo, tap);
   __syncthreads();
   LK_PHASE_STAMP(ph1);
 
@@ -904,7 +899,6 @@ __global__ void __launch_bounds__(SplitLaunch<MP, TI, TJ>::threads, SplitLaunch<
   }
   float diag = 0.f, cd0 = 0.f, cd1 = 0.f;
   const float *hwin = halo + (size_t)(ti * HJ + tj) * C::CELLF;
-  const float *dwin = dh + (size_t)(ti * HJ + tj) * 2;
   for (int ds = 0; ds < w; ++ds) {
     for (int dt = 0; dt < w; ++dt) {
       const int cell = ds * HJ + dt;
@@ -916,7 +910,7 @@ __global__ void __launch_bounds__(SplitLaunch<MP, TI, TJ>::threads, SplitLaunch<
         const float2 yl = reinterpret_cast<const float2 *>(yv)[li];
         const float cy0 = tw * yl.x, cy1 = tw * yl.y;
         diag = fmaf(cy0, yl.x, fmaf(cy1, yl.y, diag));
-        const float dj = dwin[cell * 2 + c];
+        const float dj = hwin[(size_t)cell * C::CELLF + 2 * MP + c];
         cd0 = fmaf(cy0, dj, cd0);
         cd1 = fmaf(cy1, dj, cd1);
         const float2 c0 = f2(cy0), c1 = f2(cy1);
