@@ -639,9 +639,7 @@ size_t node_smem(const LkInst &I) {
 
 template <int MP, typename S, typename T>
 cudaError_t set_node_smem(const LkInst &I) {
-  return cudaFuncSetAttribute(adjoint_node_kernel<MP, S, T>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)node_smem<MP, S, T>(I));
+  return lk_raise_smem(adjoint_node_kernel<MP, S, T>, node_smem<MP, S, T>(I));
 }
 
 cudaError_t setup_kernels(letkf_ctx *h) {

@@ -237,6 +237,18 @@ cudaError_t launch_class(letkf_ctx *h, int cls, void *mean, void *spread, const 
 
 }  // namespace
 
+cudaError_t lk_raise_smem_limit(const void *kernel, size_t bytes) {
+  static std::mutex mutex;               // reading and raising are one step
+  std::lock_guard<std::mutex> lock(mutex);
+  cudaFuncAttributes at;
+  cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+  if (e == cudaSuccess && (size_t)at.maxDynamicSharedSizeBytes < bytes)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  // reported by the caller: not to be found by the thread's next launch as its own
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e;
+}
+
 int lk_num_tile_shapes() { return LK_NUM_SHAPES; }
 
 void lk_tile_shape(int s, int *ti, int *tj) {
@@ -423,8 +435,7 @@ cudaError_t na_scratch_address(int dev, unsigned char **out) {
 
 template <int MP>
 cudaError_t na_setup_kernel(size_t smem_bytes) {
-  return cudaFuncSetAttribute(analysis_noalloc_kernel<MP>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+  return lk_raise_smem(analysis_noalloc_kernel<MP>, smem_bytes);
 }
 
 }  // namespace

@@ -285,6 +285,15 @@ cudaError_t lk_launch_list64(letkf_ctx *h, int cls, void *mean, void *spread,
 cudaError_t lk_setup_node64w();
 cudaError_t lk_setup_list();
 
+// Raises the dynamic shared memory that a kernel may take on the current device to `bytes`.
+// The limit belongs to the kernel, which every live handle launches with what its own windows
+// need: it is never lowered.
+cudaError_t lk_raise_smem_limit(const void *kernel, size_t bytes);
+template <typename... KArgs>
+cudaError_t lk_raise_smem(void (*kernel)(KArgs...), size_t bytes) {
+  return lk_raise_smem_limit(reinterpret_cast<const void *>(kernel), bytes);
+}
+
 // Whether width class cls of the handle can take tile shape `shape`: FP32
 // handles need whole warps of nodes and, in class 2 (one node per warp), at
 // most 8 nodes per tile. (FP64 handles take any shape, which they ignore.)

@@ -1159,12 +1159,9 @@ cudaError_t launch_global_rpl(letkf_ctx *h, void *mean, void *spread) {
 
 template <int RPL>
 cudaError_t setup_global_rpl(const LkDom &D, int m) {
-  cudaError_t e = cudaFuncSetAttribute(global_solve_kernel<RPL>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)global_solve_smem<RPL>());
+  cudaError_t e = lk_raise_smem(global_solve_kernel<RPL>, global_solve_smem<RPL>());
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(global_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(float) * ((size_t)m * m + 16 * (size_t)m)));
+    e = lk_raise_smem(global_apply_kernel, sizeof(float) * ((size_t)m * m + 16 * (size_t)m));
   (void)D;
   return e;
 }
@@ -1189,14 +1186,11 @@ cudaError_t launch_rpl(letkf_ctx *h, DomArgs a) {
 template <int RPL>
 cudaError_t setup_rpl(const LkDom &D) {
   const size_t smem = (size_t)dom_layout(8 * RPL, D.max_obs, 2 * D.max_nodes).total * sizeof(float);
-  const cudaError_t e = cudaFuncSetAttribute(domain_kernel<RPL>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+  const cudaError_t e = lk_raise_smem(domain_kernel<RPL>, smem);
   if (e != cudaSuccess || !D.series) return e;
   const size_t b = sizeof(float) *
                    (size_t)dom_series_layout(8 * RPL, D.max_obs, 2 * D.max_nodes).total;
-  return cudaFuncSetAttribute(domain_series_kernel<RPL>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b);
+  return lk_raise_smem(domain_series_kernel<RPL>, b);
 }
 
 // Rows per lane of the Jacobi layout (MPD = 8 RPL columns); 0: wider than the

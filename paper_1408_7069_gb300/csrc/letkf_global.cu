@@ -523,8 +523,7 @@ size_t lk_ns_workspace_bytes(int mpt, long long n_pad) {
 }
 
 cudaError_t lk_ns_setup() {
-  return cudaFuncSetAttribute(ns_root_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              NR_SMEM * (int)sizeof(float));
+  return lk_raise_smem(ns_root_kernel, NR_SMEM * sizeof(float));
 }
 
 cudaError_t lk_launch_ns_global(letkf_ctx *h, const double *gpart, const double *cpart,

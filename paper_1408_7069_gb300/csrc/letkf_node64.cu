@@ -907,16 +907,12 @@ cudaError_t launch_list64w(letkf_ctx *h, void *mean, void *spread, const LkCycle
 }  // namespace
 
 cudaError_t lk_setup_node64w() {
-  return cudaFuncSetAttribute(node64w_list_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(n64w_smem_doubles() * sizeof(double)));
+  return lk_raise_smem(node64w_list_kernel, n64w_smem_doubles() * sizeof(double));
 }
 
 cudaError_t lk_setup_list() {
-  const cudaError_t e = cudaFuncSetAttribute(
-      tri_list_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_list_smem<16>());
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(tri_list_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)tri_list_smem<32>());
+  const cudaError_t e = lk_raise_smem(tri_list_kernel<16>, tri_list_smem<16>());
+  return e == cudaSuccess ? lk_raise_smem(tri_list_kernel<32>, tri_list_smem<32>()) : e;
 }
 
 cudaError_t lk_launch_node64(letkf_ctx *h, int cls, void *mean, void *spread) {

@@ -1234,22 +1234,19 @@ cudaError_t launch_basis(letkf_ctx *h, int cls) {
 
 template <int MP, int TI, int TJ>
 cudaError_t set_shape_smem(int w, bool fp64) {
-  const int bytes = (int)pair_layout<MP, TI, TJ>(w).total;
+  const size_t bytes = pair_layout<MP, TI, TJ>(w).total;
   cudaError_t e = cudaSuccess;
   if constexpr (shape_ok<MP, TI, TJ>()) {
     if (fp64) {
       if constexpr (MP == 16 || MP == 32)
-        e = cudaFuncSetAttribute(analysis_pair_kernel<MP, TI, TJ, double, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        e = lk_raise_smem(analysis_pair_kernel<MP, TI, TJ, double, true>, bytes);
       return e;
     }
-    e = cudaFuncSetAttribute(analysis_pair_kernel<MP, TI, TJ>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    e = lk_raise_smem(analysis_pair_kernel<MP, TI, TJ>, bytes);
   }
   if constexpr (split_shape_ok<MP, TI, TJ>())
     if (e == cudaSuccess && !fp64)
-      e = cudaFuncSetAttribute(analysis_split_kernel<MP, TI, TJ>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+      e = lk_raise_smem(analysis_split_kernel<MP, TI, TJ>, bytes);
   return e;
 }
 

@@ -924,14 +924,10 @@ cudaError_t launch_series64(letkf_ctx *h, int cls, void *mean, void *spread, con
 
 template <int MPD>
 cudaError_t setup_series64(int w) {
-  cudaError_t e =
-      cudaFuncSetAttribute(series64_kernel<MPD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(Smem64<MPD>::doubles(w) * sizeof(double)));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(adjoint_series64_kernel<MPD>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(AdjSmem64<MPD>::doubles(w) * sizeof(double)));
-  return e;
+  const cudaError_t e =
+      lk_raise_smem(series64_kernel<MPD>, Smem64<MPD>::doubles(w) * sizeof(double));
+  if (e != cudaSuccess) return e;
+  return lk_raise_smem(adjoint_series64_kernel<MPD>, AdjSmem64<MPD>::doubles(w) * sizeof(double));
 }
 
 }  // namespace
