@@ -11,7 +11,7 @@
 // so it is run downwards (Miller's algorithm) and scaled by the series' value at
 // x = -1, where every term is positive and the sum is f = 1. For the inverse
 //   (chi + cos t)^-1 = (chi^2 - 1)^-1/2 sum_k eps_k (-q)^k cos(k t),
-//   q = chi - sqrt(chi^2 - 1),
+//   q = chi - sqrt(chi^2 - 1) = 1 / (chi + sqrt(chi^2 - 1)),
 // scaled the same way. The degree of a class is the first with both remainders
 // below the tolerance (relative to the functions' maximum of 1).
 #include <math.h>
@@ -25,7 +25,8 @@ namespace {
 
 // a[k], b[k], k = 0 .. degree; returns the degree.
 int cheb_series(double r, double tol, std::vector<double> &a, std::vector<double> &b) {
-  const double chi = (2.0 + r) / r, q = chi - sqrt(chi * chi - 1.0);
+  // q without the difference's cancellation (chi >> 1 at small r: 8e-15 of q at r = 0.25)
+  const double d = 2.0 / r, chi = 1.0 + d, q = 1.0 / (chi + sqrt(d * (d + 2.0)));
   // terms decay like q^k: far enough for the smallest tolerance
   const int n = (int)ceil(log(tol * 1e-3) / log(q)) + 16;
   a.assign(n + 2, 0.0);
