@@ -19,7 +19,7 @@
 // both ends of the interval equal, so that the lower one grows by up to
 // 1.5 sqrt(3) = 2.6 per step instead of 1.5, and the next interval is known
 // without looking at the matrices (Chen & Chow's and Higham's scaled iterations).
-// From x_0 = 0.003 (the prior draw's kappa of 1e5) ten steps reach 1 - 1e-5
+// From x_0 = 0.003 (the prior draw's kappa of 1e5) ten steps reach 1 - 2^-21
 // where the unscaled iteration took 26; a loop's kappa of 50 takes six.
 //
 // Everything between the Gram and the apply is one cooperative kernel: a grid
@@ -129,6 +129,10 @@ constexpr int NR_PART = NR_TILE * NR_LD;               // floats of a warp's par
 // shared floats: every warp's slices, every warp's partial tile, the tile's sums
 constexpr int NR_SMEM = NR_WARPS * (NR_STAGES * NR_SLICE + NR_PART) + NR_TILE * (NR_TILE + 1);
 constexpr int NR_MAX_ITERS = 24, NR_REFINE = 8;
+// What the iteration may leave of 1 - x at the interval's lower end: an error of Z as large in
+// every direction without slopes, so no more than the products' rounding. (At 1e-5 the spread
+// of a loop's update was wrong by up to 7e-6; the step that takes 1e-5 below this is the last.)
+constexpr float NR_LEFT = 0x1p-21f;
 constexpr unsigned NR_SPIN = 1u << 21;       // polls of a grid barrier (about a second)
 
 struct NsArgs {
@@ -353,7 +357,7 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
     // ---- Newton-Schulz; x: the lower end of the interval ----
     float *cur = a.mat, *nxt = a.mat + 4 * nn;         // Y, Y^T, Z, Z^T
     float x = (float)sqrt(I.alpha * inv);
-    for (int it = 0; x < 1.f - 1e-5f && it < NR_MAX_ITERS; ++it) {
+    for (int it = 0; x < 1.f - NR_LEFT && it < NR_MAX_ITERS; ++it) {
       const float mu2 = 3.f / (1.f + x + x * x), mu = sqrtf(mu2);
       const float ca = 1.5f * mu, cb = 0.5f * mu * mu2;
       auto first = [&](int t) {                      // Z Y

@@ -1,0 +1,67 @@
+"""The root, the mean and the status of the global ETKF of more than 64 members
+(letkf_global.cu) against the FP64 oracle, where they can go wrong."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+from oracle import letkf_domains as LD  # noqa: E402
+from paper_1408_7069_gb300 import synth  # noqa: E402
+from paper_1408_7069_gb300.letkf import Letkf  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+SIGMA2, RHO = 0.01, 1.03
+UNIT = 2.0 ** -24
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.asarray(a, np.float64) - b) / np.linalg.norm(b))
+
+
+def problem(nsub, m, seed=0):
+    """Geometry, means and unit anomalies [n, 2, m] of an ensemble, slopes, and the Gram of
+    its unit anomalies' slopes over sigma^2."""
+    mask = synth.pupil_subap_mask(nsub, 0.0)
+    dg = LD.build_domains(mask, 1, 3, 0, 0.0)
+    rng = np.random.default_rng(seed + nsub + m)
+    n = dg.geom.n_pts
+    mean = 3 * rng.standard_normal((n, 2, 1))
+    P = rng.standard_normal((n, 2, m))
+    P -= P.mean(-1, keepdims=True)
+    _, _, Yb, _ = oracle.observe(dg.geom, P)
+    y = rng.standard_normal(dg.geom.p).astype(np.float32)
+    return mask, dg, mean, P, y, Yb.T @ Yb / SIGMA2
+
+
+def analyse(mask, m, X, y):
+    f = Letkf(mask, m=m, window=3, taper=0, rho=RHO, sigma2=SIGMA2, partition=1)
+    f.set_state(torch.from_numpy(X).cuda())
+    mean, spread = f.analyze(torch.from_numpy(y).cuda())
+    try:
+        f.sync()
+        return mean.cpu().numpy(), spread.cpu().numpy(), f.get_state().cpu().numpy()
+    finally:
+        f.close()
+
+
+@pytest.mark.parametrize("kappa", [12.5, 14.0, 50.0, 100.0, 530.0, 3500.0])
+def test_the_root_converges_in_the_directions_without_slopes(kappa):
+    """Most of the eigenvalues of A sit at their lower bound (128 members, at most 32 slopes),
+    the last to converge: what is left when the iteration stops is an error of the spread. At
+    |A|_F / alpha of 14, 530 and 3500 a step ends just short of the others. Tolerance: the
+    rounding of the products, 16 units of 2^-24, and sqrt(kappa) of them that Z's own
+    condition adds."""
+    m, alpha = 128, 127 / RHO
+    mask, dg, mean, P, y, G = problem(4, m)
+    lo, hi = 1e-6, 1e3
+    for _ in range(60):                                 # the scale of the anomalies for kappa
+        s = (lo * hi) ** 0.5
+        big = np.linalg.norm(alpha * np.eye(m) + s * s * G) > kappa * alpha
+        lo, hi = (lo, s) if big else (s, hi)
+    X = (mean + s * P).astype(np.float32)
+    _, rmean, rspread = LD.analysis_domains(dg, X.astype(np.float64), y.astype(np.float64), SIGMA2,
+                                            RHO)
+    gm, gs, _ = analyse(mask, m, X, y)
+    assert rel(gs, rspread) <= (16 + kappa ** 0.5) * UNIT
