@@ -10,8 +10,11 @@
 //            Y -> (A/s_A)^1/2 and Z -> (A/s_A)^-1/2, FP32 matrix products
 //   mean     wbar = A^-1 c by iterative refinement: residual c - A wbar in
 //            FP64, correction Z (Z r) / s_A in FP32
-//   apply    T = wbar 1^T + sqrt((m-1) / s_A) Z, Xa = xbar + X' T over all
-//            state rows, mean and spread
+//   apply    P = X' sqrt((m-1) / s_A) Z over all state rows, Xa = xbar + X' wbar + P,
+//            X' wbar in FP64 (m products per row: 4 us of 909 at m = 626), mean and
+//            spread. P's mean over the members is zero but for Z's rounding, which grows
+//            with kappa, and the rounding of the slopes' means, part of whose error in
+//            X' wbar it takes back: it is kept up to NR_KEEP and taken out beyond
 //
 // Scaled steps: the singular values x = sqrt(eig(Z Y)) start in [x_0, 1] with
 // x_0 = sqrt(alpha / s_A), alpha = (m-1)/rho the smallest eigenvalue A can have.
@@ -133,6 +136,10 @@ constexpr int NR_MAX_ITERS = 24, NR_REFINE = 8;
 // every direction without slopes, so no more than the products' rounding. (At 1e-5 the spread
 // of a loop's update was wrong by up to 7e-6; the step that takes 1e-5 below this is the last.)
 constexpr float NR_LEFT = 0x1p-21f;
+// s_A / alpha up to which P keeps its mean. Measured, error of the mean of Xa at m = 128,
+// 320 and 70 (kept, taken out): 16-70 1.4-2.9e-8, 1.5-3.7e-8; 400-1000 3.6-7.8e-8, 4.0-8.5e-8;
+// 1600-3900 4.4-17e-8, 4.5-16e-8; 2.2e4-5.5e4 8.7e-8-2.6e-6, 5.4e-8-2.0e-6; at 3e6 1e-3, 1e-4.
+constexpr double NR_KEEP = 2e3;
 constexpr unsigned NR_SPIN = 1u << 21;       // polls of a grid barrier (about a second)
 
 struct NsArgs {
@@ -143,8 +150,9 @@ struct NsArgs {
   double *A64, *c64, *w64, *part;            // part [grid]: sums of squares
   float *mat;                                // eight [n][n] matrices: Y, Y^T, Z, Z^T, twice
   float *T, *TT, *rv, *vv, *Xp, *xm;
-  unsigned *sync;                            // [0] arrivals, [1] departures, [2] abort,
-                                             // [4 ..] per refinement: max |r| (float bits)
+  unsigned *sync;                            // [0] arrivals, [1] departures, [2] abort, [3] P
+                                             // keeps its mean, [4 ..] per refinement: max |r|
+                                             // (float bits)
   int *counters;
 };
 
@@ -347,6 +355,7 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
     for (int k = lane; k < (int)gridDim.x; k += 32) fro += __ldcg(a.part + k);
     fro = sqrt(lk_warp_sum(fro));
     const double inv = 1.0 / fro;
+    if (blockIdx.x == 0 && tid == 0) a.sync[3] = inv * I.alpha * NR_KEEP >= 1.0;
     for (long long e = (long long)blockIdx.x * NR_THREADS + tid; e < (long long)n * n;
          e += (long long)gridDim.x * NR_THREADS) {
       const float y = (float)(__ldcg(a.A64 + e) * inv), z = e / n == e % n ? 1.f : 0.f;
@@ -444,8 +453,8 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
       if (!(live = grid_sync(a, target, &flag))) break;
     }
     if (!live) break;
-    // ---- T = wbar 1^T + sqrt((m-1) / s_A) Z on the m x m block, zero elsewhere; the
-    // iteration failed if Z Y strays from I by more than 1e-3 ----
+    // ---- T = sqrt((m-1) / s_A) Z on the m x m block, zero elsewhere; the iteration
+    // failed if Z Y strays from I by more than 1e-3 ----
     const float f = (float)sqrt((m - 1) * inv);
     float mx = 0.f;
     for (int t = blockIdx.x; t < nt * nt; t += gridDim.x) {
@@ -457,10 +466,8 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
       const float e0 = fabsf(p.x - (r == c ? 1.f : 0.f)), e1 = fabsf(p.y - (r == c + 1 ? 1.f : 0.f));
       if (!(e0 <= 1e-3f) || !(e1 <= 1e-3f)) mx = 1.f;
       const float2 z = __ldcg(reinterpret_cast<const float2 *>(Z + (size_t)r * n + c));
-      const float w = (float)__ldcg(a.w64 + r);
       *reinterpret_cast<float2 *>(a.T + (size_t)r * n + c) =
-          make_float2(r < m && c < m ? fmaf(f, z.x, w) : 0.f,
-                      r < m && c + 1 < m ? fmaf(f, z.y, w) : 0.f);
+          make_float2(r < m && c < m ? f * z.x : 0.f, r < m && c + 1 < m ? f * z.y : 0.f);
     }
     if (mx != 0.f) atomicOr(a.counters, LK_BIT_NOCONVERGE);
   } while (false);
@@ -477,20 +484,36 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
   }
 }
 
-// Xa = xbar + (X' T), mean and spread, warp per state row.
+// Xa = xbar + X' wbar + P, P = X' T; mean and spread, warp per state row. Where P's mean is
+// taken out (*keep zero), what xbar's rounding has left in the anomalies, which P passes on, is
+// added back. The common part is a pair of floats, so that a member is rounded once.
 __global__ void __launch_bounds__(LK_WARP_CTA)
     ns_finish_kernel(const LkInst *__restrict__ insts, int mpt, const float *__restrict__ P,
-                     const float *__restrict__ xm, float *__restrict__ mean,
-                     float *__restrict__ spread, int *__restrict__ counters) {
+                     const float *__restrict__ Xp, const float *__restrict__ xm,
+                     const double *__restrict__ wbar, const unsigned *__restrict__ keep,
+                     float *__restrict__ mean, float *__restrict__ spread,
+                     int *__restrict__ counters) {
   lk_pdl_wait();
   const LkInst &I = insts[0];
   const long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31, m = I.m;
   if (r >= 2LL * I.n_pts) return;
   float *x = static_cast<float *>(I.X) + r * m;
+  float pm = 0.f, xr = 0.f;
+  double xw = 0.0;
+  for (int j = lane; j < m; j += 32) {
+    const float xp = Xp[r * mpt + j];
+    pm += P[r * mpt + j];
+    xr += xp;
+    xw = fma((double)xp, wbar[j], xw);
+  }
+  pm = *keep ? 0.f : lk_warp_sum(pm) / float(m);
+  xr = *keep ? 0.f : lk_warp_sum(xr) / float(m);
+  const double base = (double)xm[r] + ((double)xr + lk_warp_sum(xw));
+  const float bh = (float)base, bl = (float)(base - (double)bh);
   float sum = 0.f;
   for (int j = lane; j < m; j += 32) {
-    const float xa = xm[r] + P[r * mpt + j];
+    const float xa = bh + (bl + (P[r * mpt + j] - pm));
     x[j] = xa;
     sum += xa;
   }
@@ -575,7 +598,8 @@ cudaError_t lk_launch_ns_global(letkf_ctx *h, const double *gpart, const double 
   const unsigned fb = (unsigned)((2LL * I.n_pts * 32 + LK_WARP_CTA - 1) / LK_WARP_CTA);
   if (e == cudaSuccess)
     e = lk_launch_pdl(ns_finish_kernel, fb, LK_WARP_CTA, 0, h->stream,
-                      (const LkInst *)h->d_inst, mpt, (const float *)Pr, (const float *)a.xm,
+                      (const LkInst *)h->d_inst, mpt, (const float *)Pr, (const float *)a.Xp,
+                      (const float *)a.xm, (const double *)a.w64, (const unsigned *)(a.sync + 3),
                       static_cast<float *>(mean), static_cast<float *>(spread), h->counters);
   return e;
 }

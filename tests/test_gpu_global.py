@@ -65,3 +65,22 @@ def test_the_root_converges_in_the_directions_without_slopes(kappa):
                                             RHO)
     gm, gs, _ = analyse(mask, m, X, y)
     assert rel(gs, rspread) <= (16 + kappa ** 0.5) * UNIT
+
+
+@pytest.mark.parametrize("nsub,m", [(9, 192), (10, 128), (16, 320)])
+@pytest.mark.parametrize("scale", [0.05, 3.0, 10.0, 30.0])
+def test_the_mean_is_that_of_the_refined_solve(nsub, m, scale):
+    """|A|_F / alpha from 16 to 4e6: the mean's increment X' wbar is as accurate as the FP64
+    refinement leaves wbar and the FP32 slopes allow, whatever the FP32 root's rounding, 2^-23
+    |A|_F / alpha in the anomalies, does. Tolerance, relative to the increment: the slopes'
+    rounding, 2^-24 of each, amplified by sqrt(kappa) in the root mean square, a few times."""
+    mask, dg, mean, P, y, G = problem(nsub, m)
+    alpha = (m - 1) / RHO
+    X = (mean + scale * P).astype(np.float32)
+    _, rmean, _ = LD.analysis_domains(dg, X.astype(np.float64), y.astype(np.float64), SIGMA2, RHO)
+    kappa = np.linalg.norm(alpha * np.eye(m) + scale ** 2 * G) / alpha
+    _, _, Xa = analyse(mask, m, X, y)
+    got = Xa.astype(np.float64).mean(-1)
+    step = rmean - X.astype(np.float64).mean(-1)
+    assert np.linalg.norm(got - rmean) <= 6 * kappa ** 0.5 * UNIT * np.linalg.norm(step) \
+        + 2 * UNIT * np.linalg.norm(rmean)
