@@ -57,7 +57,8 @@ typedef enum {
   LETKF_OK = 0,
   LETKF_ERR_ARG = 1,        /* invalid argument: nothing was launched */
   LETKF_ERR_CUDA = 2,       /* a CUDA runtime call failed */
-  LETKF_ERR_NOCONVERGE = 3, /* a Jacobi eigensolve hit its sweep limit */
+  LETKF_ERR_NOCONVERGE = 3, /* a Jacobi eigensolve hit its sweep limit, or the global update of more
+                               than 64 members met a condition beyond FP32 (about 5e7) */
   LETKF_ERR_TIMEOUT = 4,    /* a bounded device wait gave up */
   LETKF_ERR_NONFINITE = 5,  /* NaN or Inf met in slopes or ensemble */
   LETKF_ERR_STATE = 6,      /* call not valid in the handle's current state */

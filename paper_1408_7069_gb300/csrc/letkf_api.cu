@@ -1191,7 +1191,9 @@ letkf_status letkf_sync(letkf_t h) {
   if (bits & LK_BIT_NONFINITE) return fail(h, LETKF_ERR_NONFINITE, "non-finite slopes or ensemble");
   if (bits & LK_BIT_TIMEOUT) return fail(h, LETKF_ERR_TIMEOUT, "a bounded device wait gave up");
   if (bits & LK_BIT_NOCONVERGE)
-    return fail(h, LETKF_ERR_NOCONVERGE, "a Jacobi eigensolve reached its sweep limit");
+    return fail(h, LETKF_ERR_NOCONVERGE, h->dom && h->inst[0].m > 64 && h->cfg.partition == 1
+                    ? "the global root or its mean did not converge"
+                    : "a Jacobi eigensolve reached its sweep limit");
   return LETKF_OK;
 }
 

@@ -136,6 +136,10 @@ constexpr int NR_MAX_ITERS = 24, NR_REFINE = 8;
 // every direction without slopes, so no more than the products' rounding. (At 1e-5 the spread
 // of a loop's update was wrong by up to 7e-6; the step that takes 1e-5 below this is the last.)
 constexpr float NR_LEFT = 0x1p-21f;
+// Largest last correction, relative to wbar, of corrections that ran out (a contraction
+// takes the error below it); its word and wbar's in the barrier words.
+constexpr float NR_CORRECTION = 1e-3f;
+constexpr int NR_LAST = 16;
 // s_A / alpha up to which P keeps its mean. Measured, error of the mean of Xa at m = 128,
 // 320 and 70 (kept, taken out): 16-70 1.4-2.9e-8, 1.5-3.7e-8; 400-1000 3.6-7.8e-8, 4.0-8.5e-8;
 // 1600-3900 4.4-17e-8, 4.5-16e-8; 2.2e4-5.5e4 8.7e-8-2.6e-6, 5.4e-8-2.0e-6; at 3e6 1e-3, 1e-4.
@@ -151,8 +155,8 @@ struct NsArgs {
   float *mat;                                // eight [n][n] matrices: Y, Y^T, Z, Z^T, twice
   float *T, *TT, *rv, *vv, *Xp, *xm;
   unsigned *sync;                            // [0] arrivals, [1] departures, [2] abort, [3] P
-                                             // keeps its mean, [4 ..] per refinement: max |r|
-                                             // (float bits)
+                                             // keeps its mean, [4 ..] per refinement: max |r|,
+                                             // [NR_LAST ..] last correction, wbar (float bits)
   int *counters;
 };
 
@@ -332,6 +336,7 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
     sq = lk_warp_sum(sq);
     if (lane == 0) red[warp] = sq;
     if (blockIdx.x == 0 && tid < NR_REFINE) a.sync[4 + tid] = 0u;
+    if (blockIdx.x == 0 && tid < 2) a.sync[NR_LAST + tid] = 0u;
     // the state rows' anomalies and means, a warp per row
     for (long long r = gw; r < a.n_pad; r += nw) {
       const bool real = r < 2LL * I.n_pts;
@@ -414,7 +419,8 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
     const float *Y = cur, *Z = cur + 2 * nn, *ZT = cur + 3 * nn;
     if (!live) break;
     // ---- wbar = A^-1 c by refinement with A^-1 ~ Z Z / s_A; done when the residual
-    // bounds the relative error of wbar by 1e-9 ----
+    // bounds the relative error of wbar by 1e-9, or after NR_REFINE corrections ----
+    bool met = false;
     for (int rf = 0; rf < NR_REFINE; ++rf) {
       if (rf > 0) {                                  // r = c - A w (at first w = 0)
         for (int i = gw; i < n; i += nw) {
@@ -433,8 +439,10 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
       }
       if (!(live = grid_sync(a, target, &flag))) break;
       if (rf > 0 && __uint_as_float(__ldcg(a.sync + 4 + rf)) <=
-                        1e-9f * (float)(I.alpha * inv) * __uint_as_float(__ldcg(a.sync + 4)))
+                        1e-9f * (float)(I.alpha * inv) * __uint_as_float(__ldcg(a.sync + 4))) {
+        met = true;
         break;
+      }
       for (int i = gw; i < n; i += nw) {
         float s = 0.f;
         for (int j = lane; j < n; j += 32)
@@ -448,11 +456,24 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
         for (int j = lane; j < n; j += 32)
           s = fmaf(__ldcg(Z + (size_t)i * n + j), __ldcg(a.vv + j), s);
         s = lk_warp_sum(s);
-        if (lane == 0) a.w64[i] = __ldcg(a.w64 + i) + (double)s * inv;
+        if (lane == 0) {
+          const double d = (double)s * inv, w = __ldcg(a.w64 + i) + d;
+          a.w64[i] = w;
+          if (rf == NR_REFINE - 1) {
+            atomicMax(a.sync + NR_LAST, __float_as_uint(fabsf((float)d)));
+            atomicMax(a.sync + NR_LAST + 1, __float_as_uint(fabsf((float)w)));
+          }
+        }
       }
       if (!(live = grid_sync(a, target, &flag))) break;
     }
     if (!live) break;
+    // Z Z is no inverse to FP32 any more from a condition of about 5e7 on, where Z Y still
+    // passes for I: the corrections grow instead of shrinking, and the last one says so
+    if (!met && blockIdx.x == 0 && tid == 0 &&
+        !(__uint_as_float(__ldcg(a.sync + NR_LAST)) <=
+          NR_CORRECTION * __uint_as_float(__ldcg(a.sync + NR_LAST + 1))))
+      atomicOr(a.counters, LK_BIT_NOCONVERGE);
     // ---- T = sqrt((m-1) / s_A) Z on the m x m block, zero elsewhere; the iteration
     // failed if Z Y strays from I by more than 1e-3 ----
     const float f = (float)sqrt((m - 1) * inv);

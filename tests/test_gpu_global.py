@@ -8,7 +8,7 @@ torch = pytest.importorskip("torch")
 import oracle  # noqa: E402
 from oracle import letkf_domains as LD  # noqa: E402
 from paper_1408_7069_gb300 import synth  # noqa: E402
-from paper_1408_7069_gb300.letkf import Letkf  # noqa: E402
+from paper_1408_7069_gb300.letkf import Letkf, LetkfError  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -84,3 +84,27 @@ def test_the_mean_is_that_of_the_refined_solve(nsub, m, scale):
     step = rmean - X.astype(np.float64).mean(-1)
     assert np.linalg.norm(got - rmean) <= 6 * kappa ** 0.5 * UNIT * np.linalg.norm(step) \
         + 2 * UNIT * np.linalg.norm(rmean)
+
+
+@pytest.mark.parametrize("nsub,m", [(9, 192), (10, 128), (16, 320), (8, 480), (16, 70)])
+def test_a_mean_that_did_not_converge_is_reported(nsub, m):
+    """Conditions from 6e6 past the end of FP32's range, where the corrections of the mean stop
+    converging before the root's own check fails: an error status, or a mean as accurate as
+    the slopes' rounding, amplified by sqrt(kappa), allows (16 units)."""
+    refused = 0
+    for scale in (60.0, 95.0, 130.0, 151.0, 176.0, 205.0, 240.0, 325.0):
+        mask, dg, mean, P, y, G = problem(nsub, m, seed=int(scale))
+        alpha = (m - 1) / RHO
+        X = (mean + scale * P).astype(np.float32)
+        _, rmean, _ = LD.analysis_domains(dg, X.astype(np.float64), y.astype(np.float64), SIGMA2, RHO)
+        kappa = np.linalg.norm(alpha * np.eye(m) + scale ** 2 * G) / alpha
+        try:
+            got = analyse(mask, m, X, y)[2].astype(np.float64).mean(-1)
+        except LetkfError as e:
+            assert "NOCONVERGE" in str(e) or "NONFINITE" in str(e)
+            refused += 1
+            continue
+        step = rmean - X.astype(np.float64).mean(-1)
+        assert np.linalg.norm(got - rmean) <= 16 * kappa ** 0.5 * UNIT * np.linalg.norm(step), scale
+        assert scale != 60.0 or kappa > 5e6
+    assert refused < 8                                   # not every one: the smallest is solved
