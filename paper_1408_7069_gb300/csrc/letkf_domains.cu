@@ -908,10 +908,11 @@ __global__ void __launch_bounds__(256)
     // |q| < 2^(ilogb ma + ilogb mb + 2), GL_KC = 64 of them
     int M = -100;
     if (ma > 0.f && mb > 0.f) {
-      M = ilogbf(ma) + ilogbf(mb) + 9;
+      // (an infinite slope has INT_MAX for an exponent: 127 takes its place in the sum)
+      M = ilogbf(fminf(ma, 0x1p127f)) + ilogbf(fminf(mb, 0x1p127f)) + 9;
       M = M < -100 ? -100 : M;
     }
-    const float s = scalbnf(1.5f, M);                // infinite with infinite slopes: NaN follows
+    const float s = scalbnf(1.5f, M);                // infinite where a product is: NaN follows
     const float2 sg = make_float2(s, s), msg = make_float2(-s, -s);
     float2 hi[2], lo[2];
     hi[0] = hi[1] = lo[0] = lo[1] = make_float2(0.f, 0.f);

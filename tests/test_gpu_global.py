@@ -108,3 +108,15 @@ def test_a_mean_that_did_not_converge_is_reported(nsub, m):
         assert np.linalg.norm(got - rmean) <= 16 * kappa ** 0.5 * UNIT * np.linalg.norm(step), scale
         assert scale != 60.0 or kappa > 5e6
     assert refused < 8                                   # not every one: the smallest is solved
+
+
+@pytest.mark.parametrize("value", [float("inf"), -float("inf"), float("nan")])
+@pytest.mark.parametrize("m", [48, 80])
+def test_a_nonfinite_ensemble_is_reported_by_both_forms(m, value):
+    """A member's infinite phase makes infinite slopes, whose exponent is no number to add to:
+    the Gram's anchor is infinite then, and the analysis NaN and reported."""
+    mask, dg, mean, P, y, _ = problem(6, m)
+    X = (mean + 0.06 * P).astype(np.float32)
+    X[20, 1, 5] = value
+    with pytest.raises(LetkfError, match="NONFINITE"):
+        analyse(mask, m, X, y)
