@@ -984,7 +984,7 @@ def gpu_arm(args):
     mp = next(c for c in (16, 24, 32, 48, 64) if w.m <= c)
     n_sup = opcount.taper_support_cells(w.window, w.taper, w.loc_len)
     products = mean_products(w, inp, X_last)
-    ex_flops = opcount.frame_executed_flops(mp, f.n_pts, n_sup, products)
+    ex_flops = opcount.frame_series_flops(mp, f.n_pts, n_sup, products)
     executed = {"flops_per_launch": ex_flops, "achieved": ex_flops / ana_mean_s / 1e12,
                 "frac": ex_flops / ana_mean_s / 1e12 / fp32_peak,
                 "count": f"per node: Gram 2 mp^2 over the 2 x {n_sup} slopes of the window "

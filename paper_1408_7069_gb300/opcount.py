@@ -57,12 +57,25 @@ def chebyshev_products(ratio: float, tol: float = 1e-8) -> int:
     return max(1, math.ceil(math.log(tol * (1.0 + q) / 2.0) / math.log(q)) - 1)
 
 
-def frame_executed_flops(mp: int, n_nodes: int, support_cells: int, mean_products: float) -> float:
-    """Flops the FP32 analysis kernel executes per frame (an FMA counts as two),
-    from its loop structure, beside the paper's count. Per node: the Gram over
+def frame_executed_flops(mp: int, n_nodes: int, support_cells: int, mean_sweeps: float) -> float:
+    """Flops the FP32 analysis kernel executes per frame (an FMA counts as two) where its
+    nodes take the eigensolve (handles with an explicit sweep limit), from its loop
+    structure, beside the paper's count. Per node: the Gram over
     the window cells inside the taper's support (two slopes each, 2 mp^2 flops
-    per slope, both triangles of the mp x mp matrix, pupil or not); per product of
-    the Chebyshev series with the two anomaly rows 4 mp^2.
+    per slope, both triangles of the mp x mp matrix, pupil or not); per Jacobi
+    sweep mp rounds of mp/2 column pairs, each a dot product (2 mp) and a
+    rotation of both columns, 4 mp in the even rounds (one FMA per element)
+    and 6 mp in the odd ones (a multiply and an FMA), 3.5 mp^3 in all; the
+    eigenvector normalisation, transform and apply (about 10 mp^2).
+    mean_sweeps: the measured mean sweep count per node."""
+    per_sweep = 3.5 * mp ** 3
+    per_node = 2.0 * mp * mp * 2 * support_cells + mean_sweeps * per_sweep + 10.0 * mp * mp
+    return float(n_nodes * per_node)
+
+
+def frame_series_flops(mp: int, n_nodes: int, support_cells: int, mean_products: float) -> float:
+    """The same where the nodes take the Chebyshev series, as a running loop's do. Per node:
+    the Gram as above; per product of the series with the two anomaly rows 4 mp^2.
     mean_products: the mean number of products per node (chebyshev_products)."""
     per_node = 2.0 * mp * mp * 2 * support_cells + mean_products * 4.0 * mp * mp
     return float(n_nodes * per_node)
