@@ -64,6 +64,8 @@ struct LkAdjWork {
   double *dtap = nullptr;           // [w*w] d(tau/sigma2)/dL
   int2 *queue = nullptr;            // [n_pts] nodes redone in FP64
   int *queue_len = nullptr;
+  unsigned char *left = nullptr;    // [ckpt][n_pts] FP64 handles: the nodes of one segment that the
+                                    // series left to the eigensolve
   cudaGraphExec_t graph = nullptr;
   const void *graph_y = nullptr, *graph_truth = nullptr;
 };
@@ -132,7 +134,8 @@ __global__ void __launch_bounds__(ADJ_WARPS * 32)
   if (list) {
     if (pid >= *list_len) return;
     pid = list[pid].y;
-  } else if (pid >= I.n_pts) {
+  } else if (pid >= I.n_pts || (a.left && !a.left[pid])) {
+    lk_pdl_wait();                                   // (the series' node)
     return;
   }
   const int w = I.w, wc = w * w, m = I.m;
@@ -476,6 +479,7 @@ __global__ void __launch_bounds__(ADJ_WARPS * 32)
     atomicAdd(&pc[5], 1ull);
   }
 #endif
+  lk_pdl_wait();                                     // (see launch_nodes; else nothing to wait for)
 }
 
 // Warp per valid subaperture (s, t): sums the slope adjoints the nodes whose
@@ -670,15 +674,18 @@ cudaError_t launch_nodes(letkf_ctx *h, LkAdjWork *W, const void *bk, const LkAdj
   const LkInst &I = h->inst[0];
   const int blocks = (I.n_pts + ADJ_WARPS - 1) / ADJ_WARPS;
   if (lk_series64(h)) {
-    // the series, then the nodes it queued from the eigenbases the forward
-    // list kernel stored for the same nodes
-    cudaError_t e = lk_launch_adj_series64(h, a);
+    // the series' nodes, and beside them, from the eigenbases the forward list kernel stored,
+    // those that it left: in a frame of both kinds each takes about as long as the other on a
+    // small system (8 x 8, four frames from the prior draw: one after the other 1455 us, the
+    // eigensolve form for every node 1180, side by side 1294). The second kernel launches once
+    // the first one's CTAs are all running, reads nothing of it, and waits for it at its end.
+    const cudaError_t e = lk_launch_adj_series64(h, a);
     if (e != cudaSuccess) return e;
-    adjoint_node_kernel<MP, double, double>
-        <<<blocks, ADJ_WARPS * 32, node_smem<MP, double, double>(I), h->stream>>>(
-            h->d_inst, W->queue, W->queue_len, nullptr, static_cast<const double *>(bk), 0.f,
-            nullptr, nullptr, h->tol64, a);
-    return cudaGetLastError();
+    return lk_launch_pdl(adjoint_node_kernel<MP, double, double>, blocks, ADJ_WARPS * 32,
+                         node_smem<MP, double, double>(I), h->stream, h->d_inst,
+                         (const int2 *)nullptr, (const int *)nullptr, (const float *)nullptr,
+                         static_cast<const double *>(bk), 0.f, (int2 *)nullptr, (int *)nullptr,
+                         h->tol64, a);
   }
   if (h->precision == 1) {
     // FP64 handles without the series: the FP64 eigenbasis the forward node64
@@ -709,7 +716,7 @@ void free_work(LkAdjWork *W) {
   void *bufs[] = {W->x_seg,    W->basis_seg, W->ckpt_x,   W->ckpt_frame, W->fin_x,
                   W->fin_frame, W->resvar,   W->lam[0],     W->lam[1],     W->xp_bar,
                   W->xbar_bar,  W->ybw,       W->dbw,      W->ybar,       W->dbar,       W->theta,
-                  W->acc,       W->dtap,      W->queue,    W->queue_len};
+                  W->acc,       W->dtap,      W->queue,    W->queue_len,  W->left};
   for (void *p : bufs)
     if (p) cudaFree(p);
   delete W;
@@ -755,6 +762,7 @@ letkf_status ensure_work(letkf_ctx *h, int frames, int ckpt) {
   if (e == cudaSuccess) e = walloc(&W->dtap, wc * sizeof(double));
   if (e == cudaSuccess) e = walloc(&W->queue, (size_t)I.n_pts * sizeof(int2));
   if (e == cudaSuccess) e = walloc(&W->queue_len, sizeof(int));
+  if (e == cudaSuccess && h->precision == 1) e = walloc(&W->left, (size_t)ckpt * I.n_pts);
   // window cells outside the taper's support stay zero (the support changes only
   // with the parameters, which drop this workspace), and so do the slope
   // adjoints of subapertures outside the pupil
@@ -790,10 +798,10 @@ cudaError_t load_state(letkf_ctx *h, const void *x, const long long *frame) {
 }
 
 // One forward frame (prediction in h->X): optional residual, analysis (its
-// background kept in xk, its eigenbases in bk: FP64 on FP64 handles),
-// forecast with the bank noise.
+// background kept in xk, its eigenbases in bk: FP64 on FP64 handles; the nodes beyond the
+// series in left), forecast with the bank noise.
 cudaError_t forward_frame(letkf_ctx *h, const void *y_seq, const void *truth_seq, double *resvar,
-                          void *xk, void *bk, bool forecast) {
+                          void *xk, void *bk, unsigned char *left, bool forecast) {
   const LkInst &I = h->inst[0];
   const long long *ridx = h->frame + 1;
   cudaError_t e = cudaSuccess;
@@ -801,7 +809,9 @@ cudaError_t forward_frame(letkf_ctx *h, const void *y_seq, const void *truth_seq
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(xk, h->X, h->state_total * h->rsz, cudaMemcpyDeviceToDevice, h->stream);
   if (e == cudaSuccess) e = lk_launch_obs(h, y_seq, ridx);
+  h->left64 = left;
   if (e == cudaSuccess) e = lk_launch_analysis(h, nullptr, nullptr);
+  h->left64 = nullptr;
   const size_t nb = (size_t)I.n_pts * I.mp * I.mp;
   if (e == cudaSuccess)
     e = h->basis64 ? cudaMemcpyAsync(bk, h->basis64, nb * sizeof(double), cudaMemcpyDeviceToDevice,
@@ -812,11 +822,11 @@ cudaError_t forward_frame(letkf_ctx *h, const void *y_seq, const void *truth_seq
   return e;
 }
 
-// One backward frame: background xk, analysis eigenbases bk, adjoint of the
-// analysis lam_in -> adjoint of the previous analysis lam_out.
+// One backward frame: background xk, analysis eigenbases bk, nodes beyond the series left,
+// adjoint of the analysis lam_in -> adjoint of the previous analysis lam_out.
 cudaError_t backward_frame(letkf_ctx *h, LkAdjWork *W, const void *y_k, const void *truth_k,
-                           const void *xk, const void *bk, const double *lam_in, double *lam_out,
-                           double crit_scale) {
+                           const void *xk, const void *bk, const unsigned char *left,
+                           const double *lam_in, double *lam_out, double crit_scale) {
   const LkInst &I = h->inst[0];
   cudaError_t e = cudaMemcpyAsync(h->X, xk, h->state_total * h->rsz, cudaMemcpyDeviceToDevice,
                                   h->stream);
@@ -835,8 +845,7 @@ cudaError_t backward_frame(letkf_ctx *h, LkAdjWork *W, const void *y_k, const vo
   a.sigma2 = h->cfg.sigma2;
   a.max_sweeps = h->max_sweeps;
   a.counters = h->counters;
-  a.queue = W->queue;
-  a.queue_len = W->queue_len;
+  a.left = lk_series64(h) ? left : nullptr;
   e = I.mp == 16 ? launch_nodes<16>(h, W, bk, a) : launch_nodes<32>(h, W, bk, a);
   if (e != cudaSuccess) return e;
   theta_reduce_kernel<<<1, 256, 0, h->stream>>>(W->theta, I.n_pts, W->acc);
@@ -870,6 +879,7 @@ letkf_status enqueue_grad(letkf_ctx *h, int frames, const void *y_seq, const voi
   const char *ys = static_cast<const char *>(y_seq);
   const char *ts = static_cast<const char *>(truth_seq);
   char *xs = static_cast<char *>(W->x_seg);
+  auto left = [W, &I](int slot) { return W->left ? W->left + (size_t)slot * I.n_pts : nullptr; };
   const double crit_scale = -2.0 / ((double)I.n_pts * I.m * frames);
   LK_ACUDA(h, cudaMemsetAsync(h->frame + 1, 0, sizeof(long long), h->stream));
   // ---- forward ----
@@ -879,7 +889,7 @@ letkf_status enqueue_grad(letkf_ctx *h, int frames, const void *y_seq, const voi
       LK_ACUDA(h, save_state(h, static_cast<char *>(W->ckpt_x) + (size_t)seg * st,
                              W->ckpt_frame + 2 * seg));
     LK_ACUDA(h, forward_frame(h, y_seq, truth_seq, W->resvar, xs + (size_t)slot * st,
-                              bs + (size_t)slot * bseg, true));
+                              bs + (size_t)slot * bseg, left(slot), true));
   }
   LK_ACUDA(h, save_state(h, W->fin_x, W->fin_frame));
   // ---- backward ----
@@ -894,12 +904,12 @@ letkf_status enqueue_grad(letkf_ctx *h, int frames, const void *y_seq, const voi
                              W->ckpt_frame + 2 * seg));
       for (int k = s; k < e; ++k)
         LK_ACUDA(h, forward_frame(h, y_seq, nullptr, nullptr, xs + (size_t)(k - s) * st,
-                                  bs + (size_t)(k - s) * bseg, k + 1 < e));
+                                  bs + (size_t)(k - s) * bseg, left(k - s), k + 1 < e));
     }
     for (int k = e - 1; k >= s; --k) {
       LK_ACUDA(h, backward_frame(h, W, ys + (size_t)k * h->p_total * h->rsz,
                                  ts + (size_t)k * h->n_pts_total * h->rsz,
-                                 xs + (size_t)(k - s) * st, bs + (size_t)(k - s) * bseg,
+                                 xs + (size_t)(k - s) * st, bs + (size_t)(k - s) * bseg, left(k - s),
                                  W->lam[cur], W->lam[cur ^ 1], crit_scale));
       cur ^= 1;
     }

@@ -135,6 +135,7 @@ struct letkf_ctx {
   float4 *cheb64 = nullptr;         // the FP64 one (FP64 handles), in pairs of floats
   double2 *poles = nullptr;         // [16] poles and weights of A^-1/2 (FP32 handles)
   int keep_basis = 0;               // store every node's eigenbasis (reverse mode needs it)
+  unsigned char *left64 = nullptr;  // [n_pts] where the FP64 series marks the nodes it leaves
 
   int n_inst = 0;
   std::vector<LkInst> inst;         // host copies of the descriptors
@@ -261,12 +262,14 @@ struct LkAdjArgs {
   double rho, sigma2;
   int max_sweeps;
   int *counters;
-  int2 *queue;           // nodes left to the eigensolve form
-  int *queue_len;
+  // [n_pts] nonzero: the node the forward series left to the eigensolve, which the eigensolve
+  // form takes here too; NULL: no series, every node by the eigensolve form
+  const unsigned char *left;
 };
 // FP64 node problems by Chebyshev series (letkf_series64.cu): every node of
 // width class cls of an FP64 handle, those above LK_CHEB_MAX64 queued in the
-// class's worklist; and the adjoint of every node, likewise queued in a.queue.
+// class's worklist and marked in h->left64 (if any); and the adjoint of the nodes
+// not marked in a.left.
 bool lk_series64(const letkf_ctx *h);     // whether the handle takes this form
 cudaError_t lk_launch_series64(letkf_ctx *h, int cls, void *mean, void *spread,
                                const LkCycle &cy = {});

@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(S64<MPD>::NT, (MPD <= 24 ? 768 : 512) / S64<MP
                     double *__restrict__ mean, double *__restrict__ spread,
                     const float4 *__restrict__ cheb, int *__restrict__ counters,
                     int *__restrict__ queue, int2 *__restrict__ worklist,
-                    const double *__restrict__ noise) {
+                    const double *__restrict__ noise, unsigned char *__restrict__ left) {
   using C = S64<MPD>;
   extern __shared__ __align__(16) double sm64[];
   lk_pdl_wait();
@@ -425,7 +425,9 @@ __global__ void __launch_bounds__(S64<MPD>::NT, (MPD <= 24 ? 768 : 512) / S64<MP
   const float f2 = seg_load<MPD>(g, sm, row, seg);
   // both vectors' threads hold G: half the sum of squares is |G|_F^2
   const float ratio = sqrtf(0.5f * cta_sum<C::NW>(f2, sm.red));
-  if (!(ratio <= LK_CHEB_MAX64)) {                   // (a NaN too)
+  const bool ill = !(ratio <= LK_CHEB_MAX64);        // (a NaN too)
+  if (left && t == 0) left[pid] = ill;               // (letkf_grad: one instance)
+  if (ill) {
     if (t == 0) worklist[atomicAdd(queue, 1)] = make_int2(it.x, pid);
     return;
   }
@@ -568,6 +570,8 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
   const int t = threadIdx.x, seg = t % C::KS, vec = (t / C::KS) & 1, row = t / (2 * C::KS);
   const int lane = t & 31, wv = t >> 5;
   int *ri = sm.redi();
+  lk_pdl_trigger();                                  // adjoint_node_kernel runs beside this one
+  if (a.left[pid]) return;                           // the eigensolve form's
   if (wv == 0) support<MPD>(I, ij, sm);
 #pragma unroll
   for (int r = 0; r < 2; ++r)
@@ -593,10 +597,6 @@ __global__ void __launch_bounds__(S64<MPD>::NT)
   Seg64<MPD> g;
   const float f2 = seg_load<MPD>(g, sm, row, seg);
   const float ratio = sqrtf(0.5f * cta_sum<C::NW>(f2, sm.red));
-  if (!(ratio <= LK_CHEB_MAX64)) {
-    if (t == 0) a.queue[atomicAdd(a.queue_len, 1)] = make_int2(0, pid);
-    return;
-  }
   if (t < 2) a.xbar_bar[(size_t)pid * 2 + t] = sm.red64()[10 + t];
   // s_0 x'_0 + s_1 x'_1 times 2^-eb
   const int ex0 = ri[2], ex1 = ri[3], eg0 = ri[4], eg1 = ri[5];
@@ -919,7 +919,7 @@ cudaError_t launch_series64(letkf_ctx *h, int cls, void *mean, void *spread, con
   return lk_launch_pdl(series64_kernel<MPD>, (unsigned)h->n_pts_total, S64<MPD>::NT, need,
                        h->stream, h->d_inst, h->node_items, (double *)mean, (double *)spread,
                        (const float4 *)h->cheb64, h->counters, h->counters + 4 + cls,
-                       h->worklist + (size_t)cls * h->n_pts_total, (const double *)noise);
+                       h->worklist + (size_t)cls * h->n_pts_total, (const double *)noise, h->left64);
 }
 
 template <int MPD>
