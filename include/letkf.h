@@ -76,8 +76,11 @@ typedef struct {
   double sigma2;               /* slope noise variance (rad^2), > 0 */
   double a_ar1;                /* AR(1) coefficient of the forecast */
   double noise_std;            /* forecast noise = noise_std * bank screen value */
-  int32_t precision;           /* 0 = FP32 storage and analysis with FP64 fallback, 1 = FP64 */
-  double fp64_kappa;           /* FP64 fallback threshold on kappa_hat (e.g. 300); <= 0 disables it */
+  int32_t precision;           /* 0 = FP32 storage and analysis, nodes above fp64_kappa to more digits
+                                  (letkf_analyze); 1 = FP64 storage, the arithmetic to 48 bits or
+                                  more (letkf_set_fp64_start) */
+  double fp64_kappa;           /* threshold on kappa_hat (e.g. 300) above which FP32 handles analyse a
+                                  node to more than FP32; <= 0 disables it */
   uint64_t seed;               /* SplitMix64 seed of the forecast-noise draws */
   const float *noise_bank;     /* host [bank_B][bank_G][bank_G] screens, or NULL; copied */
   int32_t bank_B, bank_G;      /* bank shape (ignored when noise_bank is NULL) */
@@ -167,9 +170,13 @@ letkf_status letkf_forecast(letkf_t h, const void *noise_dev);
  * NULL; spread is the sample standard deviation over members (m - 1). The
  * ensemble is replaced by the analysis.
  * FP32 handles: a node whose kappa_hat = 1 + rho tr(C Yb_l) / (m - 1), an upper
- * bound on the condition number of A, exceeds fp64_kappa is analysed in FP64
- * (Gram and accumulated Jacobi sweep, started from the node's FP32 eigenbasis)
- * and written back in FP32. */
+ * bound on the condition number of A, exceeds fp64_kappa is analysed to more
+ * than FP32 and written back in FP32. With m <= 32, kappa_hat <= 1e5 and
+ * (m - 1) / rho in (0.01, 1e6): in pairs of floats (Gram to 2^-42 of its norm, Householder
+ * tridiagonal form, A^-1/2 by a 15-pole rational approximation of error 4e-9,
+ * no eigensolve). Otherwise, with max_sweeps > 0 and in classes of row split 2:
+ * in FP64 (Gram and accumulated Jacobi sweep, started from the node's FP32
+ * eigenbasis). The errors of both are those of the FP32 slopes. */
 letkf_status letkf_analyze(letkf_t h, const void *y_dev, void *mean_dev, void *spread_dev);
 
 /* Loop criterion (Section 2.1 Eq. Crit_Opt; Section 5): spatial variance over
@@ -285,18 +292,19 @@ letkf_status letkf_step(letkf_t h, const void *y_host, const void *truth_host, v
  * residual variance of the prediction (Section 2.1 Eq. Crit_Opt, as in
  * letkf_residual), each frame run as in letkf_run (residual of the current
  * prediction, analysis of y_seq[k] by Section 4.2, forecast of Section 3.1.2
- * with bank noise) from the handle's current ensemble, eigenbases and frame
- * counter; and grad = (dJ/drho, dJ/dsigma2, dJ/dL), L the Gaspari-Cohn
+ * with bank noise) from the handle's current ensemble and frame counter; and
+ * grad = (dJ/drho, dJ/dsigma2, dJ/dL), L the Gaspari-Cohn
  * half-support of the taper (cfg.loc_len, or window / 4 when that is <= 0; the
  * L component is 0 without the taper). The analysis is differentiated through
  * its eigendecomposition with divided differences of lambda^-1/2 written in a
  * form exact for equal eigenvalues, so windows with fewer slopes than m - 1
  * (exactly degenerate eigenvalues) need no special case. The backward pass
  * recomputes each node's eigenbasis from the one its forward analysis stored
- * (FP32), and in FP64 for the nodes that the FP64 fallback takes; FP64 handles
- * differentiate the Chebyshev series of the nodes it solves instead.
+ * (FP32), and in FP64 for the nodes above fp64_kappa; FP64 handles
+ * differentiate the Chebyshev series of the nodes it solves instead, in the
+ * same arithmetic (letkf_set_fp64_start).
  * y_seq_dev: device [frames][p] real; truth_seq_dev: device [frames][n_pts] real.
- * ckpt_every: frames per segment; the forward keeps the ensemble and bases at
+ * ckpt_every: frames per segment; the forward keeps the ensemble and frame counters at
  *   the start of every segment and the backward recomputes one segment at a
  *   time (device memory ~ (frames / ckpt_every + ckpt_every) states); <= 0 or
  *   >= frames keeps every frame (no recomputation).
@@ -341,8 +349,13 @@ letkf_status letkf_autotune(letkf_t h, const void *y_dev, int32_t reps, int32_t 
  * one half of two columns, so a node takes twice the lanes (2 nodes per warp
  * for m <= 16, 1 for m <= 32), every dot product of the one-sided Jacobi adds
  * its partner lane's half, and a rotation round's dependent chain is about
- * half as long. It pays on systems whose nodes fill few warps per SM (a few
- * thousand nodes or fewer on 152 SMs) and costs issue slots on large ones.
+ * half as long. The split form knows the eigensolve only: a class of split = 2
+ * takes neither the Chebyshev series nor the forecast inside the analysis. Measured
+ * on one GB300, closed loops, us per frame of split 1 and 2: by the series (the
+ * default) 16.6 and 26.4 (8 x 8, m = 10), 18.9 and 55.8 (32 x 32, m = 24), 46.7 and
+ * 193 (80 x 80, m = 32); on handles with max_sweeps > 0, which sweep every node,
+ * 25.3 and 24.8, 41.1 and 56.0, 173.6 and 193.6. So it pays nowhere by default, and
+ * by 2 % on the smallest systems with an explicit sweep limit.
  * The results differ from split 1 by rounding only (sums in another order);
  * for fixed settings they are bitwise reproducible. Width classes 0 and 1 of
  * FP32 per-node handles only, with the class's current tile shape holding
@@ -352,13 +365,19 @@ letkf_status letkf_autotune(letkf_t h, const void *y_dev, int32_t reps, int32_t 
 letkf_status letkf_set_row_split(letkf_t h, int32_t width_class, int32_t split);
 
 /* Start of the FP64 eigensolve on FP64 handles (Section 4.2's EVD): warm = 1
- * (the default) solves well-conditioned nodes by a Chebyshev series (see
- * letkf_config.max_sweeps) and for the others runs the FP32 two-columns-per-lane eigensolve on the window
+ * (the default) solves nodes with |G|_F / alpha <= 42 (alpha = (m - 1) / rho, G =
+ * A - alpha I) by a Chebyshev series (see letkf_config.max_sweeps) in pairs of floats:
+ * 48 bits of every value, whatever its size; the later terms, whose coefficients
+ * add up to less than 2^-27, in floats. The members' error is within 8 kappa_hat
+ * 2^-47 of the size of anomalies and increments, 4 units of 2^-53 of the members added (tested;
+ * measured over loops 2e-14 of the anomalies, where the eigensolve has 3.6e-14). For
+ * the other nodes it runs the FP32 two-columns-per-lane eigensolve on the window
  * rounded to FP32 first and starts each node's FP64 one-sided Jacobi from that
  * basis, made orthonormal to FP64 rounding by two Newton-Schulz steps, stopping after a
  * sweep whose cosines all stay below 1e-8 (the next would rotate by about its
- * square); warm = 0 takes every node by sweeps from the identity and stops after
- * a sweep without rotations. Both give FP64 results (they differ by rounding). FP64 per-node
+ * square), all in FP64. warm = 0 takes every node by sweeps from the identity and stops after
+ * a sweep without rotations. For FP64 arithmetic at every node with the warm start, set
+ * letkf_config.max_sweeps > 0 (e.g. 20), which switches the series off. FP64 per-node
  * handles only (LETKF_ERR_ARG otherwise). The FP32 pass takes the class's
  * tile shape, so FP64 handles take the shapes of the whole-column FP32 form.
  * Synchronises; drops the cached CUDA graphs. */
@@ -368,11 +387,11 @@ letkf_status letkf_set_fp64_start(letkf_t h, int32_t warm);
  * device since the last call (LETKF_OK if none). */
 letkf_status letkf_sync(letkf_t h);
 
-/* Counters of the last analysis, host pointers (any may be NULL): nodes that
- * took the FP64 fallback, the largest and the total number of Jacobi sweeps
- * over the nodes (a node of the FP64 fallback counts the sweeps of its FP32
- * and of its FP64 eigensolve, a node solved by the Chebyshev series one).
- * Synchronises. */
+/* Counters of the last analysis, host pointers (any may be NULL): nodes of FP32
+ * handles above fp64_kappa, the largest and the total number of Jacobi sweeps
+ * over the nodes (a node above fp64_kappa that sweeps counts those of its FP32
+ * and of its FP64 eigensolve; a node solved by the Chebyshev series or in pairs
+ * of floats counts one). Synchronises. */
 letkf_status letkf_stats(letkf_t h, int32_t *fp64_points, int32_t *max_sweeps,
                          int32_t *total_sweeps);
 
@@ -431,8 +450,8 @@ letkf_status letkf_fma_peaks(double *out);
 /* Where the FP32 analysis kernel spends its time, in a library built with
  * phase clocks (build option LK_PHASE_CLOCKS; LETKF_ERR_STATE otherwise):
  * SM cycles summed over its warps since the last call, out: host uint64_t[5]
- * = halo staging, Gram and kappa_hat, Jacobi sweeps, eigenpairs + transform +
- * apply (Section 4.2's steps), and the number of warps. Synchronises the
+ * = halo staging, Gram and kappa_hat, Chebyshev series or Jacobi sweeps with
+ * their transform, apply (Section 4.2's steps), and the number of warps. Synchronises the
  * device and resets the counts. The paper has no counterpart. */
 letkf_status letkf_phase_clocks(uint64_t *out);
 

@@ -347,10 +347,11 @@ __device__ __forceinline__ T lk_warp_sum(T v) {
 // with lk_launch_pdl, so that it can be scheduled while its predecessor on the
 // stream drains; its first statement is lk_pdl_wait(), which returns once the
 // predecessor grid has completed and its writes are visible (a no-op for a
-// kernel launched without the attribute). The residual and forecast kernels
-// then call lk_pdl_trigger(), letting the next kernel launch at once. The
-// observation and analysis kernels do not: an analysis launched early has its
-// CTAs placed on SMs that are still busy, several to an SM, which doubles the
+// kernel launched without the attribute). The residual, forecast and piston sum
+// kernels, the FP64 series and node kernels and the list kernels (but for the one with
+// the tridiagonal form) then call lk_pdl_trigger(), letting the next kernel launch at
+// once. The observation and FP32 analysis kernels do not: an analysis launched early
+// has its CTAs placed on SMs that are still busy, several to an SM, which doubles the
 // time of a latency-bound analysis that does not fill the GPU (measured on the
 // 16 m system); their dependents launch as their CTAs exit.
 __device__ __forceinline__ void lk_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

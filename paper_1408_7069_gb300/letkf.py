@@ -264,7 +264,7 @@ def letkf_sync(h) -> None:
 
 
 def letkf_stats(h):
-    """(FP64 fallback nodes, max sweeps, total sweeps) of the last analysis."""
+    """(nodes above fp64_kappa, max sweeps, total sweeps) of the last analysis."""
     a, b, c = c_int32(), c_int32(), c_int32()
     _check(lib().letkf_stats(h, byref(a), byref(b), byref(c)), h)
     return a.value, b.value, c.value
