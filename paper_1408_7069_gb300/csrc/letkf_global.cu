@@ -11,8 +11,8 @@
 //   mean     wbar = A^-1 c by iterative refinement: residual c - A wbar in
 //            FP64, correction Z (Z r) / s_A in FP32
 //   apply    P = X' sqrt((m-1) / s_A) Z over all state rows, Xa = xbar + X' wbar + P,
-//            X' wbar in FP64 (m products per row: 4 us of 909 at m = 626), mean and
-//            spread. P's mean over the members is zero but for Z's rounding, which grows
+//            X' wbar in pairs of floats (FP64 took 1 us more at m = 101, 5 us at m = 626),
+//            mean and spread. P's mean over the members is zero but for Z's rounding, which grows
 //            with kappa, and the rounding of the slopes' means, part of whose error in
 //            X' wbar it takes back: it is kept up to NR_KEEP and taken out beyond
 //
@@ -34,7 +34,7 @@
 // after 20 steps where the full one converges.)
 #include <math.h>
 
-#include "letkf_device.cuh"
+#include "letkf_df.cuh"
 
 namespace {
 
@@ -474,6 +474,12 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
         !(__uint_as_float(__ldcg(a.sync + NR_LAST)) <=
           NR_CORRECTION * __uint_as_float(__ldcg(a.sync + NR_LAST + 1))))
       atomicOr(a.counters, LK_BIT_NOCONVERGE);
+    // wbar as a pair of floats, in the refinement's vectors
+    for (int i = gw * 32 + lane; i < n; i += nw * 32) {
+      const Df w = df_of(__ldcg(a.w64 + i));
+      a.rv[i] = w.h;
+      a.vv[i] = w.l;
+    }
     // ---- T = sqrt((m-1) / s_A) Z on the m x m block, zero elsewhere; the iteration
     // failed if Z Y strays from I by more than 1e-3 ----
     const float f = (float)sqrt((m - 1) * inv);
@@ -505,13 +511,15 @@ __global__ void __launch_bounds__(NR_THREADS, 1) ns_root_kernel(NsArgs a) {
   }
 }
 
+constexpr int NF_VALS = 4;             // values per lane in flight
 // Xa = xbar + X' wbar + P, P = X' T; mean and spread, warp per state row. Where P's mean is
 // taken out (*keep zero), what xbar's rounding has left in the anomalies, which P passes on, is
 // added back. The common part is a pair of floats, so that a member is rounded once.
 __global__ void __launch_bounds__(LK_WARP_CTA)
     ns_finish_kernel(const LkInst *__restrict__ insts, int mpt, const float *__restrict__ P,
                      const float *__restrict__ Xp, const float *__restrict__ xm,
-                     const double *__restrict__ wbar, const unsigned *__restrict__ keep,
+                     const float *__restrict__ wh, const float *__restrict__ wl,
+                     const unsigned *__restrict__ keep,
                      float *__restrict__ mean, float *__restrict__ spread,
                      int *__restrict__ counters) {
   lk_pdl_wait();
@@ -520,21 +528,38 @@ __global__ void __launch_bounds__(LK_WARP_CTA)
   const int lane = threadIdx.x & 31, m = I.m;
   if (r >= 2LL * I.n_pts) return;
   float *x = static_cast<float *>(I.X) + r * m;
+  const bool kept = *keep != 0;
   float pm = 0.f, xr = 0.f;
-  double xw = 0.0;
-  for (int j = lane; j < m; j += 32) {
-    const float xp = Xp[r * mpt + j];
-    pm += P[r * mpt + j];
-    xr += xp;
-    xw = fma((double)xp, wbar[j], xw);
+  Df xw = df(0.f);
+  for (int j0 = lane; j0 < m; j0 += 32 * NF_VALS) {  // (loads in flight together)
+    float p[NF_VALS], xp[NF_VALS];
+    Df w[NF_VALS];
+#pragma unroll
+    for (int u = 0; u < NF_VALS; ++u) {
+      const int j = j0 + 32 * u;
+      p[u] = j < m ? P[r * mpt + j] : 0.f;
+      xp[u] = j < m ? Xp[r * mpt + j] : 0.f;
+      w[u] = j < m ? Df{wh[j], wl[j]} : df(0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < NF_VALS; ++u) {
+      pm += p[u];
+      xr += xp[u];
+      xw = df_add(xw, df_mul(df(xp[u]), w[u]));
+    }
   }
-  pm = *keep ? 0.f : lk_warp_sum(pm) / float(m);
-  xr = *keep ? 0.f : lk_warp_sum(xr) / float(m);
-  const double base = (double)xm[r] + ((double)xr + lk_warp_sum(xw));
-  const float bh = (float)base, bl = (float)(base - (double)bh);
+  xw = df_warp_sum(xw);
+  if (kept) {
+    pm = 0.f;
+  } else {
+    pm = lk_warp_sum(pm) / float(m);
+    xw = df_add(xw, df(lk_warp_sum(xr) / float(m)));
+  }
+  const Df base = df_add(df(xm[r]), xw);
   float sum = 0.f;
+#pragma unroll 4
   for (int j = lane; j < m; j += 32) {
-    const float xa = bh + (bl + (P[r * mpt + j] - pm));
+    const float xa = base.h + (base.l + (P[r * mpt + j] - pm));
     x[j] = xa;
     sum += xa;
   }
@@ -620,7 +645,8 @@ cudaError_t lk_launch_ns_global(letkf_ctx *h, const double *gpart, const double 
   if (e == cudaSuccess)
     e = lk_launch_pdl(ns_finish_kernel, fb, LK_WARP_CTA, 0, h->stream,
                       (const LkInst *)h->d_inst, mpt, (const float *)Pr, (const float *)a.Xp,
-                      (const float *)a.xm, (const double *)a.w64, (const unsigned *)(a.sync + 3),
+                      (const float *)a.xm, (const float *)a.rv, (const float *)a.vv,
+                      (const unsigned *)(a.sync + 3),
                       static_cast<float *>(mean), static_cast<float *>(spread), h->counters);
   return e;
 }
