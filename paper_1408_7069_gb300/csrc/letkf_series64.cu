@@ -28,8 +28,9 @@
 // in pairs 424, with the second half in floats 400; gradient of ten frames at 16 m,
 // m = 24: 32.7, 7.2, 3.1, 2.45 ms (861 nodes: forward 116, 40, 33 us, adjoint 449, 161, 104,
 // 45% of the issue slots used: bound by the products' chains at 12 to 15 warps per SM).
-// Errors against FP64 of four seeds: the eigensolve's X 1e-15 to 5e-15 and gradient 8e-15 to
-// 1.4e-12, now 9e-16 to 4e-15 and 1e-14 to 4e-14.
+// Errors against FP64 of these two cases, eight seeds: the eigensolve's X 1e-15 to 5e-15 and
+// gradient 8e-15 to 1.4e-12, now 9e-16 to 1e-14 and 2e-15 to 8e-14; over 16 drawn ones the
+// geometric means are X 1.3e-15 and 5e-16, gradients 1.6e-14 and 1.1e-14.
 #include <math.h>
 
 #include "letkf_df.cuh"
