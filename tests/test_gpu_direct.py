@@ -443,3 +443,34 @@ def test_calls_are_ordered_against_the_current_stream():
     torch.cuda.synchronize()
     assert len(out) == 4 and all(torch.equal(v, X * k) for k, v in out)
     f.close()
+
+
+# ---------------------------------------------------------------------------
+# Two members (the closed form beside direct_apply). Tolerance: the members' storage and
+# the means that the innovations take (two units of 2^-24 of the members), and the roundings
+# of slopes, Gram, trace, root and products, eight units of the anomalies and increments:
+# no factor of the condition, since the trace's relative error is that of A.
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("ratio", [3.0, 20.0, 80.0, 290.0])
+@pytest.mark.parametrize("window,taper", [(3, 0), (5, 1)])
+def test_two_members_to_the_rounding_of_fp32(window, taper, ratio):
+    mask = synth.pupil_subap_mask(8, 0.0)
+    geom = oracle.build_geometry(mask, window, taper, 0.0)
+
+    def rms(v):
+        return float(np.sqrt(np.mean(np.square(v))))
+    for seed in range(6):
+        rng = np.random.default_rng(seed)
+        P = anoms(rng.standard_normal((geom.n_pts, 2, 2)))
+        _, _, Yb, _ = oracle.observe(geom, P)
+        g = [RHO * np.linalg.norm((Yb[i] * (t / SIGMA2)[:, None]).T @ Yb[i])
+             for i, t in zip(geom.win_idx, geom.win_tau)]
+        X = 3 * rng.standard_normal((geom.n_pts, 2, 1)) + (ratio / np.max(g)) ** 0.5 * P
+        X = X.astype(np.float32)
+        y = rng.standard_normal(geom.p).astype(np.float32)
+        ref = oracle.analysis(geom, X.astype(np.float64), y.astype(np.float64), SIGMA2, RHO)
+        Xa, mean, spread, st = analyse(mask, X, y, 2, window, taper, fp64_kappa=-1.0)
+        assert st[1:] == (1, geom.n_pts)
+        step = ref[1] - X.astype(np.float64).mean(-1)
+        tol = 2.0 ** -24 * (2 * rms(X) + 8 * (rms(anoms(X)) + rms(step)))
+        assert rms(Xa - ref[0]) <= tol and rms(mean - ref[1]) <= tol and rms(spread - ref[2]) <= tol
